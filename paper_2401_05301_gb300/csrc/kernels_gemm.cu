@@ -1,11 +1,21 @@
 // Grouped FP64 GEMM for the TEBD contractions (complex) and the eigenvector
 // orthonormalisation (real).
 //
-// On this GPU the FP64 pipe issues about two DFMA per clock per SM, so a tile
-// of 64 x 64 outputs over a reduction slab of 16 does ~256 complex MACs per
-// element loaded: the kernel is bound by DFMA issue, not by memory.  One
-// launch serves up to GEMM_MAXP independent problems (all triples of a
-// Trotter layer), each optionally strided-batched.
+// Bound: the FP64 pipe, which takes a warp-wide DFMA every 16 to 19 clocks per SM (1.7 to 2
+// lanes per clock, measured) however many of its lanes are active.  A tile needs no depth to
+// keep it busy (a 16 x 16 complex tile loads under 1 byte per clock from L2), so what counts is
+// that no lane computes padding and that every SM has a tile:
+//   * tiles are at most 16 x 16 outputs, one per thread, of balanced height and width
+//     (24 rows make two tiles of 12), and the threads number a tile's outputs
+//     consecutively, so a ragged tile costs only the warps that it fills;
+//   * a problem with few tiles splits its reduction over 2, 4 or 8 CTAs of a cluster, which add
+//     their partial sums through distributed shared memory in a fixed order.  The split
+//     depends on the problem's own shape only, so a result never depends on its batch.
+// One launch serves up to GEMM_MAXP independent problems (all triples of a Trotter layer), each
+// optionally strided-batched.
+// Measured against 64 x 64 tiles with padded outputs: 1000 x 250 x 3990 complex 16.8 -> 7.2 ms (1.11
+// TFLOP/s), a bond correlator of chi = 24, d = 4 (two 24 x 24 x 96 products) 806 -> 31 us, a four-step
+// quench of L = 8 60.6 -> 23.2 ms, of the blocked L = 41, d = 5 chain 153 -> 45.7 ms.
 #include "ptebd_internal.h"
 
 #include <algorithm>
@@ -15,7 +25,28 @@ namespace ptebd {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
+constexpr int TB = 16;        // largest tile height and width
+constexpr int BK = 16;        // reduction slab
+constexpr int NT = TB * TB;   // one output per thread
+constexpr int CLUSTER = 8;    // CTAs per cluster of a launch that holds a split problem
+// A problem whose tiles do not fill the 152 SMs twice is split as long as a slice keeps 8
+// reduction indices: with two tiles or more per SM the slices' exchange is the larger part.
+constexpr long long FILL = 2 * 152;
+
+__host__ __device__ __forceinline__ int tile_count(int n) { return (n + TB - 1) / TB; }
+__host__ __device__ __forceinline__ int tile_size(int n) {  // balanced: the tiles differ by the last one only
+  const int t = tile_count(n);
+  return (n + t - 1) / t;
+}
+__host__ __device__ __forceinline__ long long tiles_of(const GemmProb& p) {
+  const long long tm = tile_count(p.M), tn = tile_count(p.N);
+  return p.batch * (p.herm ? tm * (tm + 1) / 2 : tm * tn);
+}
+int split_of(const GemmProb& p) {
+  int s = 1;
+  while (s < CLUSTER && tiles_of(p) * s < FILL && p.K >= 16 * s) s *= 2;
+  return s;
+}
 
 struct R {  // real arithmetic
   using T = double;
@@ -44,23 +75,51 @@ struct C {  // complex arithmetic, interleaved (re, im)
   static __device__ __forceinline__ T add(T a, T b) { return make_double2(a.x + b.x, a.y + b.y); }
 };
 
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// A shared-memory double of another CTA of the cluster.
+__device__ __forceinline__ double peer_load(const double* mine, unsigned rank) {
+  double v;
+  asm volatile("{\n .reg .u32 a;\n mapa.shared::cluster.u32 a, %1, %2;\n ld.shared::cluster.f64 %0, [a];\n}\n"
+               : "=d"(v)
+               : "r"((unsigned)__cvta_generic_to_shared(mine)), "r"(rank)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ double peer_value(const double* mine, unsigned rank) { return peer_load(mine, rank); }
+__device__ __forceinline__ double2 peer_value(const double2* mine, unsigned rank) {
+  const double* m = reinterpret_cast<const double*>(mine);
+  return make_double2(peer_load(m, rank), peer_load(m + 1, rank));
+}
+
 template <class A_, int OPA, int OPB>
 __global__ void __launch_bounds__(NT) gemm_kernel(const __grid_constant__ GemmBatch gb) {
   using T = typename A_::T;
-  __shared__ T As[BK][BM + 1];
-  __shared__ T Bs[BK][BN + 1];
+  __shared__ T As[BK][TB + 1];
+  __shared__ T Bs[BK][TB + 1];
+  __shared__ T part[NT];
 
-  const int tile = blockIdx.x;
+  // the problem of this CTA: tile_start counts CTAs, a multiple of the cluster size per problem
   int pi = 0;
-  while (pi + 1 < gb.nprob && tile >= gb.tile_start[pi + 1]) ++pi;
+  while (pi + 1 < gb.nprob && (int)blockIdx.x >= gb.tile_start[pi + 1]) ++pi;
   const GemmProb& P = gb.p[pi];
-  const int local = tile - gb.tile_start[pi];
-  const int tn = (P.N + BN - 1) / BN, tm = (P.M + BM - 1) / BM;
+  const int split = P.split, local = blockIdx.x - gb.tile_start[pi];
+  const unsigned rank = split > 1 ? cluster_rank() : 0;
+  const int slice = (int)rank & (split - 1);
+  const long long unit = local / split;  // the CTAs of a tile are neighbours in their cluster
+  const int tn = tile_count(P.N), tm = tile_count(P.M), hm = tile_size(P.M), hn = tile_size(P.N);
   const int per_batch = P.herm ? tm * (tm + 1) / 2 : tm * tn;
-  const int bidx = local / per_batch, r = local % per_batch;
+  const bool live = unit < (long long)per_batch * P.batch;  // the last cluster may hold idle CTAs
+  const int bidx = live ? (int)(unit / per_batch) : 0, r = live ? (int)(unit % per_batch) : 0;
   int bm, bn;
   if (P.herm) {  // r enumerates the lower-triangular tiles row by row
-    bm = (int)((sqrt(8.0 * r + 1.0) - 1.0) * 0.5);
+    bm = (int)((sqrtf(8.0f * (float)r + 1.0f) - 1.0f) * 0.5f);
     while (bm * (bm + 1) / 2 > r) --bm;
     while ((bm + 1) * (bm + 2) / 2 <= r) ++bm;
     bn = r - bm * (bm + 1) / 2;
@@ -68,92 +127,152 @@ __global__ void __launch_bounds__(NT) gemm_kernel(const __grid_constant__ GemmBa
     bm = r / tn;
     bn = r % tn;
   }
+  const int m0 = bm * hm, n0 = bn * hn;
+  const int mt = live ? min(hm, P.M - m0) : 0, nt = live ? min(hn, P.N - n0) : 0;
   const T* __restrict__ A = static_cast<const T*>(P.A) + (long long)bidx * P.sA;
   const T* __restrict__ B = static_cast<const T*>(P.B) + (long long)bidx * P.sB;
   T* __restrict__ Cm = static_cast<T*>(P.C) + (long long)bidx * P.sC;
+  // this CTA's share of the reduction
+  const int ks = (P.K + split - 1) / split;
+  const int kb = min(P.K, slice * ks), ke = live ? min(P.K, kb + ks) : kb;
 
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  T acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = A_::zero();
+  // the element of each operand's slab that this thread loads
+  const int ai = (OPA == OP_C) ? threadIdx.x % TB : threadIdx.x / BK;
+  const int ak = (OPA == OP_C) ? threadIdx.x / TB : threadIdx.x % BK;
+  const int bj = (OPB == OP_C) ? threadIdx.x / BK : threadIdx.x % TB;
+  const int bk = (OPB == OP_C) ? threadIdx.x % BK : threadIdx.x / TB;
+  auto load_a = [&](int k0) {
+    T v = A_::zero();
+    const int gi = m0 + ai, gk = k0 + ak;
+    if (ai < mt && gk < ke) {
+      if (OPA == OP_N) v = A[(long long)gi * P.lda + gk];
+      else if (OPA == OP_C) v = A_::cj(A[(long long)gk * P.lda + gi]);
+      else v = A_::cj(A[(long long)gi * P.lda + gk]);
+      if (P.s_red) v = A_::scale(v, P.s_red[gk / P.red_div]);
+    }
+    return v;
+  };
+  auto load_b = [&](int k0) {
+    T v = A_::zero();
+    const int gj = n0 + bj, gk = k0 + bk;
+    if (bj < nt && gk < ke) {
+      if (OPB == OP_N) v = B[(long long)gk * P.ldb + gj];
+      else if (OPB == OP_C) v = A_::cj(B[(long long)gj * P.ldb + gk]);
+      else v = A_::cj(B[(long long)gk * P.ldb + gj]);
+      if (P.s_red_b) v = A_::scale(v, P.s_red_b[gk / P.red_div]);
+    }
+    return v;
+  };
 
-  for (int k0 = 0; k0 < P.K; k0 += BK) {
-    for (int l = threadIdx.x; l < BM * BK; l += NT) {
-      int i, kk;
-      if (OPA == OP_C) { i = l % BM; kk = l / BM; } else { kk = l % BK; i = l / BK; }
-      const int gi = bm * BM + i, gk = k0 + kk;
-      T v = A_::zero();
-      if (gi < P.M && gk < P.K) {
-        if (OPA == OP_N) v = A[(long long)gi * P.lda + gk];
-        else if (OPA == OP_C) v = A_::cj(A[(long long)gk * P.lda + gi]);
-        else v = A_::cj(A[(long long)gi * P.lda + gk]);
-        if (P.s_red) v = A_::scale(v, P.s_red[gk / P.red_div]);
-      }
-      As[kk][i] = v;
-    }
-    for (int l = threadIdx.x; l < BN * BK; l += NT) {
-      int j, kk;
-      if (OPB == OP_C) { kk = l % BK; j = l / BK; } else { j = l % BN; kk = l / BN; }
-      const int gj = bn * BN + j, gk = k0 + kk;
-      T v = A_::zero();
-      if (gj < P.N && gk < P.K) {
-        if (OPB == OP_N) v = B[(long long)gk * P.ldb + gj];
-        else if (OPB == OP_C) v = A_::cj(B[(long long)gj * P.ldb + gk]);
-        else v = A_::cj(B[(long long)gk * P.ldb + gj]);
-        if (P.s_red_b) v = A_::scale(v, P.s_red_b[gk / P.red_div]);
-      }
-      Bs[kk][j] = v;
-    }
+  const int outs = mt * nt, e = threadIdx.x;
+  const int oi = (e < outs) ? e / nt : 0, oj = (e < outs) ? e - oi * nt : 0;
+  const bool busy = (int)(threadIdx.x & ~31u) < outs;  // the warp holds an output
+  T acc = A_::zero();
+  T va = load_a(kb), vb = load_b(kb);
+  for (int k0 = kb; k0 < ke; k0 += BK) {
+    As[ak][ai] = va;
+    Bs[bk][bj] = vb;
     __syncthreads();
+    if (k0 + BK < ke) {  // the next slab is on its way while this one multiplies
+      va = load_a(k0 + BK);
+      vb = load_b(k0 + BK);
+    }
+    if (busy) {
+      const int kn = min(BK, ke - k0);
+      if (kn == BK) {
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      T a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) A_::mac(acc[i][j], a[i], b[j]);
+        for (int kk = 0; kk < BK; ++kk) A_::mac(acc, As[kk][oi], Bs[kk][oj]);
+      } else {
+        for (int kk = 0; kk < kn; ++kk) A_::mac(acc, As[kk][oi], Bs[kk][oj]);
+      }
     }
     __syncthreads();
   }
 
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gi = bm * BM + ty + 16 * i;
-    if (gi >= P.M) continue;
-    const double sr = P.s_row ? P.s_row[gi / P.row_div] : 1.0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gj = bn * BN + tx + 16 * j;
-      if (gj >= P.N) continue;
-      const double sc = P.s_col ? P.s_col[gj / P.col_div] : 1.0;
-      T v = A_::scale(A_::mul_alpha(acc[i][j], P.alpha_re, P.alpha_im), sr * sc);
-      T* dst = Cm + (long long)gi * P.ldc + gj;
-      *dst = P.accumulate ? A_::add(*dst, v) : v;
-      if (P.herm && bn < bm) {  // mirror an off-diagonal tile into the upper triangle
-        T* mir = Cm + (long long)gj * P.ldc + gi;
-        const T cv = A_::cj(v);
-        *mir = P.accumulate ? A_::add(*mir, cv) : cv;
-      }
+  int e0 = 0, e1 = outs;
+  if (split > 1) {  // add the slices' partial sums; each CTA finishes its share of the outputs
+    part[e] = acc;
+    cluster_sync();
+    const int per = (NT / split);  // at least one warp of outputs each
+    e0 = slice * per;
+    e1 = min(outs, e0 + per);
+    if (e >= e0 && e < e1) {
+      const unsigned first = rank - (unsigned)slice;
+      acc = peer_value(&part[e], first);
+      for (int q = 1; q < split; ++q) acc = A_::add(acc, peer_value(&part[e], first + q));
     }
+    cluster_sync();  // no CTA leaves while another reads its sums
+  }
+  if (e < e0 || e >= e1) return;
+  const int gi = m0 + oi, gj = n0 + oj;
+  const double f = (P.s_row ? P.s_row[gi / P.row_div] : 1.0) * (P.s_col ? P.s_col[gj / P.col_div] : 1.0);
+  const T v = A_::scale(P.alpha_im == 0.0 ? A_::scale(acc, P.alpha_re) : A_::mul_alpha(acc, P.alpha_re, P.alpha_im), f);
+  T* dst = Cm + (long long)gi * P.ldc + gj;
+  *dst = P.accumulate ? A_::add(*dst, v) : v;
+  if (P.herm && bn < bm) {  // mirror an off-diagonal tile into the upper triangle
+    T* mir = Cm + (long long)gj * P.ldc + gi;
+    const T cv = A_::cj(v);
+    *mir = P.accumulate ? A_::add(*mir, cv) : cv;
   }
 }
 
+template <class A_, int OPA, int OPB>
+void launch_one(const GemmBatch& gb, int ctas, bool clustered, cudaStream_t s) {
+  if (!clustered) {
+    gemm_kernel<A_, OPA, OPB><<<ctas, NT, 0, s>>>(gb);
+    return;
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(NT);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = CLUSTER;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, gemm_kernel<A_, OPA, OPB>, gb);  // a failure stays pending for the caller's check
+}
+
 template <class A_>
-void dispatch(const GemmBatch& gb, int tiles, cudaStream_t s) {
+void dispatch(const GemmBatch& gb, int ctas, bool clustered, cudaStream_t s) {
   const int key = gb.opA * 3 + gb.opB;
   switch (key) {
 #define CASE(a, b) \
-  case a * 3 + b: gemm_kernel<A_, a, b><<<tiles, NT, 0, s>>>(gb); break;
+  case a * 3 + b: launch_one<A_, a, b>(gb, ctas, clustered, s); break;
     CASE(0, 0) CASE(0, 1) CASE(0, 2) CASE(1, 0) CASE(1, 1) CASE(1, 2) CASE(2, 0) CASE(2, 1) CASE(2, 2)
 #undef CASE
     default: throw std::runtime_error("bad gemm op");
   }
+}
+
+// Launches the problems [i, n) that fit one batch; returns the index after the last one taken.
+size_t launch_batch(bool cplx, int opA, int opB, const GemmProb* p, size_t i, size_t n, int& launches, cudaStream_t s) {
+  GemmBatch gb{};
+  gb.opA = opA;
+  gb.opB = opB;
+  long long ctas = 0;
+  bool clustered = false;
+  const size_t first = i;
+  for (; i < n && gb.nprob < GEMM_MAXP; ++i) {
+    const GemmProb& q = p[i];
+    if (q.M <= 0 || q.N <= 0 || q.batch <= 0) continue;
+    const int split = split_of(q);
+    long long c = tiles_of(q) * split;
+    c = (c + CLUSTER - 1) / CLUSTER * CLUSTER;
+    if (gb.nprob > 0 && ctas + c > 0x7fffffffLL) break;  // the rest goes to the next launch
+    gb.p[gb.nprob] = q;
+    gb.p[gb.nprob].split = split;
+    clustered = clustered || split > 1;
+    gb.tile_start[gb.nprob++] = (int)ctas;
+    ctas += c;
+  }
+  if (ctas == 0) return std::max(i, first + 1);
+  gb.tile_start[gb.nprob] = (int)ctas;
+  if (cplx) dispatch<C>(gb, (int)ctas, clustered, s); else dispatch<R>(gb, (int)ctas, clustered, s);
+  ++launches;
+  return i;
 }
 
 }  // namespace
@@ -173,17 +292,9 @@ GemmProb& Gemm::add(int M, int N, int K, const void* A, long long lda, const voi
 }
 
 int gemm_launch_single(bool complex_, int opA, int opB, const GemmProb& p, cudaStream_t s) {
-  if (p.M <= 0 || p.N <= 0 || p.batch <= 0) return 0;
-  GemmBatch gb{};
-  gb.opA = opA;
-  gb.opB = opB;
-  gb.nprob = 1;
-  gb.p[0] = p;
-  gb.tile_start[0] = 0;
-  const int tm = (p.M + BM - 1) / BM;
-  gb.tile_start[1] = p.batch * (p.herm ? tm * (tm + 1) / 2 : tm * ((p.N + BN - 1) / BN));
-  if (complex_) dispatch<C>(gb, gb.tile_start[1], s); else dispatch<R>(gb, gb.tile_start[1], s);
-  return 1;
+  int launches = 0;
+  launch_batch(complex_, opA, opB, &p, 0, 1, launches, s);
+  return launches;
 }
 
 int Gemm::launch(cudaStream_t s, bool mixed, int* status) {
@@ -209,25 +320,8 @@ int Gemm::launch(cudaStream_t s, bool mixed, int* status) {
     }
   }
   int launches = 0;
-  size_t i = 0;
-  while (i < probs_.size()) {
-    GemmBatch gb{};
-    gb.opA = opA_; gb.opB = opB_;
-    int tiles = 0;
-    while (i < probs_.size() && gb.nprob < GEMM_MAXP) {
-      const GemmProb& p = probs_[i++];
-      if (p.M <= 0 || p.N <= 0 || p.batch <= 0) continue;
-      gb.p[gb.nprob] = p;
-      gb.tile_start[gb.nprob] = tiles;
-      const int tm = (p.M + BM - 1) / BM;
-      tiles += p.batch * (p.herm ? tm * (tm + 1) / 2 : tm * ((p.N + BN - 1) / BN));
-      gb.nprob++;
-    }
-    gb.tile_start[gb.nprob] = tiles;
-    if (tiles == 0) continue;
-    if (cplx_) dispatch<C>(gb, tiles, s); else dispatch<R>(gb, tiles, s);
-    ++launches;
-  }
+  for (size_t i = 0; i < probs_.size();)
+    i = launch_batch(cplx_, opA_, opB_, probs_.data(), i, probs_.size(), launches, s);
   probs_.clear();
   return launches;
 }

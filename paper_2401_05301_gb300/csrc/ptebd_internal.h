@@ -45,6 +45,7 @@ struct GemmProb {
   int red_div, row_div, col_div, accumulate;
   int herm;  // result is Hermitian (M == N, B = A^+): only lower tiles are computed, then mirrored
   const double* s_red_b;  // optional factor of B along the reduction index (red_div as s_red)
+  int split;  // CTAs of a cluster that share a tile's reduction (set by the launch)
 };
 
 struct GemmBatch {
