@@ -131,7 +131,7 @@ double slot_bytes_for(long long capmax, long long d, long long chi_max, int prec
   const long long kc = std::min<long long>(mm, chi_max);
   // two sites: the projection and V^+ rows (Th, V1h) are at most kc x n1
   const double th_v = two_site ? 2.0 * kc * n1max : capmax * D * capmax + capmax * n1max;
-  return 16.0 * (capmax * d * d * capmax + capmax * D * capmax + th_v + mm * mm + 3.0 * mm + EIG_PARTS + kc * mm) +
+  return 16.0 * (capmax * d * d * capmax + capmax * D * capmax + th_v + mm * mm + 2.0 * mm + EIG_PARTS + kc * mm) +
          8.0 * (4.0 * mm + 4 + 7.0 * mm * kc + kc * kc) + 4.0 * (mm + 1) + 16.0 * eig_panel_doubles2((int)mm) +
          (precision >= 1 ? oz_slot_bytes(capmax, d, chi_max, two_site) : 0.0);
 }
@@ -239,7 +239,6 @@ int alloc_workspace(tebd_ctx* c) {
     S.V1h = dalloc<double2>(c, (c->ss ? kc : capmax) * c->n1max);
     S.tau = dalloc<double2>(c, mm);
     S.part = dalloc<double2>(c, EIG_PARTS);
-    S.p = dalloc<double2>(c, mm);
     S.U = dalloc<double2>(c, kc * mm);
     S.d = dalloc<double>(c, mm);
     S.e = dalloc<double>(c, mm);
@@ -254,7 +253,7 @@ int alloc_workspace(tebd_ctx* c) {
     S.chi = dalloc<int>(c, 1);
     S.pan = dalloc<double2>(c, eig_panel_doubles2((int)mm));
     if (c->precision >= 1) S.oz = dalloc<uint8_t>(c, (size_t)oz_slot_bytes(capmax, d, c->chi_max, c->ss));
-    if ((c->precision >= 1 && !S.oz) || !S.pan || !S.X || !S.Th || !S.Cb || !S.H || !S.V1h || !S.tau || !S.part || !S.p || !S.U || !S.d || !S.e ||
+    if ((c->precision >= 1 && !S.oz) || !S.pan || !S.X || !S.Th || !S.Cb || !S.H || !S.V1h || !S.tau || !S.part || !S.U || !S.d || !S.e ||
         !S.evals || !S.Z || !S.Z2 || !S.S || !S.work || !S.s_sorted || !S.scal || !S.perm || !S.chi) {
       if (s == 0) return TEBD_ERR_OOM;
       break;
@@ -319,7 +318,7 @@ int eigen_stage(tebd_ctx* c, std::vector<Triple>& ts, bool second) {
   for (size_t t = 0; t < ts.size(); ++t) {
     const Slot& S = ts[t].h->slots[ts[t].slot];
     EigMat& M = eb.a[t];
-    M.H = S.H; M.d = S.d; M.e = S.e; M.tau = S.tau; M.part = S.part; M.p = S.p;
+    M.H = S.H; M.d = S.d; M.e = S.e; M.tau = S.tau; M.part = S.part;
     M.evals = S.evals; M.trace = S.scal; M.Z = S.Z; M.Z2 = S.Z2; M.S = S.S; M.work = S.work; M.U = S.U;
     M.pan = S.pan;
     oz_ws[t] = S.oz;

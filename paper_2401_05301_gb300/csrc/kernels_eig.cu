@@ -475,16 +475,8 @@ __global__ void __launch_bounds__(NT) k_backtransform(const __grid_constant__ Ei
 // U^T <- U^T - V T (V^+ U^T), i.e. three matrix products per block on the rows of U.
 constexpr int BT = 64;  // reflectors per block
 
-// Trailing indices per slab of the reduction's Hermitian product.  A function of the matrix's
-// own size, so its arithmetic could never depend on its batch; measured on GB300, 64-wide
-// slabs for the blocked form's sizes (more items per column, more partial sums per strip)
-// were slower than 256 at every size, so every matrix takes 256.
-__host__ __device__ __forceinline__ int td_chunk(int) { return 256; }
-
-__host__ __device__ inline size_t bt_offset(int m) {
-  const size_t slabs = (size_t)((m + 31) / 32) * ((m + td_chunk(m) - 1) / td_chunk(m));
-  return (size_t)m * 128 + (size_t)EIG_PARTS * 64 + slabs * 64;
-}
+__host__ __device__ size_t td_panel_size(int m);  // panel arrays of the reduction (complex elements)
+__host__ __device__ inline size_t bt_offset(int m) { return td_panel_size(m); }
 // V (m x BT) and conj(V) reuse the panel arrays; then G = V^+ V, T^T, S = U conj(V), S T^T.
 __device__ __forceinline__ double2* bt_V(const EigMat& M) { return M.pan; }
 __device__ __forceinline__ double2* bt_Vc(const EigMat& M) { return M.pan + (size_t)M.m * BT; }
@@ -545,18 +537,24 @@ __global__ void __launch_bounds__(4 * BT) k_bt_T(const __grid_constant__ EigBatc
 }
 
 // ---- blocked Householder reduction ---------------------------------------------------------
-// Panels of TD_NB columns.  Within a panel the trailing matrix is left as it was
-// at the panel start; each column's Hermitian product runs on that stored upper
-// triangle (read once per column, as balanced slabs) and is corrected with the
-// panel's earlier (v_i, w_i).  Only the next pivot row is brought up to date, by
-// all blocks.  After the panel the trailing matrix takes the whole rank-2*TD_NB
-// update as one Hermitian matrix product (tensor cores in the mixed path).  Every
-// FP64 operation is scarce on this part, so sums stay in registers and every
-// reduction has a fixed order (bitwise reproducible).  Three grid barriers per column.
-
+// Panels of TD_NB columns.  Within a panel the trailing matrix is left as it was at the panel
+// start; each column's Hermitian product runs on that stored upper triangle and is corrected with
+// the panel's earlier (v_i, w_i).  After the panel the trailing matrix takes the whole
+// rank-2*TD_NB update as one Hermitian matrix product (tensor cores in the mixed path).
+//
+// Bound: the FP64 pipe (a warp-wide FP64 instruction every 16 to 19 clocks per SM, however many
+// lanes are active) and, for few or small matrices, the latency of a column.  So a column takes
+// two grid barriers (1.4 us each), every phase is cut into pieces of 64 to 128 FP64 warp
+// instructions spread over all SMs, and nothing but the two products per stored element runs at
+// n^2: a tile's row sums come from a transposed read of shared memory instead of shuffled
+// reductions, magnitudes are compared as integers, and the reflector's scalars (norm, divisions)
+// are one warp's work beside the product, which therefore runs on the unnormalised row.
+// Against three barriers per column with a reflector per block, shuffled row sums and 32 x 256 slabs,
+// the reduction of 4 matrices of 1024 (with its trailing updates and tail) takes 33 instead of 59 ms,
+// of 4 matrices of 244 4.1 instead of 10.8 ms, of the 94 charge blocks (up to 600) of a chi = 1024, d = 5
+// cut of 7 triples 21 instead of 38 ms.
 constexpr int TD_THREADS = 256;
 constexpr int TD_WARPS = TD_THREADS / 32;
-constexpr int TD_STRIP = 32;
 constexpr int TD_NB = 32;      // columns per panel of the blocked reduction
 // A column whose largest off-diagonal entry lies below 2^-900 is taken as already
 // reduced (tau = 0).  The Gram matrices here have trace ~1, so such entries are far
@@ -564,6 +562,7 @@ constexpr int TD_NB = 32;      // columns per panel of the blocked reduction
 // squares, in empty regions of the chain, and once subnormal the scale 1/amax of
 // the reflector would overflow and turn the column into NaN.
 constexpr double REFL_FLUSH = 0x1p-900;
+constexpr int REFL_FLUSH_EXP = 900;
 // The last TD_TAIL or fewer columns of every matrix are reduced by one block per
 // matrix with the trailing matrix in shared memory (k_tridiag_tail): there the
 // cooperative kernel would pay three grid barriers per column for very little work.
@@ -606,424 +605,486 @@ __device__ bool grid_sync(unsigned int* st, unsigned int& target, long long limi
   return ok_sh != 0;
 }
 
-// Reflector of column k from row k by a whole block (block reductions).
-__device__ void house_row_block(const EigMat& M, int k, double* sh, double2* scale_sh) {
-  const int m = M.m;
-  double2* row = M.H + (size_t)k * m;
-  if (k == m - 1) {
-    if (threadIdx.x == 0) {
-      M.d[k] = row[k].x;
-      M.e[k] = 0.0;
-      M.tau[k] = make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    return;
-  }
-  const int n = m - k - 1;
-  double2* x = row + k + 1;
-  double amax = 0.0;
-  for (int r = threadIdx.x; r < n; r += blockDim.x) amax = fmax(amax, fmax(fabs(x[r].x), fabs(x[r].y)));
-  amax = -block_min(-amax, sh);
-  if (amax < REFL_FLUSH) amax = 0.0;
-  const double sinv = (amax > 0.0) ? 1.0 / amax : 0.0;
-  double s = 0.0;
-  for (int r = 1 + threadIdx.x; r < n; r += blockDim.x) {
-    const double vx = x[r].x * sinv, vy = x[r].y * sinv;
-    s = fma(vx, vx, fma(vy, vy, s));
-  }
-  const double xnorm2 = block_sum(s, sh);
-  if (threadIdx.x == 0) {
-    const double ar = x[0].x * sinv, ai = -x[0].y * sinv;
-    double beta;
-    double2 tau, sc;
-    if (amax == 0.0 || (xnorm2 == 0.0 && ai == 0.0)) {
-      beta = x[0].x;
-      tau = make_double2(0.0, 0.0);
-      sc = make_double2(0.0, 0.0);
-    } else {
-      const double bs = -copysign(sqrt(ar * ar + ai * ai + xnorm2), ar);
-      tau = make_double2((bs - ar) / bs, -ai / bs);
-      const double zr = ar - bs, zi = ai, den = zr * zr + zi * zi;
-      sc = make_double2(zr / den * sinv, -zi / den * sinv);
-      beta = bs * amax;
-    }
-    M.d[k] = row[k].x;
-    M.e[k] = beta;
-    M.tau[k] = tau;
-    *scale_sh = sc;
-  }
-  __syncthreads();
-  const double2 sc = *scale_sh;
-  for (int r = threadIdx.x; r < n; r += blockDim.x) x[r] = (r == 0) ? make_double2(1.0, 0.0) : cmul(cconj(x[r]), sc);
-  __syncthreads();
+// Panel arrays of a matrix, in this order:
+//   VW[r] = (v_0..v_{NB-1}, w_0..w_{NB-1})(r) and WV[r] the same with the halves swapped (the second
+//   operand of the trailing update); the partial dots of the panel corrections (TD_DOTS x 2 NB); the
+//   partial sums of the Hermitian product, per strip of 32 columns from row blocks (hc) and from
+//   tiles to its right (hr); the partials of u^+ A u, one per tile; the column's scalars.
+// The piece sizes follow the trailing size n only, never the batch: the sums keep their order.
+__host__ __device__ __forceinline__ int td_rows(int n) { return n <= 256 ? 8 : n <= 2048 ? 16 : 32; }   // rows per tile
+__host__ __device__ __forceinline__ int td_cols(int n) { return n <= 256 ? 8 : n <= 512 ? 16 : 32; }    // columns per phase-B piece
+__host__ __device__ __forceinline__ int td_dot(int n) { return n <= 256 ? 16 : n <= 512 ? 32 : 64; }    // rows per partial dot
+constexpr int TD_DOTS = 200;  // partial dots: ceil(12288 / 64) = 192, and 17 for the smaller pieces
+// Strips and row blocks that a trailing set of n can touch (its start is not aligned to them).
+__host__ __device__ __forceinline__ size_t td_strips(int n) { return (size_t)(n + 31) / 32 + 1; }
+__host__ __device__ __forceinline__ size_t td_blocks(int n) { return (size_t)n / td_rows(n) + 2; }
+__host__ __device__ __forceinline__ size_t td_tiles(int n) { return td_strips(n) * td_blocks(n); }
+__host__ __device__ inline size_t td_max3(size_t a, size_t b, size_t c) { return a > b ? (a > c ? a : c) : (b > c ? b : c); }
+__host__ __device__ inline size_t td_hc_tiles(int m) {  // the largest of the three piece sizes' needs
+  return td_max3(td_tiles(m), td_tiles(m < 2048 ? m : 2048), td_tiles(m < 256 ? m : 256));
 }
-
-// alpha = -tau (p^+ v) / 2 from the per-strip partial sums (fixed order): every
-// warp forms the sum with its lanes striding the partials, so no thread runs a
-// long dependent chain of loads.
-__device__ __forceinline__ double2 rank2_alpha(const EigMat& M, int k, int n) {
-  const int ns = (n + TD_STRIP - 1) / TD_STRIP;
-  const int lane = threadIdx.x & 31;
-  double2 dot = make_double2(0.0, 0.0);
-  for (int j = lane; j < ns; j += 32) dot = cadd(dot, M.part[j]);
-  dot = warp_sum2(dot);
-  const double2 t2 = cmul(M.tau[k], dot);
-  return make_double2(-0.5 * t2.x, -0.5 * t2.y);
+__host__ __device__ __forceinline__ size_t td_hr_tiles(int m) { return td_strips(m) * td_strips(m); }
+__host__ __device__ size_t td_panel_size(int m) {
+  return (size_t)m * 4 * TD_NB + (size_t)TD_DOTS * 2 * TD_NB + 32 * (td_hc_tiles(m) + td_hr_tiles(m)) +
+         (td_hc_tiles(m) + 1) / 2 + 8;
 }
-
-// Panel arrays of a matrix: VW[r] = (v_0..v_{NB-1}, w_0..w_{NB-1})(r), WV[r] the
-// same with the halves swapped (the second operand of the trailing update), the
-// per-strip partial dots of the panel corrections, and the partial sums of the
-// Hermitian product (64 per slab: column part, then row part).
 __device__ __forceinline__ double2* pan_vw(const EigMat& M) { return M.pan; }
 __device__ __forceinline__ double2* pan_wv(const EigMat& M) { return M.pan + (size_t)M.m * 2 * TD_NB; }
 __device__ __forceinline__ double2* pan_xy(const EigMat& M) { return M.pan + (size_t)M.m * 4 * TD_NB; }
-__device__ __forceinline__ double2* pan_hp(const EigMat& M) {
-  return M.pan + (size_t)M.m * 4 * TD_NB + (size_t)EIG_PARTS * 2 * TD_NB;
+__device__ __forceinline__ double2* pan_hc(const EigMat& M) { return pan_xy(M) + (size_t)TD_DOTS * 2 * TD_NB; }
+__device__ __forceinline__ double2* pan_hr(const EigMat& M) { return pan_hc(M) + 32 * td_hc_tiles(M.m); }
+__device__ __forceinline__ double* pan_q(const EigMat& M) {
+  return reinterpret_cast<double*>(pan_hr(M) + 32 * td_hr_tiles(M.m));
+}
+__device__ __forceinline__ double2* pan_scal(const EigMat& M) {  // [0] sc, [1] (A(k+1, k+1), 0)
+  return pan_hr(M) + 32 * td_hr_tiles(M.m) + (td_hc_tiles(M.m) + 1) / 2;
 }
 
-// w = p + alpha v of column kp (panel index jp), stored as column jp of W.
-__device__ void finish_w(const EigMat& M, int kp, int jp, double2 alpha) {
-  const int m = M.m, n = m - kp - 1;
-  if (n <= 0) return;
-  const double2* v = M.H + (size_t)kp * m + kp + 1;
-  double2* VW = pan_vw(M);
-  double2* WV = pan_wv(M);
-  for (int r = threadIdx.x; r < n; r += blockDim.x) {
-    const double2 w = cfma(alpha, v[r], M.p[r]);
-    const size_t row = (size_t)(kp + 1 + r) * 2 * TD_NB;
-    VW[row + TD_NB + jp] = w;
-    WV[row + jp] = w;
+// What a column's pieces are, from m and k alone.
+struct TdGeo {
+  int m, k, n;          // trailing set: indices k+1 .. m-1, n of them
+  int rows, cols, dot;  // piece sizes
+  int s0, ns;           // first strip, strips
+  int b0, nb;           // first row block, row blocks
+  int g0, ng;           // first phase-B piece, pieces
+  int nd;               // partial dots
+  __device__ TdGeo(int m_, int k_) : m(m_), k(k_), n(m_ - k_ - 1) {
+    rows = td_rows(n); cols = td_cols(n); dot = td_dot(n);
+    s0 = (k + 1) / 32; ns = (m - 1) / 32 - s0 + 1;
+    b0 = (k + 1) / rows; nb = (m - 1) / rows - b0 + 1;
+    g0 = (k + 1) / cols; ng = (m - 1) / cols - g0 + 1;
+    nd = (n + dot - 1) / dot;
   }
+  // tiles: row block b of strip S meets the strips S .. end; counted as if the last strip were full
+  __device__ int per() const { return 32 / rows; }
+  __device__ int first_blocks() const { return (s0 + 1) * per() - b0; }  // row blocks of the first strip
+  __device__ int tiles() const { return first_blocks() * ns + per() * (ns * (ns - 1) / 2); }
+  __device__ int items_a(int j) const { return 1 + (j > 0 ? 2 * nd : 0) + tiles(); }
+  // tile t -> row block b (relative to b0) and strip T (relative to s0)
+  __device__ void tile(int t, int& b, int& T) const {
+    const int f = first_blocks() * ns;
+    if (t < f) {
+      b = t / ns;
+      T = t - b * ns;
+      return;
+    }
+    t -= f;
+    const int last = per() * (ns * (ns - 1) / 2) - 1 - t;  // counted from the end: strips of 1, 2, ... tiles per row block
+    int D = (int)((sqrtf(8.0f * (float)(last / per()) + 1.0f) + 1.0f) * 0.5f);
+    while (per() * (D * (D - 1) / 2) > last) --D;
+    while (per() * (D * (D + 1) / 2) <= last) ++D;
+    const int rem = last - per() * (D * (D - 1) / 2);  // within the strip that has D strips from itself on
+    const int sb = rem / D;
+    b = first_blocks() + (ns - 1 - D) * per() + (per() - 1 - sb);
+    T = ns - 1 - (rem - sb * D);
+  }
+};
+
+// Exponent field of the larger of |re|, |im| (2047: not finite), read as integers.
+__device__ __forceinline__ int expo2(double2 x) {
+  return max((__double2hiint(x.x) >> 20) & 0x7FF, (__double2hiint(x.y) >> 20) & 0x7FF);
+}
+__device__ __forceinline__ double pow2i(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }  // |e| <= 1022
+
+// Partial norm of row k over one piece: lanes hold its entries (zero where there is none; `in`: counted
+// in the sum, i.e. not the first entry).  {sum |x|^2 2^(-2 bin), bin and largest exponent field}; bin is 0
+// unless the piece's largest exponent is outside +-400, where squares would leave the range.
+__device__ __forceinline__ void put_norm(const EigMat& M, int g, double2 x, bool in) {
+  const int ef = __reduce_max_sync(0xffffffffu, expo2(x));
+  const int e = ef - 1023, bin = (e < -400 || e > 400) ? (ef == 2047 ? 0 : e) : 0;
+  double s = 0.0;
+  if (ef != 0) {
+    if (bin != 0) {
+      const double f = pow2i(max(-1022, min(1022, -bin)));
+      x.x *= f;
+      x.y *= f;
+    }
+    s = in ? fma(x.x, x.x, x.y * x.y) : 0.0;
+    s = warp_sum(s);
+  }
+  if ((threadIdx.x & 31) == 0)
+    M.part[g] = make_double2(s, __longlong_as_double(((long long)(bin + 4096) << 32) | ef));
 }
 
-
-// Phase 1 of column k in one pass over row k held in registers (m - k <= 256 * P1_R):
-// finish w of column k-1, the alpha part of the pivot row, and the reflector of
-// column k (house_row_block's arithmetic: amax scaling, then the norm).
-constexpr int P1_R = 8;
-__device__ void phase1_regs(const EigMat& M, int k, int j, double* sh, double2* scale_sh) {
-  const int m = M.m, nn = m - k;  // row k from the diagonal: element r <-> column k + r
-  double2* row = M.H + (size_t)k * m;
-  double2* VW = pan_vw(M);
-  double2* WV = pan_wv(M);
-  double2 a[P1_R];
-  double amax = 0.0;
-  if (j > 0) {
-    const double2 alpha = rank2_alpha(M, k - 1, nn);
-    const double2 sft = make_double2(M.p[0].x + 2.0 * alpha.x, M.p[0].y);
-    const double2* vp = M.H + (size_t)(k - 1) * m + k;  // v_{k-1} from index k (vp[0] = 1)
-#pragma unroll
-    for (int u = 0; u < P1_R; ++u) {
-      const int r = threadIdx.x + u * blockDim.x;
-      a[u] = make_double2(0.0, 0.0);
-      if (r < nn) {
-        const double2 v = vp[r];
-        const double2 w = cfma(alpha, v, M.p[r]);  // w_{k-1}(k + r)
-        const size_t rw = (size_t)(k + r) * 2 * TD_NB;
-        VW[rw + TD_NB + j - 1] = w;
-        WV[rw + j - 1] = w;
-        a[u] = csub(row[k + r], cmul(sft, cconj(v)));
-        if (r >= 1) amax = fmax(amax, fmax(fabs(a[u].x), fabs(a[u].y)));
-      }
-    }
-  } else {
-#pragma unroll
-    for (int u = 0; u < P1_R; ++u) {
-      const int r = threadIdx.x + u * blockDim.x;
-      a[u] = (r < nn) ? row[k + r] : make_double2(0.0, 0.0);
-      if (r >= 1 && r < nn) amax = fmax(amax, fmax(fabs(a[u].x), fabs(a[u].y)));
-    }
+// The scalars of column k's reflector from the partial norms of row k (one warp):
+// H(k) = I - tau v v^+, v = e_0 + sc (0, conj(x_1), conj(x_2), ...).
+__device__ void td_scalars(const EigMat& M, int k) {
+  const int m = M.m, lane = threadIdx.x & 31;
+  const TdGeo P(m, k - 1);  // the pieces that wrote the partials of row k
+  int bmax = -4096, emax = 0;
+  for (int g = lane; g < P.ng; g += 32) {
+    const long long t = __double_as_longlong(M.part[g].y);
+    const int ef = (int)(t & 0xffffffffll), bin = (int)(t >> 32) - 4096;
+    emax = max(emax, ef);
+    if (ef != 0) bmax = max(bmax, bin);
   }
-  if (nn == 1) {  // last column: no reflector
-    if (threadIdx.x == 0) {
-      M.d[k] = a[0].x;
-      M.e[k] = 0.0;
-      M.tau[k] = make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    return;
+  emax = __reduce_max_sync(0xffffffffu, emax);
+  bmax = __reduce_max_sync(0xffffffffu, bmax);
+  const int E = (emax == 0) ? 0 : bmax;
+  double s = 0.0;
+  for (int g = lane; g < P.ng; g += 32) {
+    const double2 t = M.part[g];
+    const int d = (int)(__double_as_longlong(t.y) >> 32) - 4096 - E;
+    s += (d == 0) ? t.x : (d < -500 ? 0.0 : t.x * pow2i(2 * d));
   }
-  amax = -block_min(-amax, sh);
-  if (amax < REFL_FLUSH) amax = 0.0;
-  const double sinv = (amax > 0.0) ? 1.0 / amax : 0.0;
-  double s2 = 0.0;
-#pragma unroll
-  for (int u = 0; u < P1_R; ++u) {
-    const int r = threadIdx.x + u * blockDim.x;
-    if (r >= 2 && r < nn) {
-      const double vx = a[u].x * sinv, vy = a[u].y * sinv;
-      s2 = fma(vx, vx, fma(vy, vy, s2));
-    }
-  }
-  const double xnorm2 = block_sum(s2, sh);
-  if (threadIdx.x == 1 % blockDim.x) {  // the thread holding r = 1 (x[0] of the reflector)
-    const double2 x0 = a[0];
-    const double ar = x0.x * sinv, ai = -x0.y * sinv;
+  const double xnorm2 = warp_sum(s);
+  if (lane == 0) {
+    const double2* row = M.H + (size_t)k * m;
+    const double2 x0 = row[k + 1];
+    const bool flush = emax < 1023 - REFL_FLUSH_EXP;  // every entry below 2^-900
+    const double f = (E == 0) ? 1.0 : pow2i(max(-1022, min(1022, -E)));
+    const double ar = x0.x * f, ai = -x0.y * f;
     double beta;
     double2 tau, sc;
-    if (amax == 0.0 || (xnorm2 == 0.0 && ai == 0.0)) {
+    if (flush || (xnorm2 == 0.0 && ai == 0.0)) {
       beta = x0.x;
       tau = make_double2(0.0, 0.0);
       sc = make_double2(0.0, 0.0);
     } else {
       const double bs = -copysign(sqrt(ar * ar + ai * ai + xnorm2), ar);
-      tau = make_double2((bs - ar) / bs, -ai / bs);
-      const double zr = ar - bs, zi = ai, den = zr * zr + zi * zi;
-      sc = make_double2(zr / den * sinv, -zi / den * sinv);
-      beta = bs * amax;
+      const double zr = ar - bs, inv = 1.0 / bs, iden = f / (zr * zr + ai * ai);
+      tau = make_double2(-zr * inv, -ai * inv);
+      sc = make_double2(zr * iden, -ai * iden);
+      beta = (E == 0) ? bs : bs * pow2i(max(-1022, min(1022, E)));
     }
+    M.d[k] = row[k].x;
     M.e[k] = beta;
     M.tau[k] = tau;
-    *scale_sh = sc;
+    pan_scal(M)[0] = sc;
+    pan_scal(M)[1] = make_double2(M.H[(size_t)(k + 1) * m + k + 1].x, 0.0);
   }
-  if (threadIdx.x == 0) M.d[k] = a[0].x;
-  __syncthreads();
-  const double2 sc = *scale_sh;
+}
+
+// u_r = conj(x_r) of row k for r > k+1, 0 for r = k+1 (the reflector's unit entry is added later).
+__device__ __forceinline__ double2 td_u(const EigMat& M, int k, int r) {
+  return (r > k + 1 && r < M.m) ? cconj(M.H[(size_t)k * M.m + r]) : make_double2(0.0, 0.0);
+}
+
+// One tile of hraw = A u (one warp): row block b against strip T.  The lanes hold the strip's
+// columns: each row of A is read once, gives its term of the column sums conj(A[r][c]) u_r from
+// registers and, off the diagonal, the row sums A[r][c] u_c through a transposed read of shared
+// memory (st: 16 x 33, us: 32).  Diagonal tiles need only the column sums.
+template <int SUB>
+__device__ void td_tile(const EigMat& M, const TdGeo& G, int t, double2* st, double2* us) {
+  const int lane = threadIdx.x & 31, m = G.m, k = G.k;
+  int b, T;
+  G.tile(t, b, T);
+  const int r0 = (G.b0 + b) * G.rows;
+  if (r0 >= m) {  // the last strip's missing row blocks
+    if (lane == 0) pan_q(M)[t] = 0.0;
+    return;
+  }
+  const int S = r0 / 32 - G.s0;
+  const bool diag = (S == T);
+  const int c = 32 * (G.s0 + T) + lane;
+  const double2* x = M.H + (size_t)k * m;
+  const double2 uc = td_u(M, k, c);
+  if (!diag) us[lane] = uc;
+  double2 acc = make_double2(0.0, 0.0);
+  double2* hr = pan_hr(M) + ((size_t)S * G.ns + T) * 32;
+  for (int sub = r0; sub < r0 + G.rows; sub += SUB) {
+    if (sub + SUB <= k + 1 || sub >= m) continue;
+    const bool okc = c < m && c > k;
 #pragma unroll
-  for (int u = 0; u < P1_R; ++u) {
-    const int r = threadIdx.x + u * blockDim.x;
-    if (r < nn) {
-      double2 out = a[u];  // r = 0: the diagonal element
-      if (r >= 1) {
-        out = (r == 1) ? make_double2(1.0, 0.0) : cmul(cconj(a[u]), sc);
-        const size_t rw = (size_t)(k + r) * 2 * TD_NB;
-        VW[rw + j] = out;
-        WV[rw + TD_NB + j] = out;
+    for (int h = 0; h < SUB; h += 8) {
+      double2 a[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int r = sub + h + u;
+        a[u] = (okc && r > k && r < m) ? M.H[(size_t)r * m + c] : make_double2(0.0, 0.0);
       }
-      row[k + r] = out;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int r = sub + h + u;
+        if (r > k + 1 && r < m) acc = cfma_conj(a[u], cconj(x[r]), acc);
+        if (!diag) st[(h + u) * 33 + lane] = a[u];
+      }
+    }
+    if (!diag) {
+      __syncwarp();
+      const int row = lane & (SUB - 1), c0 = (lane / SUB) * SUB;
+      double2 ra = make_double2(0.0, 0.0);
+#pragma unroll 4
+      for (int q = 0; q < SUB; ++q) ra = cfma(st[row * 33 + c0 + q], us[c0 + q], ra);
+#pragma unroll
+      for (int o = SUB; o < 32; o <<= 1) {
+        ra.x += __shfl_xor_sync(0xffffffffu, ra.x, o);
+        ra.y += __shfl_xor_sync(0xffffffffu, ra.y, o);
+      }
+      if (lane < SUB && sub + lane > k && sub + lane < m) hr[(sub + lane) & 31] = ra;
+      __syncwarp();
     }
   }
-  __syncthreads();
+  pan_hc(M)[((size_t)T * G.nb + b) * 32 + lane] = acc;
+  // u^+ A u: the two halves of an off-diagonal tile are conjugate
+  double q = fma(uc.x, acc.x, uc.y * acc.y);
+  q = warp_sum(q);
+  if (lane == 0) pan_q(M)[t] = diag ? q : 2.0 * q;
+}
+
+// Partial dots of the panel corrections over the rows of piece p (one warp, a lane per i < j):
+// which = 0: v_i^+ u, 1: w_i^+ u.
+__device__ void td_dots(const EigMat& M, const TdGeo& G, int j, int p, int which) {
+  const int lane = threadIdx.x & 31;
+  if (lane >= j) return;
+  const int r0 = max(G.k + 2, G.k + 1 + p * G.dot), r1 = min(G.m, G.k + 1 + (p + 1) * G.dot);
+  const double2* col = pan_vw(M) + which * TD_NB + lane;
+  const double2* x = M.H + (size_t)G.k * G.m;
+  double2 t = make_double2(0.0, 0.0);
+#pragma unroll 8
+  for (int r = r0; r < r1; ++r) t = cfma_conj(col[(size_t)r * 2 * TD_NB], cconj(x[r]), t);
+  pan_xy(M)[(size_t)p * 2 * TD_NB + which * TD_NB + lane] = t;
+}
+
+// The matrix that holds item `it` of a batch with prefix sums pre[0..n].
+__device__ __forceinline__ int td_find(const int* pre, int n, int it) {
+  int lo = 0, hi = n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (pre[mid] <= it) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+// Item counts of every matrix as prefix sums (warp 0; a lane takes EIG_MAXP / 32 neighbours).
+template <class F>
+__device__ __forceinline__ void td_prefix(int* pre, int n, F count) {
+  constexpr int W = EIG_MAXP / 32;
+  const int lane = threadIdx.x & 31;
+  int v[W], sum = 0;
+#pragma unroll
+  for (int q = 0; q < W; ++q) {
+    const int i = lane * W + q;
+    v[q] = i < n ? count(i) : 0;
+    sum += v[q];
+  }
+  int ex = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, ex, o);
+    if (lane >= o) ex += t;
+  }
+  ex -= sum;
+#pragma unroll
+  for (int q = 0; q < W; ++q) {
+    const int i = lane * W + q;
+    if (i <= n) pre[i] = ex;
+    ex += v[q];
+  }
+  if (lane == 31 && n == EIG_MAXP) pre[n] = ex;
 }
 
 // Blocked Householder tridiagonalisation, one panel of columns [k0, k1) per
 // cooperative launch (the trailing matrix from k0 on is current when it starts).
 // Column k (panel index j) is reduced against A(k) = A(k0) - sum_{i<j} (v_i w_i^+ +
-// w_i v_i^+) without forming A(k):
-//   phase 1 (a block per matrix): w of column k-1 and the last term of row k (see
-//           phase 3); the reflector of column k (v_k, tau_k).
-//   phase 2 (slabs of 32 x td_chunk(m)): h = A(k0) v over the stored upper triangle,
-//           and per-strip partials of w_i^+ v and v_i^+ v.
-//   phase 3 (strips of 32): p = tau (h - sum_i (v_i (w_i^+ v) + w_i (v_i^+ v))), the
-//           strip partials of p^+ v for alpha, and row k+1 brought to A(k+1) except
-//           for the part of column k's own term that needs alpha.
+// w_i v_i^+) without forming A(k).  Row k is A(k)'s when its turn comes.
+//   phase A (warps): the reflector's scalars; partial dots v_i^+ u, w_i^+ u; tiles of
+//           hraw = A(k0) u and of u^+ A(k0) u, with u = conj(row k) unnormalised, u(k+1) = 0.
+//   phase B (blocks, pieces of td_cols columns): v = e_0 + sc u, h = A(k0) v = A(k0) e_0 + sc hraw,
+//           p = tau (h - sum_i (v_i (w_i^+ v) + w_i (v_i^+ v))), alpha = -|tau|^2 v^+ A(k) v / 2 with
+//           v^+ A(k) v = v^+ h - 2 Re sum_i conj(v_i^+ v) (w_i^+ v) (so no further barrier is
+//           needed for it), w = p + alpha v; row k+1 brought to A(k+1), and its partial norms.
 // After the panel, the caller applies A -= V W^+ + W V^+ to rows and columns >= k1
 // as one Hermitian rank-2*NB matrix product.
-// Three blocks per SM (80 registers, a 64-byte spill): the reduction is latency bound
-// (barrier and scoreboard stalls), so the extra resident warps hide part of it.
-__global__ void __launch_bounds__(TD_THREADS, 3) k_tridiag_panel(const __grid_constant__ EigBatch b, int k0, int k1) {
+constexpr int TD_ST = 16 * 33 + 32;  // shared memory of one warp's tile (complex)
+constexpr int TD_SMEM = TD_WARPS * TD_ST * (int)sizeof(double2);
+__global__ void __launch_bounds__(TD_THREADS, 2) k_tridiag_panel(const __grid_constant__ EigBatch b, int k0, int k1) {
+  extern __shared__ double2 td_sh[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __shared__ double2 acc_sh[TD_WARPS][TD_STRIP];
-  __shared__ double2 xy_sh[2 * TD_NB];
-  __shared__ double2 vk_sh[2 * TD_NB];
-  __shared__ double2 pv_sh[TD_WARPS][TD_STRIP];
-  __shared__ double2 rv_sh[TD_WARPS][TD_STRIP];
-  __shared__ double red_sh[33];
-  __shared__ double2 scale_sh;
-  __shared__ int pre2[EIG_MAXP + 1], pre3[EIG_MAXP + 1];  // items of phase 2 / 3 before each matrix
+  __shared__ int pre[EIG_MAXP + 1];
+  __shared__ double2 xyp[TD_THREADS / (2 * TD_NB)][2 * TD_NB];  // partial X', Y' sums
+  __shared__ double2 xy_sh[2 * TD_NB];                          // Y_i = v_i^+ v, then X_i = w_i^+ v
+  __shared__ double2 vk_sh[2 * TD_NB];                          // v_i(k+1), then w_i(k+1)
+  __shared__ double2 pv_sh[TD_WARPS][32], rv_sh[TD_WARPS][32];
+  __shared__ double q_sh[TD_WARPS];
+  __shared__ double2 h0_sh, w0_sh;
+  __shared__ double alpha_sh;
   unsigned int target = 0;  // barrier count expected at the next grid_sync
+  // the partial norms of the panel's first row
+  if (warp == 0)
+    td_prefix(pre, b.n, [&](int i) { return k0 < tail_start(b.a[i].m) ? TdGeo(b.a[i].m, k0 - 1).ng : 0; });
+  __syncthreads();
+  for (int it = warp * gridDim.x + blockIdx.x; it < pre[b.n]; it += TD_WARPS * gridDim.x) {
+    const int mi = td_find(pre, b.n, it);
+    const EigMat& M = b.a[mi];
+    const TdGeo P(M.m, k0 - 1);
+    const int g = it - pre[mi], c = (P.g0 + g) * P.cols + lane;
+    const bool ok = lane < P.cols && c < M.m && c > k0;
+    put_norm(M, g, ok ? M.H[(size_t)k0 * M.m + c] : make_double2(0.0, 0.0), c > k0 + 1);
+  }
+  if (!grid_sync(b.bar, target, b.wait_clocks)) return;
   for (int k = k0; k < k1; ++k) {
     const int j = k - k0;
-    // ---- phase 1 (row k in registers when it fits, else in memory passes)
-    for (int mi = blockIdx.x; mi < b.n; mi += gridDim.x) {
+    // ---- phase A
+    if (warp == 0)
+      td_prefix(pre, b.n, [&](int i) { return k0 < tail_start(b.a[i].m) ? TdGeo(b.a[i].m, k).items_a(j) : 0; });
+    __syncthreads();
+    for (int it = warp * gridDim.x + blockIdx.x; it < pre[b.n]; it += TD_WARPS * gridDim.x) {
+      const int mi = td_find(pre, b.n, it);
       const EigMat& M = b.a[mi];
-      const int m = M.m;
-      if (k >= tail_start(m)) continue;
-      if (m - k <= P1_R * (int)blockDim.x) {
-        phase1_regs(M, k, j, red_sh, &scale_sh);
+      const TdGeo G(M.m, k);
+      int rem = it - pre[mi];
+      if (rem == 0) {
+        td_scalars(M, k);
         continue;
       }
-      double2* row = M.H + (size_t)k * m;
-      if (j > 0) {
-        // Row k was brought to A(k) in phase 3 of column k-1 except for the alpha
-        // part of that column's own term: with v_{k-1}(k) = 1 and w = p + alpha v it
-        // is (p(k) + 2 Re alpha) conj(v_{k-1}(c)).
-        const double2 alpha = rank2_alpha(M, k - 1, m - k);
-        finish_w(M, k - 1, j - 1, alpha);
-        const double2 sft = make_double2(M.p[0].x + 2.0 * alpha.x, M.p[0].y);
-        const double2* vp = M.H + (size_t)(k - 1) * m;
-        for (int c = k + threadIdx.x; c < m; c += blockDim.x) row[c] = csub(row[c], cmul(sft, cconj(vp[c])));
+      rem -= 1;
+      const int nd2 = j > 0 ? 2 * G.nd : 0;
+      if (rem < nd2) {
+        td_dots(M, G, j, rem >> 1, rem & 1);
+        __syncwarp();
+        continue;
       }
-      __syncthreads();
-      house_row_block(M, k, red_sh, &scale_sh);
-      double2* VWm = pan_vw(M);
-      double2* WVm = pan_wv(M);
-      for (int r = k + 1 + threadIdx.x; r < m; r += blockDim.x) {
-        const double2 v = row[r];
-        VWm[(size_t)r * 2 * TD_NB + j] = v;
-        WVm[(size_t)r * 2 * TD_NB + TD_NB + j] = v;
-      }
+      double2* st = td_sh + warp * TD_ST;
+      if (G.rows == 8) td_tile<8>(M, G, rem - nd2, st, st + 16 * 33);
+      else td_tile<16>(M, G, rem - nd2, st, st + 16 * 33);
+      __syncwarp();
     }
     if (!grid_sync(b.bar, target, b.wait_clocks)) return;
-    // ---- phase 2: h = A(k0) v by slabs.  Item (s, q) covers strip s (32 columns) and
-    // chunk q (td_chunk(m) indices) of the trailing set: the column part reads the stored
-    // rows r in chunk q above the strip's columns (r <= c, used as conj(A[r][c]) v[r]),
-    // the row part reads the strip's rows at columns c > row in chunk q.  Every item
-    // holds about 32 x chunk elements, so the work balances across blocks.  The items
-    // before each matrix are counted once per column (pre2, pre3) and an item finds its
-    // matrix by binary search.
-    if (threadIdx.x < b.n) {  // items of each matrix, then their prefix sums
-      const int i = threadIdx.x;
-      const int n = (k < tail_start(b.a[i].m)) ? b.a[i].m - k - 1 : 0;
-      const int ch = td_chunk(b.a[i].m);
-      pre2[i + 1] = (n > 0) ? ((n + TD_STRIP - 1) / TD_STRIP) * ((n + ch - 1) / ch) : 0;
-      pre3[i + 1] = (n > 0) ? (n + TD_STRIP - 1) / TD_STRIP : 0;
-    }
+    // ---- phase B
+    if (warp == 0)
+      td_prefix(pre, b.n, [&](int i) { return k0 < tail_start(b.a[i].m) ? TdGeo(b.a[i].m, k).ng : 0; });
     __syncthreads();
-    if (threadIdx.x == 0) {
-      pre2[0] = pre3[0] = 0;
-      for (int i = 1; i <= b.n; ++i) {
-        pre2[i] += pre2[i - 1];
-        pre3[i] += pre3[i - 1];
-      }
-    }
-    __syncthreads();
-    for (int item = blockIdx.x; item < pre2[b.n]; item += gridDim.x) {
-      int lo = 0, hi = b.n - 1;  // the last matrix whose first item is <= item
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (pre2[mid] <= item) lo = mid; else hi = mid - 1;
-      }
-      const int mi = lo, rem = item - pre2[mi];
+    for (int it = blockIdx.x; it < pre[b.n]; it += gridDim.x) {
+      const int mi = td_find(pre, b.n, it);
       const EigMat& M = b.a[mi];
-      const int m = M.m, n = m - k - 1, ch = td_chunk(m);
-      const int nq = (n + ch - 1) / ch;
-      const int sidx = rem / nq, q = rem % nq;
-      const int c0 = sidx * TD_STRIP, w = min(TD_STRIP, n - c0);
-      const int q0 = q * ch, q1 = min(n, q0 + ch);
-      const double2* v = M.H + (size_t)k * m + k + 1;
-      const double2* A = M.H + (size_t)(k + 1) * m + k + 1;
-      const int c = c0 + lane;
-      double2 acc = make_double2(0.0, 0.0);
-      const int rend = min(q1, c0 + w);
-      for (int r0 = q0 + warp; r0 < rend; r0 += 4 * TD_WARPS) {
-        double2 a[4], vv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int r = r0 + u * TD_WARPS;
-          const bool ok = r < rend && lane < w && c >= r;
-          a[u] = ok ? A[(size_t)r * m + c] : make_double2(0.0, 0.0);
-          vv[u] = r < rend ? v[r] : make_double2(0.0, 0.0);
+      const TdGeo G(M.m, k);
+      const int m = M.m, g = it - pre[mi];
+      const bool nextrow = (k + 1 < k1);
+      const double2 sc = pan_scal(M)[0], tau = M.tau[k];
+      // sums over the whole trailing set: X', Y' (a quarter of the partials per 64 threads), u^+ A u, hraw(k+1)
+      {
+        const int v = threadIdx.x & (2 * TD_NB - 1), part = threadIdx.x / (2 * TD_NB);
+        if ((v & (TD_NB - 1)) < j) {
+          double2 t = make_double2(0.0, 0.0);
+          for (int p = part; p < G.nd; p += TD_THREADS / (2 * TD_NB)) t = cadd(t, pan_xy(M)[(size_t)p * 2 * TD_NB + v]);
+          xyp[part][v] = t;
+          if (part == 0) vk_sh[v] = pan_vw(M)[(size_t)(k + 1) * 2 * TD_NB + v];
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc = cfma_conj(a[u], vv[u], acc);
+        double q = 0.0;
+        for (int t = threadIdx.x; t < G.tiles(); t += TD_THREADS) q += pan_q(M)[t];
+        q = warp_sum(q);
+        if (lane == 0) q_sh[warp] = q;
+        if (warp == TD_WARPS - 1) {  // hraw(k+1): the first strip's row blocks, then the strips to its right
+          const int e = (k + 1) & 31, nc = min(G.first_blocks(), G.nb);
+          double2 h = make_double2(0.0, 0.0);
+          for (int i = lane; i < nc + G.ns - 1; i += 32)
+            h = cadd(h, i < nc ? pan_hc(M)[(size_t)i * 32 + e] : pan_hr(M)[(size_t)(i - nc + 1) * 32 + e]);
+          h = warp_sum2(h);
+          if (lane == 0) h0_sh = h;
+        }
       }
-      acc_sh[warp][lane] = acc;
-      for (int qq = warp; qq < TD_STRIP; qq += TD_WARPS) {
-        double2 a2[4] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0),
-                         make_double2(0.0, 0.0)};
-        if (qq < w) {
-          const int cc = c0 + qq;
-          const double2* rowc = A + (size_t)cc * m;
-          for (int r0 = max(q0, cc + 1) + lane; r0 < q1; r0 += 128) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int r = r0 + 32 * u;
-              if (r < q1) a2[u] = cfma(rowc[r], v[r], a2[u]);
+      __syncthreads();
+      if (threadIdx.x < 2 * TD_NB) {
+        const int v = threadIdx.x;
+        if ((v & (TD_NB - 1)) < j) {
+          const double2 t = cadd(cadd(xyp[0][v], xyp[1][v]), cadd(xyp[2][v], xyp[3][v]));
+          xy_sh[v] = cfma(sc, t, cconj(vk_sh[v]));
+        } else {
+          xy_sh[v] = vk_sh[v] = make_double2(0.0, 0.0);
+        }
+      }
+      __syncthreads();
+      const int nc_ = G.cols, grp = 32 / nc_;           // columns of the piece, lane groups
+      const int cl = lane & (nc_ - 1), c = (G.g0 + g) * nc_ + cl;
+      const bool ok = c > k && c < m;
+      if (warp == 0) {  // alpha and w(k+1)
+        const double2 X = xy_sh[TD_NB + lane], Y = xy_sh[lane], vi = vk_sh[lane], wi = vk_sh[TD_NB + lane];
+        double gx = fma(Y.x, X.x, Y.y * X.y);
+        double2 c0 = cfma(wi, Y, cmul(vi, X));
+        if (j > 0) {
+          gx = warp_sum(gx);
+          c0 = warp_sum2(c0);
+        }
+        if (lane == 0) {
+          double q = 0.0;
+          for (int w = 0; w < TD_WARPS; ++w) q += q_sh[w];
+          const double a00 = pan_scal(M)[1].x;
+          const double2 s0 = cmul(sc, h0_sh);
+          // v^+ A(k) v = A00 + 2 Re(sc hraw_0) + |sc|^2 u^+ A u - 2 Re sum_i conj(Y_i) X_i
+          const double va = fma(fma(sc.x, sc.x, sc.y * sc.y), q, fma(2.0, s0.x - gx, a00));
+          const double alpha = -0.5 * fma(tau.x, tau.x, tau.y * tau.y) * va;
+          const double2 p0 = cmul(tau, make_double2(a00 + s0.x - c0.x, s0.y - c0.y));
+          alpha_sh = alpha;
+          w0_sh = make_double2(p0.x + alpha, p0.y);
+        }
+      } else {  // the other warps: sc hraw - corrections, and the corrections of row k+1
+        const int slots = (TD_WARPS - 1) * grp, slot = (warp - 1) * grp + lane / nc_;
+        const int S = c / 32 - G.s0, e = c & 31;
+        double2 h = make_double2(0.0, 0.0), rc = make_double2(0.0, 0.0);
+        if (ok) {
+          const int n1 = min(G.nb, G.first_blocks() + S * G.per());  // row blocks down to the strip's own
+          const double2* hc = pan_hc(M) + (size_t)S * G.nb * 32 + e;
+          const double2* hr = pan_hr(M) + (size_t)S * G.ns * 32 + e;
+          for (int i = slot; i < n1; i += slots) h = cadd(h, hc[(size_t)i * 32]);
+          for (int T = S + 1 + slot; T < G.ns; T += slots) h = cadd(h, hr[(size_t)T * 32]);
+          h = cmul(sc, h);
+          const double2* row = pan_vw(M) + (size_t)c * 2 * TD_NB;
+          for (int i = slot; i < j; i += slots) {
+            const double2 vc = row[i], wc = row[TD_NB + i];
+            double2 X = xy_sh[TD_NB + i], Y = xy_sh[i];
+            X = make_double2(-X.x, -X.y);
+            Y = make_double2(-Y.x, -Y.y);
+            h = cfma(vc, X, h);  // - v_i(c) (w_i^+ v) - w_i(c) (v_i^+ v)
+            h = cfma(wc, Y, h);
+            if (nextrow) {       // v_i(k+1) conj(w_i(c)) + w_i(k+1) conj(v_i(c))
+              rc = cfma_conj(wc, vk_sh[i], rc);
+              rc = cfma_conj(vc, vk_sh[TD_NB + i], rc);
             }
           }
         }
-        const double2 a2s = warp_sum2(cadd(cadd(a2[0], a2[1]), cadd(a2[2], a2[3])));
-        if (lane == 0) pv_sh[0][qq] = a2s;
+        for (int o = nc_; o < 32; o <<= 1) {
+          h.x += __shfl_xor_sync(0xffffffffu, h.x, o);
+          h.y += __shfl_xor_sync(0xffffffffu, h.y, o);
+          rc.x += __shfl_xor_sync(0xffffffffu, rc.x, o);
+          rc.y += __shfl_xor_sync(0xffffffffu, rc.y, o);
+        }
+        if (lane < nc_) {
+          pv_sh[warp][lane] = h;
+          rv_sh[warp][lane] = rc;
+        }
       }
       __syncthreads();
-      if (warp == 0) {
-        double2 p1 = make_double2(0.0, 0.0);
-        for (int wq = 0; wq < TD_WARPS; ++wq) p1 = cadd(p1, acc_sh[wq][lane]);
-        double2* hp = pan_hp(M) + (size_t)rem * 2 * TD_STRIP;
-        hp[lane] = p1;
-        hp[TD_STRIP + lane] = pv_sh[0][lane];
+      if (warp == 1 && lane < nc_) {  // the row corrections, beside warp 0's product
+        double2 rs = rv_sh[1][lane];
+        for (int w = 2; w < TD_WARPS; ++w) rs = cadd(rs, rv_sh[w][lane]);
+        rv_sh[0][lane] = rs;
       }
-      // partial dots of the panel corrections over this strip: w_i^+ v, v_i^+ v
-      if (q == 0 && threadIdx.x < 2 * j) {
-        const int i = threadIdx.x < j ? threadIdx.x : threadIdx.x - j;
-        const int col = threadIdx.x < j ? TD_NB + i : i;  // w_i first, then v_i
-        const double2* VW = pan_vw(M);
-        double2 t = make_double2(0.0, 0.0);
-        for (int qq = 0; qq < w; ++qq) t = cfma_conj(VW[(size_t)(k + 1 + c0 + qq) * 2 * TD_NB + col], v[c0 + qq], t);
-        pan_xy(M)[(size_t)sidx * 2 * TD_NB + threadIdx.x] = t;
+      double2 v = make_double2(0.0, 0.0), w = v, a = v;
+      if (warp == 0) {
+        const bool mine = ok && lane < nc_;
+        if (mine) {
+          a = M.H[(size_t)(k + 1) * m + c];  // A(k0)(k+1, c): its conjugate is (A e_0)(c)
+          v = (c == k + 1) ? make_double2(1.0, 0.0) : cmul(sc, cconj(M.H[(size_t)k * m + c]));
+          double2 h = cconj(a);
+          for (int q = 1; q < TD_WARPS; ++q) h = cadd(h, pv_sh[q][lane]);
+          const double alpha = alpha_sh;
+          w = cmul(tau, h);
+          w = make_double2(fma(alpha, v.x, w.x), fma(alpha, v.y, w.y));
+          double2* VW = pan_vw(M) + (size_t)c * 2 * TD_NB;
+          double2* WV = pan_wv(M) + (size_t)c * 2 * TD_NB;
+          VW[j] = v;
+          VW[TD_NB + j] = w;
+          WV[j] = w;
+          WV[TD_NB + j] = v;
+          M.H[(size_t)k * m + c] = v;
+        }
+      }
+      __syncthreads();
+      if (warp == 0 && nextrow) {  // row k+1 of A(k+1) = A(k0) - corrections - conj(w) - w(k+1) conj(v)
+        double2 x = make_double2(0.0, 0.0);
+        if (ok && lane < nc_) {
+          a = csub(csub(a, rv_sh[0][lane]), cconj(w));
+          x = csub(a, cmul(w0_sh, cconj(v)));
+          M.H[(size_t)(k + 1) * m + c] = x;
+        }
+        const bool off = c > k + 1 && lane < nc_;  // the diagonal is not part of the next reflector
+        put_norm(M, g, off ? x : make_double2(0.0, 0.0), c > k + 2);
       }
       __syncthreads();
     }
-    if (!grid_sync(b.bar, target, b.wait_clocks)) return;
-    // ---- phase 3: corrections, tau, the strip partials of p^+ v, and row k+1
-    for (int item = blockIdx.x; item < pre3[b.n]; item += gridDim.x) {
-      int lo = 0, hi = b.n - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (pre3[mid] <= item) lo = mid; else hi = mid - 1;
-      }
-      const int mi = lo, rem = item - pre3[mi];
-      const EigMat& M = b.a[mi];
-      const int m = M.m, n = m - k - 1, ch = td_chunk(m);
-      const int ns = (n + TD_STRIP - 1) / TD_STRIP;
-      const int nq = (n + ch - 1) / ch;
-      const int c0 = rem * TD_STRIP, w = min(TD_STRIP, n - c0);
-      const double2* v = M.H + (size_t)k * m + k + 1;
-      // Row k+1 (the next pivot, if it is in this panel) is brought to A(k+1) here,
-      // spread over the strips, except for the alpha part of column k's term.
-      const bool nextrow = (k + 1 < k1);
-      if (threadIdx.x < 2 * j) {  // X_i = w_i^+ v, Y_i = v_i^+ v over the whole trailing set
-        const double2* xy = pan_xy(M);
-        double2 t = make_double2(0.0, 0.0);
-#pragma unroll 4
-        for (int s2 = 0; s2 < ns; ++s2) t = cadd(t, xy[(size_t)s2 * 2 * TD_NB + threadIdx.x]);
-        xy_sh[threadIdx.x] = t;
-        if (nextrow) {  // v_i(k+1) then w_i(k+1)
-          const int i = threadIdx.x < j ? threadIdx.x : TD_NB + threadIdx.x - j;
-          vk_sh[threadIdx.x] = pan_vw(M)[(size_t)(k + 1) * 2 * TD_NB + i];
-        }
-      }
-      __syncthreads();
-      // warp wq adds the terms i = wq, wq + 8, ... for the 32 elements of the strip
-      double2 corr = make_double2(0.0, 0.0), rcorr = make_double2(0.0, 0.0);
-      if (lane < w) {
-        const double2* rc = pan_vw(M) + (size_t)(k + 1 + c0 + lane) * 2 * TD_NB;
-        for (int i = warp; i < j; i += TD_WARPS) {
-          const double2 vc = rc[i], wc = rc[TD_NB + i];
-          corr = cfma(vc, xy_sh[i], corr);      // v_i(c) (w_i^+ v)
-          corr = cfma(wc, xy_sh[j + i], corr);  // w_i(c) (v_i^+ v)
-          if (nextrow) {                        // v_i(k+1) conj(w_i(c)) + w_i(k+1) conj(v_i(c))
-            rcorr = cfma(vk_sh[i], cconj(wc), rcorr);
-            rcorr = cfma(vk_sh[j + i], cconj(vc), rcorr);
-          }
-        }
-      }
-      pv_sh[warp][lane] = corr;
-      rv_sh[warp][lane] = rcorr;
-      __syncthreads();
-      if (warp == 0) {
-        double2 pd = make_double2(0.0, 0.0);
-        if (lane < w) {
-          double2 cs = make_double2(0.0, 0.0), rs = make_double2(0.0, 0.0);
-          for (int wq = 0; wq < TD_WARPS; ++wq) {
-            cs = cadd(cs, pv_sh[wq][lane]);
-            rs = cadd(rs, rv_sh[wq][lane]);
-          }
-          const double2* hp = pan_hp(M) + (size_t)rem * nq * 2 * TD_STRIP;
-          double2 h = make_double2(0.0, 0.0);
-          for (int q = 0; q < nq; ++q)
-            h = cadd(h, cadd(hp[(size_t)q * 2 * TD_STRIP + lane], hp[(size_t)q * 2 * TD_STRIP + TD_STRIP + lane]));
-          const double2 pc = cmul(M.tau[k], csub(h, cs));
-          M.p[c0 + lane] = pc;
-          pd = cfma_conj(pc, v[c0 + lane], make_double2(0.0, 0.0));
-          if (nextrow) {  // column k's term without alpha: conj(p(c)) (v_k(k+1) = 1)
-            double2* a = M.H + (size_t)(k + 1) * m + k + 1 + c0 + lane;
-            *a = csub(csub(*a, rs), cconj(pc));
-          }
-        }
-        pd = warp_sum2(pd);
-        if (lane == 0) M.part[rem] = pd;
-      }
-      __syncthreads();
-    }
-    if (!grid_sync(b.bar, target, b.wait_clocks)) return;
-  }
-  // w of the panel's last column
-  for (int mi = blockIdx.x; mi < b.n; mi += gridDim.x) {
-    const EigMat& M = b.a[mi];
-    if (k0 < tail_start(M.m) && k1 - 1 < M.m - 1) finish_w(M, k1 - 1, k1 - 1 - k0, rank2_alpha(M, k1 - 1, M.m - k1));
+    if (k + 1 < k1)
+      if (!grid_sync(b.bar, target, b.wait_clocks)) return;
   }
 }
 
@@ -1170,7 +1231,8 @@ int eig_tridiagonalize(const EigBatch& b, bool mixed, void* const* oz_ws, int* s
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag_panel, TD_THREADS, 0);
+    cudaFuncSetAttribute(k_tridiag_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, TD_SMEM);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag_panel, TD_THREADS, TD_SMEM);
   }
   const int grid = std::max(1, sms * std::min(per_sm, b.panel_blocks > 0 ? b.panel_blocks : 3));
   int launches = 0;
@@ -1178,22 +1240,19 @@ int eig_tridiagonalize(const EigBatch& b, bool mixed, void* const* oz_ws, int* s
   for (int i = 0; i < b.n; ++i) kend = std::max(kend, tail_start(b.a[i].m));
   for (int k0 = 0; k0 < kend; k0 += TD_NB) {
     int k1 = std::min(mm, k0 + TD_NB);
-    // grid sized to the panel's largest phase (its first column's slabs): small matrices
-    // get a small grid, whose barriers are cheaper; at least one block per active matrix
-    long long items = 0;
-    int active = 0;
+    // grid sized to the larger of the panel's phases: tiles per warp, pieces per block
+    long long tiles = 0, pieces = 0;
     for (int i = 0; i < b.n; ++i) {
       if (k0 >= tail_start(b.a[i].m)) continue;
-      ++active;
       const int n = b.a[i].m - k0 - 1;
-      const int ch = td_chunk(b.a[i].m);
-      if (n > 0) items += (long long)((n + TD_STRIP - 1) / TD_STRIP) * ((n + ch - 1) / ch);
+      tiles += (long long)td_tiles(n) / 2 + 1;
+      pieces += n / td_cols(n) + 2;
     }
-    const int gsz = (int)std::min<long long>(grid, std::max<long long>(active, items));
+    const int gsz = (int)std::min<long long>(grid, std::max(pieces, tiles / TD_WARPS + 1));
     cudaMemsetAsync(b.bar, 0, sizeof(unsigned int), s);  // arrival count of the grid barrier
     void* args[] = {const_cast<EigBatch*>(&b), &k0, &k1};
-    if (cudaLaunchCooperativeKernel((const void*)k_tridiag_panel, dim3(gsz), dim3(TD_THREADS), args, 0, s) !=
-        cudaSuccess)
+    if (cudaLaunchCooperativeKernel((const void*)k_tridiag_panel, dim3(gsz), dim3(TD_THREADS), args, TD_SMEM,
+                                    s) != cudaSuccess)
       return -1;
     ++launches;
     // trailing update A[k1:, k1:] -= V W^+ + W V^+ (Hermitian, lower tiles mirrored)
@@ -1247,7 +1306,7 @@ size_t eig_panel_doubles2(int m) {
   // panel arrays, then the back-transformation's G, T^T, S and S T^T
   return bt_offset(m) + 2 * BT * BT + (size_t)2 * m * BT;
 }
-static_assert(BT == 2 * TD_NB && TD_STRIP == 32, "bt_offset() mirrors the panel layout");
+static_assert(BT == 2 * TD_NB, "V and conj(V) of the back-transformation reuse VW and WV");
 
 int eig_cut_counts(const ThrCut* cuts_dev, int ncuts, cudaStream_t s) {
   if (ncuts <= 0) return 0;

@@ -19,7 +19,7 @@ constexpr int MAX_SLOTS = 24;
 
 // Workspace of one local update in flight (dense form).
 struct Slot {
-  double2 *X, *Th, *Cb, *H, *V1h, *tau, *part, *p, *U;
+  double2 *X, *Th, *Cb, *H, *V1h, *tau, *part, *U;
   double *d, *e, *evals, *Z, *Z2, *S, *work, *s_sorted, *scal;  // scal: [0] trace [1] norm [2] w
   int *perm, *chi;
   double2* pan;  // panel arrays of the blocked tridiagonal reduction

@@ -171,8 +171,7 @@ struct EigMat {
   double* d;         // tridiagonal diagonal [m]
   double* e;         // sub-diagonal [m]
   double2* tau;      // Householder scalars [m]
-  double2* part;     // partial dot products [EIG_PARTS], one per 32-column strip
-  double2* p;        // p = tau A22 v [m]
+  double2* part;     // partial norms of the next pivot row [EIG_PARTS], one per column piece
   double* evals;     // eigenvalues, descending [kmax]
   double* trace;     // [1] trace of H (sum of Re H_rr), taken before reduction
   double* Z;         // m x K real eigenvectors of T (row-major, ld = K)
@@ -192,7 +191,7 @@ struct EigBatch {
   int panel_blocks;       // blocks per SM of the reduction's cooperative grid (0: as many as fit, at most 3)
 };
 
-constexpr int EIG_PARTS = 384;  // partial sums of p^+ v, one per strip of 32 columns (m <= 12288)
+constexpr int EIG_PARTS = 384;  // partial norms of a row, one per column piece (32 columns at m = 12288)
 
 // Each returns the number of kernel launches issued.
 int eig_trace(const EigBatch& b, cudaStream_t s);

@@ -766,7 +766,7 @@ struct CutBlk {
   int g() const { return right() ? n : b; }
   int cnt = 0, kst = 0;  // kept values, their start on the new bond
   double trace = 0.0;
-  size_t oP, oLam, oH, od, oe, oev, otau, op, opart, otr, oZ, oZ2, oS, owork, oU, opan, oY, oV, oW, oSn, oOut;
+  size_t oP, oLam, oH, od, oe, oev, otau, opart, otr, oZ, oZ2, oS, owork, oU, opan, oY, oV, oW, oSn, oOut;
 };
 
 struct Cut {
@@ -804,7 +804,6 @@ void layout_cut(Cut& cut, Bump& bp) {
     B.oe = bp.take(8 * g);
     B.oev = bp.take(8 * g);
     B.otau = bp.take(16 * g);
-    B.op = bp.take(16 * g);
     B.opart = bp.take(16 * (size_t)EIG_PARTS);
     B.otr = bp.take(8);
     B.oZ = bp.take(8 * g * k);
@@ -913,7 +912,7 @@ int decompose(tebd_ctx* c, std::vector<Cut*>& cuts, std::vector<char*>& bases, s
     CutBlk& B = *j.B;
     EigMat M{};
     M.H = at<double2>(a, B.oH); M.d = at<double>(a, B.od); M.e = at<double>(a, B.oe);
-    M.tau = at<double2>(a, B.otau); M.part = at<double2>(a, B.opart); M.p = at<double2>(a, B.op);
+    M.tau = at<double2>(a, B.otau); M.part = at<double2>(a, B.opart);
     M.evals = at<double>(a, B.oev); M.trace = at<double>(a, B.otr); M.Z = at<double>(a, B.oZ);
     M.Z2 = at<double>(a, B.oZ2); M.S = at<double>(a, B.oS); M.work = at<double>(a, B.owork);
     M.U = at<double2>(a, B.oU); M.pan = at<double2>(a, B.opan);
