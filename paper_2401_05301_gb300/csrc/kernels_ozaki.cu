@@ -39,7 +39,14 @@
 // (the TMA engine, completion on mbarriers), one thread issues
 // tcgen05.mma.kind::f16 (M = 128, N = 64, K = 16) into eight accumulators that
 // fill the 512 columns of tensor memory, and sixteen warps drain the
-// accumulators into the 64-bit sums after each chunk and write the tile.  Every wait is
+// accumulators into the 64-bit sums after each chunk and write the tile.
+//
+// Digits, row exponents and the final conversion run on the integer pipe: the FP64 pipe takes a
+// warp-wide instruction every 16 to 19 clocks per SM, and the packer and the epilogue of the many
+// products with a short reduction (the rank-64 updates) were bound by it.  Measured against FP64
+// ldexp, conversions and comparisons (same bits): 4096 x 1024 x 256 complex 633 -> 545 us, a step of
+// six small blocked simulations 140 -> 108 ms (1500 products), of the chi = 1024, d = 5 charge blocks
+// on 24 sites 582 -> 510 ms.  Every wait is
 // bounded (~1 s): on timeout the CTA records TEBD_ERR_TIMEOUT, lets its issued
 // copies and MMAs finish (bounded), frees its tensor memory and returns.
 #include "ptebd_internal.h"
@@ -68,6 +75,9 @@ constexpr int OZ_BARS = 16;
 constexpr int OZ_SMEM = 2 * OZ_BSTAGE + OZ_AR * OZ_A_BYTES + 1024 + OZ_BARS * 8 + 64;
 constexpr int OZ_STAGE_LD = 65;                 // epilogue staging row (doubles), padded
 constexpr long long OZ_WAIT = 2000000000LL;     // ~1 s at 2 GHz
+// k-steps up to which the packer finds the row exponents itself: each of a row block's nkt packing
+// blocks then reads all nkt k-steps, against a launch of its own (3 us) for the exponents.
+constexpr int OZ_OWN_EXP = 4;
 constexpr int OZ_BAD = 1 << 20;                 // row exponent of a row holding NaN or Inf
 
 static_assert(OZ_TM * OZ_STAGE_LD * 8 <= 2 * OZ_BSTAGE, "epilogue staging must fit the B stages");
@@ -153,23 +163,37 @@ __device__ __forceinline__ uint32_t swz16(int row, int k) {
   return (uint32_t)(row * 128 + ((((k >> 3) ^ (row & 7)) & 7) << 4) + ((k & 7) << 1));
 }
 
-// The eight balanced base-128 digits of round(x 2^(56 - e)) (|x| < 2^e), taken
-// from |x| with the sign applied afterwards, so that the digits of -x are exactly
-// the negated digits of x (conjugate operands share digits up to sign).
-__device__ __forceinline__ void oz_digits(double x, int e, int (&d)[OZ_S]) {
-  long long F = 0;
-  if (x != 0.0 && e != OZ_BAD) F = __double2ll_rn(ldexp(fabs(x), 56 - e));
-  const int sg = (x < 0.0) ? -1 : 1;
-#pragma unroll
-  for (int s = OZ_S - 1; s >= 1; --s) {
-    const int r = (int)((F + 64) & 127) - 64;
-    d[s] = sg * r;
-    F = (F - r) >> 7;
-  }
-  d[0] = sg * (int)F;
+// round(|x| 2^(56 - e)) for |x| < 2^e, ties to even, from the IEEE-754 fields: the FP64 pipe takes a
+// warp-wide instruction every 16 to 19 clocks per SM, so the packing stays on the integer pipe.
+__device__ __forceinline__ unsigned long long oz_fixed(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)(b >> 52) & 0x7FF;
+  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (ex ? 1ull << 52 : 0ull);
+  const int sh = max(ex, 1) - 1019 - e;  // |x| = m 2^(max(ex, 1) - 1075)
+  if (e == OZ_BAD) return 0;
+  if (sh >= 0) return m << min(sh, 63);
+  if (sh < -54) return 0;
+  return (m + ((1ull << (-sh - 1)) - 1) + ((m >> -sh) & 1)) >> -sh;
 }
 
-__device__ __forceinline__ uint32_t bf16_bits(int v) { return __float_as_uint((float)v) >> 16; }
+// The eight balanced base-128 digits of F with the sign of x, as the bits of floats (exact in bf16:
+// the upper half).  Adding 64 at every digit position makes the lower seven plain bit fields; the
+// sign is applied afterwards, so that the digits of -x are exactly the negated digits of x.
+__device__ __forceinline__ void oz_digits(double x, int e, uint32_t (&d)[OZ_S]) {
+  const unsigned long long F = oz_fixed(x, e) + 0x1020408102040ull;  // sum of 64 * 128^i, i = 0..6
+  const uint32_t sg = (uint32_t)__double2hiint(x) & 0x80000000u;
+  const uint32_t lo = (uint32_t)F & 0xFFFFFFFu, hi = (uint32_t)(F >> 28);
+#pragma unroll
+  for (int s = 0; s < OZ_S; ++s) {
+    const uint32_t w = (s < 4) ? hi : lo;
+    const int f = (s == 0) ? (int)(w >> 21) : (int)((w >> (7 * ((OZ_S - 1 - s) & 3))) & 127u) - 64;
+    // an integer of at most 2^22 as a float: offset it into the last bits of 1.5 * 2^23
+    d[s] = __float_as_uint(__int_as_float(0x4B400000 + f) - 12582912.0f) ^ sg;
+  }
+}
+
+// bf16 pair (u in the lower half) of two floats that bf16 holds exactly
+__device__ __forceinline__ uint32_t bf16_pair(uint32_t u, uint32_t v) { return __byte_perm(u, v, 0x7632); }
 
 // ---- packing ----------------------------------------------------------------------
 
@@ -192,55 +216,61 @@ __device__ __forceinline__ int find_job(const OzPackBatch& pb, int blk) {
   return j;
 }
 
-// Row exponents: one block per 32 rows of a job.
-__global__ void __launch_bounds__(256) k_oz_exp(const __grid_constant__ OzPackBatch pb) {
-  const int j = find_job(pb, blockIdx.x);
-  const OzPackJob& J = pb.job[j];
-  const int rb = blockIdx.x - pb.block_start[j];
+// Magnitude of an element for the row exponents: the upper words of |re|, |im| order as integers.
+__device__ __forceinline__ int mag2(double2 x) {
+  return max(__double2hiint(x.x) & 0x7FFFFFFF, __double2hiint(x.y) & 0x7FFFFFFF);
+}
+
+// Row exponent from the largest upper word (rows of zeros and denormals take the smallest one, at which
+// every denormal is exact).
+__device__ __forceinline__ int row_exp(int hi) {
+  if (hi > 0x7FE1CCF3) return OZ_BAD;  // NaN, Inf or beyond 1e308 somewhere in the row
+  return max(hi >> 20, 1) - 1022;
+}
+
+// Largest magnitude of each of the 32 rows of row block rb into mx[32] (256 threads).
+__device__ __forceinline__ void row_magnitudes(const OzPackJob& J, int rb, int (&part)[8][33]) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __shared__ double part[8][33];
   if (J.ks == 1) {  // rows contiguous along k: a warp per row
 #pragma unroll
     for (int rr = 0; rr < 4; ++rr) {
       const int r = rb * 32 + warp + 8 * rr;
-      double m = 0.0;
+      int m = 0;
       if (r < J.rows)
-        for (int k = lane; k < J.K; k += 32) {
-          const double2 x = job_elem(J, r, k);
-          m = fmax(m, fmax(fabs(x.x), fabs(x.y)));
-        }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+#pragma unroll 4
+        for (int k = lane; k < J.K; k += 32) m = max(m, mag2(job_elem(J, r, k)));
+      m = __reduce_max_sync(0xffffffffu, m);
       if (lane == 0) part[0][warp + 8 * rr] = m;
     }
     __syncthreads();
   } else {  // rows contiguous across lanes: lane = row, warps split k
     const int r = rb * 32 + lane;
-    double m = 0.0;
+    int m = 0;
     if (r < J.rows)
-      for (int k = warp; k < J.K; k += 8) {
-        const double2 x = job_elem(J, r, k);
-        m = fmax(m, fmax(fabs(x.x), fabs(x.y)));
-      }
+#pragma unroll 4
+      for (int k = warp; k < J.K; k += 8) m = max(m, mag2(job_elem(J, r, k)));
     part[warp][lane] = m;
     __syncthreads();
     if (warp == 0) {
-      double t = part[0][lane];
-      for (int w = 1; w < 8; ++w) t = fmax(t, part[w][lane]);
-      part[0][lane] = t;
+      for (int w = 1; w < 8; ++w) m = max(m, part[w][lane]);
+      part[0][lane] = m;
     }
     __syncthreads();
   }
-  if (threadIdx.x < 32) {
-    const double m = part[0][threadIdx.x];
-    int e = 0;
-    if (!(m <= 1.0e308)) e = OZ_BAD;  // NaN or Inf somewhere in the row
-    else if (m > 0.0) frexp(m, &e);   // m < 2^e
-    J.e[rb * 32 + threadIdx.x] = e;
-  }
 }
 
-// Digits: one block per (row block, k-step) of a job; writes one or two planes.
+// Row exponents: one block per 32 rows of a job.
+__global__ void __launch_bounds__(256) k_oz_exp(const __grid_constant__ OzPackBatch pb) {
+  const int j = find_job(pb, blockIdx.x);
+  const OzPackJob& J = pb.job[j];
+  const int rb = blockIdx.x - pb.block_start[j];
+  __shared__ int part[8][33];
+  row_magnitudes(J, rb, part);
+  if (threadIdx.x < 32) J.e[rb * 32 + threadIdx.x] = row_exp(part[0][threadIdx.x]);
+}
+
+// Digits: one block per (row block, k-step) of a job; writes one or two planes.  A job with few
+// k-steps (J.own_exp) finds its row exponents here, reading its rows once more from cache.
 __global__ void __launch_bounds__(256) k_oz_pack(const __grid_constant__ OzPackBatch pb) {
   const int j = find_job(pb, blockIdx.x);
   const OzPackJob& J = pb.job[j];
@@ -249,6 +279,7 @@ __global__ void __launch_bounds__(256) k_oz_pack(const __grid_constant__ OzPackB
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __shared__ double tre[32][33], tim[32][33];
   __shared__ int esh[32];
+  __shared__ int part[8][33];
 #pragma unroll
   for (int rr = 0; rr < 4; ++rr) {
     int row, kk;
@@ -259,7 +290,16 @@ __global__ void __launch_bounds__(256) k_oz_pack(const __grid_constant__ OzPackB
     tre[row][kk] = x.x;
     tim[row][kk] = x.y;
   }
-  if (threadIdx.x < 32) esh[threadIdx.x] = J.e[rb * 32 + threadIdx.x];
+  if (J.own_exp) {
+    row_magnitudes(J, rb, part);
+    if (threadIdx.x < 32) {
+      const int e = row_exp(part[0][threadIdx.x]);
+      esh[threadIdx.x] = e;
+      if (kt == 0) J.e[rb * 32 + threadIdx.x] = e;
+    }
+  } else if (threadIdx.x < 32) {
+    esh[threadIdx.x] = J.e[rb * 32 + threadIdx.x];
+  }
   __syncthreads();
   const size_t blk = ((size_t)kt * J.nrb + rb) * (OZ_BLK / 2);  // in bf16 elements, slice 0
   const size_t slice = (size_t)J.nkt * J.nrb * (OZ_BLK / 2);
@@ -267,7 +307,7 @@ __global__ void __launch_bounds__(256) k_oz_pack(const __grid_constant__ OzPackB
   for (int rr = 0; rr < 4; ++rr) {
     const int row = warp + 8 * rr;
     const int e = esh[row];
-    int dr[OZ_S], di[OZ_S];
+    uint32_t dr[OZ_S], di[OZ_S];
     oz_digits(tre[row][lane], e, dr);
     oz_digits(tim[row][lane], e, di);
     const uint32_t off = swz16(row, 2 * lane) >> 1;
@@ -276,15 +316,12 @@ __global__ void __launch_bounds__(256) k_oz_pack(const __grid_constant__ OzPackB
       uint16_t* P = pl ? J.P1 : J.P0;
       const int type = pl ? J.type1 : J.type0;
       if (!P) continue;
+      const bool swap = type >= 2;  // types: 0 (re, im), 1 (re, -im), 2 (im, re), 3 (-im, re)
+      const uint32_t neg = (type == 1) ? 0x80000000u : (type == 3 ? 0x00008000u : 0u);
 #pragma unroll
-      for (int s = 0; s < OZ_S; ++s) {
-        int u, v;  // types: 0 (re, im), 1 (re, -im), 2 (im, re), 3 (-im, re)
-        if (type == 0) { u = dr[s]; v = di[s]; }
-        else if (type == 1) { u = dr[s]; v = -di[s]; }
-        else if (type == 2) { u = di[s]; v = dr[s]; }
-        else { u = -di[s]; v = dr[s]; }
-        *reinterpret_cast<uint32_t*>(P + s * slice + blk + off) = bf16_bits(u) | (bf16_bits(v) << 16);
-      }
+      for (int s = 0; s < OZ_S; ++s)
+        *reinterpret_cast<uint32_t*>(P + s * slice + blk + off) =
+            (swap ? bf16_pair(di[s], dr[s]) : bf16_pair(dr[s], di[s])) ^ neg;
     }
   }
 }
@@ -306,6 +343,43 @@ __device__ __forceinline__ void tile_of(const OzTile& P, int local, int& mt, int
     ++mt;
   }
   nt = rem;
+}
+
+// (P_hi 2^28 + P_lo) 2^x rounded once to FP64, on the integer pipe.
+__device__ __forceinline__ double oz_value(long long Phi, long long Plo, int x) {
+  unsigned long long lo = (unsigned long long)Phi << 28;
+  long long hi = Phi >> 36;
+  const unsigned long long l2 = lo + (unsigned long long)Plo;
+  hi += (Plo >> 63) + (l2 < lo ? 1 : 0);
+  lo = l2;
+  const bool neg = hi < 0;
+  if (neg) {
+    lo = 0ull - lo;
+    hi = ~hi + (lo == 0 ? 1 : 0);
+  }
+  if (hi == 0 && lo == 0) return 0.0;
+  // the leading 64 bits, and whether anything lies below them
+  int n;  // position of the leading one
+  unsigned long long t, rest;
+  if (hi == 0) {
+    const int z = __clzll((long long)lo);
+    n = 63 - z;
+    t = lo << z;
+    rest = 0;
+  } else {
+    const int z = __clzll(hi);
+    n = 127 - z;
+    t = z ? ((unsigned long long)hi << z) | (lo >> (64 - z)) : (unsigned long long)hi;
+    rest = z ? lo << z : lo;
+  }
+  const int ex = n + x + 1023;
+  const unsigned long long sticky = (t & 0x3FFull) | (rest ? 1ull : 0ull), half = t & 0x400ull;
+  unsigned long long m = t >> 11;  // 53 bits with the leading one
+  if (half && (sticky || (m & 1ull))) ++m;
+  if (ex <= 0 || ex >= 2046)  // near the ends of the range: let the library round or overflow
+    return ldexp(neg ? -(double)m : (double)m, n - 52 + x);
+  const unsigned long long bits = (m + ((unsigned long long)(ex - 1) << 52)) | (neg ? 1ull << 63 : 0ull);
+  return __longlong_as_double((long long)bits);
 }
 
 __global__ void __launch_bounds__(OZ_NT, 1) k_oz_gemm(const __grid_constant__ OzGemmBatch gb) {
@@ -491,20 +565,27 @@ __global__ void __launch_bounds__(OZ_NT, 1) k_oz_gemm(const __grid_constant__ Oz
       for (int i = 0; i < 16; ++i) {
         const int col = nt * OZ_TNC + ((c0 + i) & (OZ_TNC - 1));
         const int eb = (col < P.N) ? P.eB[col] : 0;
-        double v = fma((double)Phi[i], 268435456.0, (double)Plo[i]);
-        v = (ea == OZ_BAD || eb == OZ_BAD) ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(v, ea + eb - 63);
-        stage[il * OZ_STAGE_LD + c0 + i] = v;
+        stage[il * OZ_STAGE_LD + c0 + i] = (ea == OZ_BAD || eb == OZ_BAD) ? __longlong_as_double(0x7ff8000000000000ll)
+                                                                          : oz_value(Phi[i], Plo[i], ea + eb - 63);
       }
       asm volatile("bar.sync 1, %0;" ::"r"(32 * OZ_DW) : "memory");
       const int tid = threadIdx.x;
+      const bool scaled = P.s_row || P.s_col || fabs(P.alpha) != 1.0;  // +-1 takes no FP64 multiply
       for (int e = tid; e < OZ_TM * OZ_TNC; e += 32 * OZ_DW) {
         const int r = e / OZ_TNC, cc = e % OZ_TNC;
         const int i = mt * OZ_TM + r, jj = nt * OZ_TNC + cc;
         if (i >= P.M || jj >= P.N || (P.herm && jj > i)) continue;
-        double f = P.alpha;
-        if (P.s_row) f *= P.s_row[i / P.row_div];
-        if (P.s_col) f *= P.s_col[jj / P.col_div];
-        double2 val = make_double2(stage[r * OZ_STAGE_LD + cc] * f, stage[r * OZ_STAGE_LD + OZ_TNC + cc] * f);
+        double2 val = make_double2(stage[r * OZ_STAGE_LD + cc], stage[r * OZ_STAGE_LD + OZ_TNC + cc]);
+        if (scaled) {
+          double f = P.alpha;
+          if (P.s_row) f *= P.s_row[i / P.row_div];
+          if (P.s_col) f *= P.s_col[jj / P.col_div];
+          val.x *= f;
+          val.y *= f;
+        } else if (P.alpha < 0.0) {
+          val.x = -val.x;
+          val.y = -val.y;
+        }
         if (P.Creal) {  // real result (real operands): only the real part is stored
           double* dst = P.Creal + (long long)i * P.ldc + jj;
           if (P.beta) val.x += *dst;
@@ -613,7 +694,8 @@ int oz_gemm_launch(const std::vector<OzProb>& probs, int* status, cudaStream_t s
       if (gram) {  // b = conj(a): D1 = digits of (ar, ai) = DA, D2 = (-ai, ar)
         ja.P1 = D2; ja.type1 = 3;
       }
-      add_job(eb, eblocks, ja, g.nrbA);
+      ja.own_exp = g.nkt <= OZ_OWN_EXP;
+      if (!ja.own_exp) add_job(eb, eblocks, ja, g.nrbA);
       add_job(pk, pblocks, ja, g.nrbA * g.nkt);
       if (!gram) {
         OzPackJob jb{};
@@ -621,7 +703,8 @@ int oz_gemm_launch(const std::vector<OzProb>& probs, int* status, cudaStream_t s
         jb.conj = p.b.conj; jb.real = p.b.real; jb.rows = p.N; jb.K = p.K; jb.nrb = g.nrbB; jb.nkt = g.nkt; jb.e = eB;
         jb.P0 = D1; jb.type0 = 1;
         jb.P1 = D2; jb.type1 = 2;
-        add_job(eb, eblocks, jb, g.nrbB);
+        jb.own_exp = g.nkt <= OZ_OWN_EXP;
+        if (!jb.own_exp) add_job(eb, eblocks, jb, g.nrbB);
         add_job(pk, pblocks, jb, g.nrbB * g.nkt);
       }
       OzTile& t = gb.p[gb.nprob];
@@ -645,10 +728,13 @@ int oz_gemm_launch(const std::vector<OzProb>& probs, int* status, cudaStream_t s
     pk.block_start[pk.njob] = pblocks;
     gb.tile_start[gb.nprob] = tiles;
     if (tiles > 0) {
-      k_oz_exp<<<eblocks, 256, 0, s>>>(eb);
+      if (eblocks > 0) {
+        k_oz_exp<<<eblocks, 256, 0, s>>>(eb);
+        ++launches;
+      }
       k_oz_pack<<<pblocks, 256, 0, s>>>(pk);
       k_oz_gemm<<<tiles, OZ_NT, OZ_SMEM, s>>>(gb);
-      launches += 3;
+      launches += 2;
     }
     i0 = i1;
   }

@@ -108,6 +108,7 @@ struct OzPackJob {
   uint16_t* P0;  // digit plane written with form type0 (null: none)
   uint16_t* P1;
   int type0, type1;
+  int own_exp;  // the packing blocks find the row exponents themselves
   int* e;  // row exponents [nrb * 32]
 };
 struct OzPackBatch {
