@@ -16,7 +16,7 @@
 using namespace ptebd;
 
 namespace {
-constexpr int MEAS_CHUNK = GEMM_MAXP;
+constexpr int MEAS_CHUNK = 16;  // bonds measured together (buffers of a site tensor each)
 }  // namespace
 
 namespace ptebd {

@@ -12,9 +12,7 @@
 //      eigenvector, LU with partial pivoting of T - lambda I), with
 //      Gram-Schmidt inside groups of nearly equal eigenvalues.
 //   4. Newton-Schulz orthonormalisation Z <- Z (3I - Z^T Z)/2, three rounds.
-//   5. Back-transformation U = Q Z: in blocks of 64 reflectors (compact WY
-//      form) in the tensor-core paths, reflector by reflector with 8
-//      eigenvectors per block in the FP64 path.
+//   5. Back-transformation U = Q Z in blocks of 64 reflectors (compact WY form).
 // All reductions use a fixed order, so results are bitwise reproducible.
 #include "ptebd_internal.h"
 
@@ -414,103 +412,45 @@ __global__ void k_z_to_u(const __grid_constant__ EigBatch b, int use_z2) {
   }
 }
 
-constexpr int CPB = 8;  // eigenvectors per block in the back-transformation
-
-// FP64 path: U <- H(0) H(1) ... H(m-2) U reflector by reflector, one block per CPB
-// eigenvectors; per reflector the CPB dot products v^+ u are reduced together.
-// (On FP64 CUDA cores this keeps more blocks busy than the blocked form's thin products.)
-__global__ void __launch_bounds__(NT) k_backtransform(const __grid_constant__ EigBatch b) {
-  const EigMat& M = b.a[blockIdx.y];
-  const int m = M.m, K = M.K;
-  const int c0 = blockIdx.x * CPB;
-  if (c0 >= K) return;
-  const int ncol = min(CPB, K - c0);
-  __shared__ double2 red[NT / 32][CPB];
-  __shared__ double2 wsh[CPB];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int k = m - 2; k >= 0; --k) {
-    const double2 tau = M.tau[k];
-    if (tau.x == 0.0 && tau.y == 0.0) continue;
-    const int n = m - k - 1;
-    const double2* v = M.H + (size_t)k * m + k + 1;
-    double2 acc[CPB];
-#pragma unroll
-    for (int cc = 0; cc < CPB; ++cc) acc[cc] = make_double2(0.0, 0.0);
-    for (int r = threadIdx.x; r < n; r += blockDim.x) {
-      const double2 vr = v[r];
-#pragma unroll
-      for (int cc = 0; cc < CPB; ++cc)
-        if (cc < ncol) acc[cc] = cfma_conj(vr, M.U[(size_t)(c0 + cc) * m + k + 1 + r], acc[cc]);
-    }
-#pragma unroll
-    for (int cc = 0; cc < CPB; ++cc) {
-      const double2 t = warp_sum2(acc[cc]);
-      if (lane == 0) red[warp][cc] = t;
-    }
-    __syncthreads();
-    if (threadIdx.x < CPB) {
-      double2 t = make_double2(0.0, 0.0);
-      for (int w = 0; w < NT / 32; ++w) t = cadd(t, red[w][threadIdx.x]);
-      wsh[threadIdx.x] = cmul(tau, t);
-    }
-    __syncthreads();
-    for (int r = threadIdx.x; r < n; r += blockDim.x) {
-      const double2 vr = v[r];
-#pragma unroll
-      for (int cc = 0; cc < CPB; ++cc) {
-        if (cc < ncol) {
-          double2* u = M.U + (size_t)(c0 + cc) * m + k + 1 + r;
-          *u = csub(*u, cmul(vr, wsh[cc]));
-        }
-      }
-    }
-    __syncthreads();
-  }
-}
-
 // ---- blocked back-transformation ----------------------------------------------------------
 // U <- Q Z with Q = H(0) H(1) ... H(m-2) is applied as blocks of BT reflectors,
 // Q_p = H(k0) ... H(k0+BT-1) = I - V T V^+ (compact WY form, T upper triangular:
 // T[i][i] = tau_i, T[0:i, i] = -tau_i T[0:i, 0:i] (V^+ V)[0:i, i]), last block first:
 // U^T <- U^T - V T (V^+ U^T), i.e. three matrix products per block on the rows of U.
+// V is read from where the reduction left it: row k of H is v_k, once its part up to the diagonal is
+// cleared.  V^+ V and T do not depend on U, so those of all blocks of all matrices are formed at
+// once (one block each), and only the three products run one block after the other.
+// Measured against T of one block after the other on the chain (165 us each) and, in FP64, reflector by
+// reflector with shuffled dot products: eigenvectors of 4 matrices of 1024 (K = 256) 14.8 -> 10.1 ms, of 4 of
+// 244 (K = 61, FP64) 3.8 -> 1.5 ms, of the chi = 1024, d = 5 charge blocks of 7 triples 11.8 -> 9.7 ms.
 constexpr int BT = 64;  // reflectors per block
 
 __host__ __device__ size_t td_panel_size(int m);  // panel arrays of the reduction (complex elements)
-__host__ __device__ inline size_t bt_offset(int m) { return td_panel_size(m); }
-// V (m x BT) and conj(V) reuse the panel arrays; then G = V^+ V, T^T, S = U conj(V), S T^T.
-__device__ __forceinline__ double2* bt_V(const EigMat& M) { return M.pan; }
-__device__ __forceinline__ double2* bt_Vc(const EigMat& M) { return M.pan + (size_t)M.m * BT; }
-__device__ __forceinline__ double2* bt_G(const EigMat& M) { return M.pan + bt_offset(M.m); }
-__device__ __forceinline__ double2* bt_Tt(const EigMat& M) { return bt_G(M) + BT * BT; }
+__host__ __device__ __forceinline__ int bt_blocks(int m) { return (m - 1 + BT - 1) / BT; }
+// After the panel arrays: conj(V^+ V) of every block, then T^T of every block, then S and S T^T (m x BT each).
+__host__ __device__ __forceinline__ double2* bt_G(const EigMat& M, int p) {
+  return M.pan + td_panel_size(M.m) + (size_t)p * BT * BT;
+}
+__host__ __device__ __forceinline__ double2* bt_Tt(const EigMat& M, int p) { return bt_G(M, bt_blocks(M.m) + p); }
+__host__ __device__ __forceinline__ double2* bt_S(const EigMat& M) { return bt_G(M, 2 * bt_blocks(M.m)); }
 
-// Column i of V = v_{k0+i} (unit entry at row k0+i+1, zero above), from the rows of H.
-__global__ void k_bt_prep(const __grid_constant__ EigBatch b, int k0) {
+// H[k][c] = 0 for c <= k: what is left of row k is v_k.
+__global__ void k_bt_clear(const __grid_constant__ EigBatch b) {
   const EigMat& M = b.a[blockIdx.y];
-  const int m = M.m;
-  if (M.K == 0 || k0 >= m - 1) return;
-  double2* V = bt_V(M);
-  double2* Vc = bt_Vc(M);
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < m * BT; idx += gridDim.x * blockDim.x) {
-    const int r = idx / BT, i = idx % BT, k = k0 + i;
-    double2 v = make_double2(0.0, 0.0);
-    if (k < m - 1) {
-      if (r == k + 1) v = make_double2(1.0, 0.0);
-      else if (r > k + 1) v = M.H[(size_t)k * m + r];
-    }
-    V[idx] = v;
-    Vc[idx] = cconj(v);
-  }
+  if (M.K == 0) return;
+  for (int k = blockIdx.x; k < M.m; k += gridDim.x)
+    for (int c = threadIdx.x; c <= k; c += blockDim.x) M.H[(size_t)k * M.m + c] = make_double2(0.0, 0.0);
 }
 
-// T of the block from G = V^+ V and tau (one block per matrix; four threads per
+// T of block p from conj(V^+ V) and tau (one block per matrix and p; four threads per
 // row of T share each column's sum), written transposed.
-__global__ void __launch_bounds__(4 * BT) k_bt_T(const __grid_constant__ EigBatch b, int k0) {
-  const EigMat& M = b.a[blockIdx.x];
-  const int m = M.m;
+__global__ void __launch_bounds__(4 * BT) k_bt_T(const __grid_constant__ EigBatch b) {
+  const EigMat& M = b.a[blockIdx.y];
+  const int m = M.m, p = blockIdx.x, k0 = p * BT;
   if (M.K == 0 || k0 >= m - 1) return;
   const int nb = min(BT, m - 1 - k0);
   extern __shared__ double2 Tsh[];  // BT x (BT + 1)
-  const double2* G = bt_G(M);
+  const double2* G = bt_G(M, p);    // nb x nb
   for (int idx = threadIdx.x; idx < BT * (BT + 1); idx += blockDim.x) Tsh[idx] = make_double2(0.0, 0.0);
   __syncthreads();
   const int l = threadIdx.x >> 2, part = threadIdx.x & 3;
@@ -518,20 +458,21 @@ __global__ void __launch_bounds__(4 * BT) k_bt_T(const __grid_constant__ EigBatc
     const double2 ti = M.tau[k0 + i];
     double2 acc = make_double2(0.0, 0.0);
     if (l < i)
-      for (int q = l + part; q < i; q += 4) acc = cfma(Tsh[l * (BT + 1) + q], G[q * BT + i], acc);
-    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
-    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
-    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 2);
-    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 2);
-    if (part == 0) {
-      if (l < i) Tsh[l * (BT + 1) + i] = make_double2(-(ti.x * acc.x - ti.y * acc.y), -(ti.x * acc.y + ti.y * acc.x));
-      else if (l == i) Tsh[l * (BT + 1) + i] = ti;
+      for (int q = l + part; q < i; q += 4) acc = cfma(Tsh[l * (BT + 1) + q], G[i * nb + q], acc);
+    if ((threadIdx.x & ~31) < 4 * i) {  // warps without a row of this column add nothing
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 2);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 2);
+      if (part == 0 && l < i)
+        Tsh[l * (BT + 1) + i] = make_double2(-(ti.x * acc.x - ti.y * acc.y), -(ti.x * acc.y + ti.y * acc.x));
     }
+    if (part == 0 && l == i) Tsh[l * (BT + 1) + i] = ti;
     __syncthreads();
   }
-  double2* Tt = bt_Tt(M);
-  for (int idx = threadIdx.x; idx < BT * BT; idx += blockDim.x) {
-    const int r = idx / BT, c = idx % BT;  // Tt[r][c] = T[c][r]
+  double2* Tt = bt_Tt(M, p);
+  for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
+    const int r = idx / nb, c = idx - r * nb;  // Tt[r][c] = T[c][r]
     Tt[idx] = Tsh[c * (BT + 1) + r];
   }
 }
@@ -1303,10 +1244,9 @@ int eig_tridiagonalize(const EigBatch& b, bool mixed, void* const* oz_ws, int* s
 }
 
 size_t eig_panel_doubles2(int m) {
-  // panel arrays, then the back-transformation's G, T^T, S and S T^T
-  return bt_offset(m) + 2 * BT * BT + (size_t)2 * m * BT;
+  // panel arrays, then the back-transformation's V^+ V, T^T, S and S T^T
+  return td_panel_size(m) + (size_t)2 * bt_blocks(m) * BT * BT + (size_t)2 * m * BT;
 }
-static_assert(BT == 2 * TD_NB, "V and conj(V) of the back-transformation reuse VW and WV");
 
 int eig_cut_counts(const ThrCut* cuts_dev, int ncuts, cudaStream_t s) {
   if (ncuts <= 0) return 0;
@@ -1379,31 +1319,38 @@ int eig_vectors(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status,
   const int mm = max_m(b);
   k_z_to_u<<<dim3((mm + 31) / 32, (Kmax + 31) / 32, b.n), dim3(32, 8), 0, s>>>(b, in_z2 ? 1 : 0);
   ++launches;
-  if (!mixed) {
-    k_backtransform<<<dim3((Kmax + CPB - 1) / CPB, b.n), NT, 0, s>>>(b);
-    return launches + 1;
-  }
+  const int nblk = bt_blocks(mm);
+  if (nblk == 0) return launches;  // 1 x 1 matrices only
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_bt_T, cudaFuncAttributeMaxDynamicSharedMemorySize, BT * (BT + 1) * 16);
     attr = true;
   }
-  const int nblk = (mm - 1 + BT - 1) / BT;
+  k_bt_clear<<<dim3(std::min(mm, 152), b.n), 128, 0, s>>>(b);
+  Gemm gG(true, OP_N, OP_C);  // conj(V^+ V): FP64 on the CUDA cores (64 rows per block: too few for a tensor tile's cost)
+  for (int i = 0; i < b.n; ++i) {
+    const EigMat& M = b.a[i];
+    if (M.K == 0) continue;
+    for (int p = 0; p < bt_blocks(M.m); ++p) {
+      const int k0 = p * BT, nb = std::min(BT, M.m - 1 - k0);
+      const double2* V = M.H + (size_t)k0 * M.m + k0 + 1;
+      gG.add(nb, nb, M.m - k0 - 1, V, M.m, V, M.m, bt_G(M, p), nb).herm = 1;
+    }
+  }
+  launches += gG.launch(s);
+  k_bt_T<<<dim3(nblk, b.n), 4 * BT, BT * (BT + 1) * 16, s>>>(b);
+  launches += 2;
   for (int p = nblk - 1; p >= 0; --p) {
     const int k0 = p * BT;
-    k_bt_prep<<<dim3(64, b.n), 256, 0, s>>>(b, k0);
-    ++launches;
-    std::vector<OzProb> oG, oS, oS2, oU;
-    Gemm gG(true, OP_C, OP_N), gS(true, OP_N, OP_CJ), gS2(true, OP_N, OP_N), gU(true, OP_N, OP_C);
+    std::vector<OzProb> oS, oS2, oU;
+    Gemm gS(true, OP_N, OP_C), gN(true, OP_N, OP_N), gU(true, OP_N, OP_N);
     for (int i = 0; i < b.n; ++i) {
       const EigMat& M = b.a[i];
-      const int m = M.m, K = M.K, mr = m - k0 - 1;
+      const int m = M.m, K = M.K, mr = m - k0 - 1, nb = std::min(BT, mr);
       if (K == 0 || mr <= 0) continue;
-      const double2* V = M.pan + (size_t)(k0 + 1) * BT;
-      const double2* Vc = M.pan + (size_t)m * BT + (size_t)(k0 + 1) * BT;
-      double2* G = M.pan + bt_offset(m);
-      double2* Tt = G + BT * BT;
-      double2* S = Tt + BT * BT;
+      const double2* V = M.H + (size_t)k0 * m + k0 + 1;  // row i: v_{k0+i} from index k0 + 1 on
+      const double2* Tt = bt_Tt(M, p);
+      double2* S = bt_S(M);
       double2* S2 = S + (size_t)m * BT;
       double2* U = M.U + k0 + 1;
       if (mixed) {
@@ -1411,39 +1358,31 @@ int eig_vectors(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status,
         q.row_div = q.col_div = 1;
         q.alpha = 1.0;
         q.ws = oz_ws[i];
-        OzProb g = q;  // G = V^+ V
-        g.a = OzOperand{V, 1, BT, nullptr, 1, 1};
-        g.M = g.N = BT; g.K = mr; g.C = G; g.ldc = BT; g.gram = g.herm = 1;
-        oG.push_back(g);
         OzProb t = q;  // S = U conj(V): S[j][i] = sum_r U[j][r] conj(V[r][i])
         t.a = OzOperand{U, m, 1, nullptr, 1, 0};
-        t.b = OzOperand{V, 1, BT, nullptr, 1, 1};
-        t.M = K; t.N = BT; t.K = mr; t.C = S; t.ldc = BT;
+        t.b = OzOperand{V, m, 1, nullptr, 1, 1};
+        t.M = K; t.N = nb; t.K = mr; t.C = S; t.ldc = nb;
         oS.push_back(t);
         OzProb t2 = q;  // S2 = S T^T
-        t2.a = OzOperand{S, BT, 1, nullptr, 1, 0};
-        t2.b = OzOperand{Tt, 1, BT, nullptr, 1, 0};
-        t2.M = K; t2.N = BT; t2.K = BT; t2.C = S2; t2.ldc = BT;
+        t2.a = OzOperand{S, nb, 1, nullptr, 1, 0};
+        t2.b = OzOperand{Tt, 1, nb, nullptr, 1, 0};
+        t2.M = K; t2.N = nb; t2.K = nb; t2.C = S2; t2.ldc = nb;
         oS2.push_back(t2);
         OzProb u = q;  // U -= S2 V^T
-        u.a = OzOperand{S2, BT, 1, nullptr, 1, 0};
-        u.b = OzOperand{V, BT, 1, nullptr, 1, 0};
-        u.M = K; u.N = mr; u.K = BT; u.C = U; u.ldc = m; u.alpha = -1.0; u.beta = 1;
+        u.a = OzOperand{S2, nb, 1, nullptr, 1, 0};
+        u.b = OzOperand{V, 1, m, nullptr, 1, 0};
+        u.M = K; u.N = mr; u.K = nb; u.C = U; u.ldc = m; u.alpha = -1.0; u.beta = 1;
         oU.push_back(u);
       } else {
-        gG.add(BT, BT, mr, V, BT, V, BT, G, BT);
-        gS.add(K, BT, mr, U, m, V, BT, S, BT);
-        gS2.add(K, BT, BT, S, BT, Tt, BT, S2, BT);
-        GemmProb& pu = gU.add(K, mr, BT, S2, BT, Vc, BT, U, m);
+        gS.add(K, nb, mr, U, m, V, m, S, nb);
+        gN.add(K, nb, nb, S, nb, Tt, nb, S2, nb);
+        GemmProb& pu = gU.add(K, mr, nb, S2, nb, V, m, U, m);
         pu.alpha_re = -1.0;
         pu.accumulate = 1;
       }
     }
-    launches += mixed ? oz_gemm_launch(oG, status, s) : gG.launch(s);
-    k_bt_T<<<b.n, 4 * BT, BT * (BT + 1) * 16, s>>>(b, k0);
-    ++launches;
     launches += mixed ? oz_gemm_launch(oS, status, s) : gS.launch(s);
-    launches += mixed ? oz_gemm_launch(oS2, status, s) : gS2.launch(s);
+    launches += mixed ? oz_gemm_launch(oS2, status, s) : gN.launch(s);
     launches += mixed ? oz_gemm_launch(oU, status, s) : gU.launch(s);
   }
   return launches;

@@ -106,8 +106,11 @@ __global__ void __launch_bounds__(NT) gemm_kernel(const __grid_constant__ GemmBa
   __shared__ T part[NT];
 
   // the problem of this CTA: tile_start counts CTAs, a multiple of the cluster size per problem
-  int pi = 0;
-  while (pi + 1 < gb.nprob && (int)blockIdx.x >= gb.tile_start[pi + 1]) ++pi;
+  int pi = 0, hi = gb.nprob - 1;
+  while (pi < hi) {
+    const int mid = (pi + hi + 1) >> 1;
+    if (gb.tile_start[mid] <= (int)blockIdx.x) pi = mid; else hi = mid - 1;
+  }
   const GemmProb& P = gb.p[pi];
   const int split = P.split, local = blockIdx.x - gb.tile_start[pi];
   const unsigned rank = split > 1 ? cluster_rank() : 0;
@@ -277,7 +280,7 @@ size_t launch_batch(bool cplx, int opA, int opB, const GemmProb* p, size_t i, si
 
 }  // namespace
 
-static_assert(sizeof(GemmBatch) < 4000, "kernel parameter block too large");
+static_assert(sizeof(GemmBatch) < 32000, "kernel parameter block too large (32 KB on sm_70 and later)");
 
 GemmProb& Gemm::add(int M, int N, int K, const void* A, long long lda, const void* B, long long ldb, void* C,
                     long long ldc) {

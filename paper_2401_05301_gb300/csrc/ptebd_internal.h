@@ -30,7 +30,7 @@ bool build_gate_supersite(int L, int n_max, double U, double J, double Jnnn, dou
 //   s_red[k / red_div]  multiplies A(i, k) along the reduction index,
 //   s_row[i / row_div], s_col[j / col_div] multiply the result.
 enum { OP_N = 0, OP_C = 1, OP_CJ = 2 };  // CJ: element-wise conjugate, no transpose
-constexpr int GEMM_MAXP = 16;
+constexpr int GEMM_MAXP = 64;  // a batch of the blocked form holds hundreds of small products: fewer launches
 
 struct GemmProb {
   const void* A;
@@ -215,9 +215,8 @@ struct ThrCut {
 };
 int eig_cut_counts(const ThrCut* cuts_dev, int ncuts, cudaStream_t s);
 // Inverse iteration on T for eigenvalues 0..K-1, Newton-Schulz orthonormalisation,
-// and back-transformation U = Q Z: in the mixed path in blocks of 64 reflectors
-// (compact WY form, block products on the exact-digit engine), in the FP64 path
-// reflector by reflector.
+// and back-transformation U = Q Z in blocks of 64 reflectors (compact WY form, block products on
+// the exact-digit engine when mixed).  The matrix's H no longer holds it afterwards.
 // Reads a[i].K (set from the eigenvalues).
 int eig_vectors(const EigBatch& b, bool mixed, void* const* oz_ws, int* status, cudaStream_t s);
 
