@@ -502,7 +502,6 @@ constexpr int TD_NB = 32;      // columns per panel of the blocked reduction
 // below their rounding; they do arise, as rounding noise that each Gram product
 // squares, in empty regions of the chain, and once subnormal the scale 1/amax of
 // the reflector would overflow and turn the column into NaN.
-constexpr double REFL_FLUSH = 0x1p-900;
 constexpr int REFL_FLUSH_EXP = 900;
 // The last TD_TAIL or fewer columns of every matrix are reduced by one block per
 // matrix with the trailing matrix in shared memory (k_tridiag_tail): there the
@@ -1031,120 +1030,130 @@ __global__ void __launch_bounds__(TD_THREADS, 2) k_tridiag_panel(const __grid_co
 
 // The columns [tail_start(m), m) of one matrix per block, unblocked, with the
 // trailing matrix (n <= TD_TAIL, current when the kernel starts) in shared memory
-// as a full Hermitian matrix.  The reflectors are those of the panel kernel
-// (phase1_regs' arithmetic on the pivot row), stored the same way in the rows of H;
-// each column then applies A <- A - v w^+ - w v^+ with p = tau A v,
-// w = p - (tau (p^+ v) / 2) v.  One fixed order per reduction.
+// as a full Hermitian matrix.  The reflectors are those of the panel kernel, stored the same way
+// in the rows of H; each column then applies A <- A - v w^+ - w v^+ with p = tau A v,
+// w = p - (|tau|^2 v^+ A v / 2) v.  One fixed order per reduction.
+// Bound: one SM's FP64 pipe (8 n^2 / 32 warp instructions a column: the product, and the update of one
+// triangle, mirrored) and the chain from a row to its w.  The reflector's scalars are a ninth warp's
+// work beside the product, which runs on the unnormalised row as in the panel kernel.
+// Measured against 8 + 8 instructions per element of the full square and block-wide reductions: the last 64
+// columns of 4 matrices 0.84 -> 0.40 ms, whole matrices of 4 to 24 128 -> 68 us.
 constexpr int TL_LD = TD_TAIL + 1;
-__global__ void __launch_bounds__(256) k_tridiag_tail(const __grid_constant__ EigBatch b) {
+constexpr int TL_WARPS = 8;                       // warps of the product and the update
+constexpr int TL_THREADS = 32 * (TL_WARPS + 1);
+__global__ void __launch_bounds__(TL_THREADS) k_tridiag_tail(const __grid_constant__ EigBatch b) {
   extern __shared__ double2 tl_sh[];
   double2* As = tl_sh;                      // TD_TAIL x TL_LD
   double2* vs = As + TD_TAIL * TL_LD;       // v of the current column
-  double2* ws = vs + TD_TAIL;               // p, then w
-  __shared__ double red_sh[33];
-  __shared__ double2 sc_sh, alpha_sh;
+  double2* ws = vs + TD_TAIL;               // A u, then w
+  __shared__ double2 sc_sh, tau_sh;
+  __shared__ double q_sh[2];
   const EigMat& M = b.a[blockIdx.x];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m = M.m, k0 = tail_start(m), nt = m - k0;
   if (nt <= 0) return;
-  for (int e = threadIdx.x; e < nt * nt; e += blockDim.x) {
-    const int r = e / nt, c = e % nt;
-    if (c >= r) {
+  for (int r = warp; r < nt; r += TL_WARPS + 1)
+    for (int c = r + lane; c < nt; c += 32) {
       const double2 x = M.H[(size_t)(k0 + r) * m + k0 + c];
       As[r * TL_LD + c] = x;
       As[c * TL_LD + r] = cconj(x);
     }
-  }
   __syncthreads();
-  for (int j = 0; j < nt; ++j) {
-    const int k = k0 + j, nn = nt - j;  // row j of the current matrix from its diagonal: nn entries
-    const double2* row = As + j * TL_LD + j;
-    if (nn == 1) {
-      if (threadIdx.x == 0) {
-        M.d[k] = row[0].x;
-        M.e[k] = 0.0;
-        M.tau[k] = make_double2(0.0, 0.0);
-        M.H[(size_t)k * m + k] = row[0];
+  for (int j = 0; j + 1 < nt; ++j) {
+    const int k = k0 + j, n = nt - j - 1;  // trailing indices r = 0..n-1 <-> rows/columns j+1+r
+    const double2* x = As + j * TL_LD + j + 1;                // row j beyond its diagonal
+    double2* At = As + (j + 1) * TL_LD + (j + 1);
+    if (warp == TL_WARPS) {  // the reflector's scalars (td_scalars' arithmetic)
+      const double2 xa = lane < n ? x[lane] : make_double2(0.0, 0.0);
+      const double2 xb = lane + 32 < n ? x[lane + 32] : make_double2(0.0, 0.0);
+      const int ef = __reduce_max_sync(0xffffffffu, max(expo2(xa), expo2(xb))), e = ef - 1023;
+      const int E = (ef != 0 && ef != 2047 && (e < -400 || e > 400)) ? e : 0;
+      const double f = (E == 0) ? 1.0 : pow2i(max(-1022, min(1022, -E)));
+      double s = 0.0;
+      {
+        const double ax = xa.x * f, ay = xa.y * f, bx = xb.x * f, by = xb.y * f;
+        if (lane > 0) s = fma(ax, ax, ay * ay);
+        s = fma(bx, bx, fma(by, by, s));
       }
-      break;
-    }
-    double amax = 0.0;
-    for (int r = 1 + threadIdx.x; r < nn; r += blockDim.x) amax = fmax(amax, fmax(fabs(row[r].x), fabs(row[r].y)));
-    amax = -block_min(-amax, red_sh);
-    if (amax < REFL_FLUSH) amax = 0.0;
-    const double sinv = (amax > 0.0) ? 1.0 / amax : 0.0;
-    double s2 = 0.0;
-    for (int r = 2 + threadIdx.x; r < nn; r += blockDim.x) {
-      const double vx = row[r].x * sinv, vy = row[r].y * sinv;
-      s2 = fma(vx, vx, fma(vy, vy, s2));
-    }
-    const double xnorm2 = block_sum(s2, red_sh);
-    if (threadIdx.x == 0) {
-      const double2 x0 = row[1];
-      const double ar = x0.x * sinv, ai = -x0.y * sinv;
-      double beta;
-      double2 tau, sc;
-      if (amax == 0.0 || (xnorm2 == 0.0 && ai == 0.0)) {
-        beta = x0.x;
-        tau = make_double2(0.0, 0.0);
-        sc = make_double2(0.0, 0.0);
-      } else {
-        const double bs = -copysign(sqrt(ar * ar + ai * ai + xnorm2), ar);
-        tau = make_double2((bs - ar) / bs, -ai / bs);
-        const double zr = ar - bs, zi = ai, den = zr * zr + zi * zi;
-        sc = make_double2(zr / den * sinv, -zi / den * sinv);
-        beta = bs * amax;
+      const double xnorm2 = warp_sum(s);
+      if (lane == 0) {
+        const double ar = xa.x * f, ai = -xa.y * f;
+        double beta;
+        double2 tau, sc;
+        if (ef < 1023 - REFL_FLUSH_EXP || (xnorm2 == 0.0 && ai == 0.0)) {
+          beta = xa.x;
+          tau = make_double2(0.0, 0.0);
+          sc = make_double2(0.0, 0.0);
+        } else {
+          const double bs = -copysign(sqrt(ar * ar + ai * ai + xnorm2), ar);
+          const double zr = ar - bs, inv = 1.0 / bs, iden = f / (zr * zr + ai * ai);
+          tau = make_double2(-zr * inv, -ai * inv);
+          sc = make_double2(zr * iden, -ai * iden);
+          beta = (E == 0) ? bs : bs * pow2i(max(-1022, min(1022, E)));
+        }
+        M.d[k] = As[j * TL_LD + j].x;
+        M.e[k] = beta;
+        M.tau[k] = tau;
+        tau_sh = tau;
+        sc_sh = sc;
       }
-      M.d[k] = row[0].x;
-      M.e[k] = beta;
-      M.tau[k] = tau;
-      M.H[(size_t)k * m + k] = row[0];
-      sc_sh = sc;
-    }
-    __syncthreads();
-    const double2 sc = sc_sh, tau = M.tau[k];
-    const int n = nn - 1;  // trailing indices r = 0..n-1 <-> rows/columns j+1+r
-    for (int r = threadIdx.x; r < n; r += blockDim.x) {
-      const double2 v = (r == 0) ? make_double2(1.0, 0.0) : cmul(cconj(row[1 + r]), sc);
-      vs[r] = v;
-      M.H[(size_t)k * m + k + 1 + r] = v;
-    }
-    __syncthreads();
-    // p = tau A v over the trailing block, four threads per row
-    const double2* At = As + (j + 1) * TL_LD + (j + 1);
-    {
+    } else {  // A u with u = (0, conj(x_1), ...), four threads per row
       const int r = threadIdx.x >> 2, part = threadIdx.x & 3;
-      double2 acc = make_double2(0.0, 0.0);
-      if (r < n)
-        for (int c = part; c < n; c += 4) acc = cfma(At[r * TL_LD + c], vs[c], acc);
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 2);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 2);
-      if (part == 0 && r < n) ws[r] = cmul(tau, acc);
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {  // alpha = -tau (p^+ v) / 2
-      double2 dot = make_double2(0.0, 0.0);
-      for (int r = threadIdx.x; r < n; r += 32) dot = cfma_conj(ws[r], vs[r], dot);
-      dot = warp_sum2(dot);
-      if (threadIdx.x == 0) {
-        const double2 t2 = cmul(tau, dot);
-        alpha_sh = make_double2(-0.5 * t2.x, -0.5 * t2.y);
+      if (8 * warp < n) {
+        double2 acc = make_double2(0.0, 0.0);
+        if (r < n)
+          for (int c = 1 + part; c < n; c += 4) acc = cfma(At[r * TL_LD + c], cconj(x[c]), acc);
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 2);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 2);
+        if (part == 0 && r < n) ws[r] = acc;
       }
     }
     __syncthreads();
-    const double2 alpha = alpha_sh;
-    for (int r = threadIdx.x; r < n; r += blockDim.x) ws[r] = cfma(alpha, vs[r], ws[r]);
-    __syncthreads();
-    double2* Aw = As + (j + 1) * TL_LD + (j + 1);
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-      const int r = e / n, c = e % n;
-      double2 a = Aw[r * TL_LD + c];
-      a = csub(a, cmul(vs[r], cconj(ws[c])));
-      a = csub(a, cmul(ws[r], cconj(vs[c])));
-      Aw[r * TL_LD + c] = a;
+    if (warp < 2) {  // v, g = A v = A e_0 + sc A u, w = tau g - (|tau|^2 Re v^+ g / 2) v
+      const int r = threadIdx.x;
+      const double2 sc = sc_sh, tau = tau_sh;
+      double2 v = make_double2(0.0, 0.0), g = v;
+      if (r < n) {
+        v = (r == 0) ? make_double2(1.0, 0.0) : cmul(sc, cconj(x[r]));
+        g = cfma(sc, ws[r], At[r * TL_LD]);
+        vs[r] = v;
+        M.H[(size_t)k * m + k + 1 + r] = v;
+      }
+      double q = warp_sum(fma(v.x, g.x, v.y * g.y));
+      if (lane == 0) q_sh[warp] = q;
+      asm volatile("bar.sync 1, 64;" ::: "memory");
+      const double alpha = -0.5 * fma(tau.x, tau.x, tau.y * tau.y) * (q_sh[0] + q_sh[1]);
+      if (r < n) {
+        const double2 w = cmul(tau, g);
+        ws[r] = make_double2(fma(alpha, v.x, w.x), fma(alpha, v.y, w.y));
+      }
     }
     __syncthreads();
+    for (int r = warp; r < n; r += TL_WARPS + 1) {
+      const double2 vr = vs[r], wr = ws[r];
+      for (int c = r + lane; c < n; c += 32) {
+        const double2 vc = vs[c], wc = ws[c];
+        double2 a = At[r * TL_LD + c];  // - v_r conj(w_c) - w_r conj(v_c)
+        a.x = fma(-vr.x, wc.x, a.x);
+        a.x = fma(-vr.y, wc.y, a.x);
+        a.y = fma(-vr.y, wc.x, a.y);
+        a.y = fma(vr.x, wc.y, a.y);
+        a.x = fma(-wr.x, vc.x, a.x);
+        a.x = fma(-wr.y, vc.y, a.x);
+        a.y = fma(-wr.y, vc.x, a.y);
+        a.y = fma(wr.x, vc.y, a.y);
+        At[r * TL_LD + c] = a;
+        At[c * TL_LD + r] = cconj(a);
+      }
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    M.d[m - 1] = As[(nt - 1) * TL_LD + nt - 1].x;
+    M.e[m - 1] = 0.0;
+    M.tau[m - 1] = make_double2(0.0, 0.0);
   }
 }
 
@@ -1236,7 +1245,7 @@ int eig_tridiagonalize(const EigBatch& b, bool mixed, void* const* oz_ws, int* s
       cudaFuncSetAttribute(k_tridiag_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, TL_SMEM);
       attr = true;
     }
-    k_tridiag_tail<<<b.n, 256, TL_SMEM, s>>>(b);
+    k_tridiag_tail<<<b.n, TL_THREADS, TL_SMEM, s>>>(b);
     ++launches;
   }
   k_esq<<<dim3(std::max(1, std::min(64, (mm + 255) / 256)), b.n), 256, 0, s>>>(b);
