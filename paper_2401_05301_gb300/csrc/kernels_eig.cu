@@ -12,7 +12,8 @@
 //      eigenvector, LU with partial pivoting of T - lambda I), with
 //      Gram-Schmidt inside groups of nearly equal eigenvalues.
 //   4. Newton-Schulz orthonormalisation Z <- Z (3I - Z^T Z)/2, three rounds.
-//   5. Back-transformation U = Q Z in blocks of 64 reflectors (compact WY form).
+//   5. Back-transformation U = Q Z: in blocks of 64 reflectors (compact WY form) in the tensor-core
+//      paths, reflector by reflector with a warp per eigenvector in the FP64 path.
 // All reductions use a fixed order, so results are bitwise reproducible.
 #include "ptebd_internal.h"
 
@@ -412,7 +413,44 @@ __global__ void k_z_to_u(const __grid_constant__ EigBatch b, int use_z2) {
   }
 }
 
-// ---- blocked back-transformation ----------------------------------------------------------
+// ---- back-transformation, reflector by reflector (FP64 path) ------------------------------
+// U <- H(0) H(1) ... H(m-2) U, a warp per eigenvector, which it keeps in shared memory.  The Gram
+// matrices are graded (rows scaled by lambda), and applying the reflectors one at a time keeps the small
+// leading components of the eigenvectors of small singular values to their own relative accuracy; a
+// compact-WY block of 64 in FP64 loses a digit of them (rows u^+ theta' of a graded 24 to 60 row matrix:
+// 4e-15 against 2e-14 of s_k).
+// Bound: the FP64 pipe, 8 instructions per 32 rows and reflector and 14 for the dot product's sum.
+// Measured: 61 vectors of 4 matrices of 244 1.9 ms (8 vectors per block with block-wide sums 2.7 ms), 8 vectors
+// of matrices of 4 to 24 35 us (167 us).
+constexpr int BTS_SMEM = 12288 * 16;  // one vector of the largest matrix (m <= 12288)
+__global__ void k_backtransform(const __grid_constant__ EigBatch b, int stride) {
+  extern __shared__ double2 bts_sh[];
+  const EigMat& M = b.a[blockIdx.y];
+  const int m = M.m, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int j = blockIdx.x * (blockDim.x >> 5) + warp;
+  if (j >= M.K) return;
+  double2* u = bts_sh + (size_t)warp * stride;
+  double2* out = M.U + (size_t)j * m;
+  for (int r = lane; r < m; r += 32) u[r] = out[r];
+  for (int k = m - 2; k >= 0; --k) {
+    const double2 tau = M.tau[k];
+    if (tau.x == 0.0 && tau.y == 0.0) continue;
+    const double2* v = M.H + (size_t)k * m;
+    const int r0 = ((k + 1) & ~31) + lane;  // rows keep their lane
+    double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int r = r0; r < m; r += 32)
+      if (r > k) acc = cfma_conj(v[r], u[r], acc);
+    double2 w = cmul(tau, warp_sum2(acc));
+    w = make_double2(-w.x, -w.y);
+#pragma unroll 4
+    for (int r = r0; r < m; r += 32)
+      if (r > k) u[r] = cfma(w, v[r], u[r]);
+  }
+  for (int r = lane; r < m; r += 32) out[r] = u[r];
+}
+
+// ---- blocked back-transformation (tensor-core paths) ----------------------------------------
 // U <- Q Z with Q = H(0) H(1) ... H(m-2) is applied as blocks of BT reflectors,
 // Q_p = H(k0) ... H(k0+BT-1) = I - V T V^+ (compact WY form, T upper triangular:
 // T[i][i] = tau_i, T[0:i, i] = -tau_i T[0:i, 0:i] (V^+ V)[0:i, i]), last block first:
@@ -420,9 +458,8 @@ __global__ void k_z_to_u(const __grid_constant__ EigBatch b, int use_z2) {
 // V is read from where the reduction left it: row k of H is v_k, once its part up to the diagonal is
 // cleared.  V^+ V and T do not depend on U, so those of all blocks of all matrices are formed at
 // once (one block each), and only the three products run one block after the other.
-// Measured against T of one block after the other on the chain (165 us each) and, in FP64, reflector by
-// reflector with shuffled dot products: eigenvectors of 4 matrices of 1024 (K = 256) 14.8 -> 10.1 ms, of 4 of
-// 244 (K = 61, FP64) 3.8 -> 1.5 ms, of the chi = 1024, d = 5 charge blocks of 7 triples 11.8 -> 9.7 ms.
+// Measured against T of one block after the other on the chain (165 us each): eigenvectors of 4 matrices of
+// 1024 (K = 256) 14.8 -> 10.1 ms, of the chi = 1024, d = 5 charge blocks of 7 triples 11.8 -> 9.7 ms.
 constexpr int BT = 64;  // reflectors per block
 
 __host__ __device__ size_t td_panel_size(int m);  // panel arrays of the reduction (complex elements)
@@ -1332,8 +1369,14 @@ int eig_vectors(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status,
   if (nblk == 0) return launches;  // 1 x 1 matrices only
   static bool attr = false;
   if (!attr) {
+    cudaFuncSetAttribute(k_backtransform, cudaFuncAttributeMaxDynamicSharedMemorySize, BTS_SMEM);
     cudaFuncSetAttribute(k_bt_T, cudaFuncAttributeMaxDynamicSharedMemorySize, BT * (BT + 1) * 16);
     attr = true;
+  }
+  if (!mixed) {  // as many warps per block as their vectors fit, at most 4: few vectors spread over the SMs
+    const int stride = (mm + 31) & ~31, warps = std::max(1, std::min(4, BTS_SMEM / (stride * 16)));
+    k_backtransform<<<dim3((Kmax + warps - 1) / warps, b.n), 32 * warps, (size_t)warps * stride * 16, s>>>(b, stride);
+    return launches + 1;
   }
   k_bt_clear<<<dim3(std::min(mm, 152), b.n), 128, 0, s>>>(b);
   Gemm gG(true, OP_N, OP_C);  // conj(V^+ V): FP64 on the CUDA cores (64 rows per block: too few for a tensor tile's cost)
@@ -1352,7 +1395,6 @@ int eig_vectors(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status,
   for (int p = nblk - 1; p >= 0; --p) {
     const int k0 = p * BT;
     std::vector<OzProb> oS, oS2, oU;
-    Gemm gS(true, OP_N, OP_C), gN(true, OP_N, OP_N), gU(true, OP_N, OP_N);
     for (int i = 0; i < b.n; ++i) {
       const EigMat& M = b.a[i];
       const int m = M.m, K = M.K, mr = m - k0 - 1, nb = std::min(BT, mr);
@@ -1362,37 +1404,29 @@ int eig_vectors(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status,
       double2* S = bt_S(M);
       double2* S2 = S + (size_t)m * BT;
       double2* U = M.U + k0 + 1;
-      if (mixed) {
-        OzProb q{};
-        q.row_div = q.col_div = 1;
-        q.alpha = 1.0;
-        q.ws = oz_ws[i];
-        OzProb t = q;  // S = U conj(V): S[j][i] = sum_r U[j][r] conj(V[r][i])
-        t.a = OzOperand{U, m, 1, nullptr, 1, 0};
-        t.b = OzOperand{V, m, 1, nullptr, 1, 1};
-        t.M = K; t.N = nb; t.K = mr; t.C = S; t.ldc = nb;
-        oS.push_back(t);
-        OzProb t2 = q;  // S2 = S T^T
-        t2.a = OzOperand{S, nb, 1, nullptr, 1, 0};
-        t2.b = OzOperand{Tt, 1, nb, nullptr, 1, 0};
-        t2.M = K; t2.N = nb; t2.K = nb; t2.C = S2; t2.ldc = nb;
-        oS2.push_back(t2);
-        OzProb u = q;  // U -= S2 V^T
-        u.a = OzOperand{S2, nb, 1, nullptr, 1, 0};
-        u.b = OzOperand{V, 1, m, nullptr, 1, 0};
-        u.M = K; u.N = mr; u.K = nb; u.C = U; u.ldc = m; u.alpha = -1.0; u.beta = 1;
-        oU.push_back(u);
-      } else {
-        gS.add(K, nb, mr, U, m, V, m, S, nb);
-        gN.add(K, nb, nb, S, nb, Tt, nb, S2, nb);
-        GemmProb& pu = gU.add(K, mr, nb, S2, nb, V, m, U, m);
-        pu.alpha_re = -1.0;
-        pu.accumulate = 1;
-      }
+      OzProb q{};
+      q.row_div = q.col_div = 1;
+      q.alpha = 1.0;
+      q.ws = oz_ws[i];
+      OzProb t = q;  // S = U conj(V): S[j][i] = sum_r U[j][r] conj(V[r][i])
+      t.a = OzOperand{U, m, 1, nullptr, 1, 0};
+      t.b = OzOperand{V, m, 1, nullptr, 1, 1};
+      t.M = K; t.N = nb; t.K = mr; t.C = S; t.ldc = nb;
+      oS.push_back(t);
+      OzProb t2 = q;  // S2 = S T^T
+      t2.a = OzOperand{S, nb, 1, nullptr, 1, 0};
+      t2.b = OzOperand{Tt, 1, nb, nullptr, 1, 0};
+      t2.M = K; t2.N = nb; t2.K = nb; t2.C = S2; t2.ldc = nb;
+      oS2.push_back(t2);
+      OzProb u = q;  // U -= S2 V^T
+      u.a = OzOperand{S2, nb, 1, nullptr, 1, 0};
+      u.b = OzOperand{V, 1, m, nullptr, 1, 0};
+      u.M = K; u.N = mr; u.K = nb; u.C = U; u.ldc = m; u.alpha = -1.0; u.beta = 1;
+      oU.push_back(u);
     }
-    launches += mixed ? oz_gemm_launch(oS, status, s) : gS.launch(s);
-    launches += mixed ? oz_gemm_launch(oS2, status, s) : gN.launch(s);
-    launches += mixed ? oz_gemm_launch(oU, status, s) : gU.launch(s);
+    launches += oz_gemm_launch(oS, status, s);
+    launches += oz_gemm_launch(oS2, status, s);
+    launches += oz_gemm_launch(oU, status, s);
   }
   return launches;
 }

@@ -215,8 +215,8 @@ struct ThrCut {
 };
 int eig_cut_counts(const ThrCut* cuts_dev, int ncuts, cudaStream_t s);
 // Inverse iteration on T for eigenvalues 0..K-1, Newton-Schulz orthonormalisation,
-// and back-transformation U = Q Z in blocks of 64 reflectors (compact WY form, block products on
-// the exact-digit engine when mixed).  The matrix's H no longer holds it afterwards.
+// and back-transformation U = Q Z: when mixed in blocks of 64 reflectors (compact WY form, block
+// products on the exact-digit engine), else reflector by reflector.  H does not survive it.
 // Reads a[i].K (set from the eigenvalues).
 int eig_vectors(const EigBatch& b, bool mixed, void* const* oz_ws, int* status, cudaStream_t s);
 
