@@ -246,7 +246,7 @@ int alloc_workspace(tebd_ctx* c) {
     S.Z = dalloc<double>(c, mm * kc);
     S.Z2 = dalloc<double>(c, mm * kc);
     S.S = dalloc<double>(c, kc * kc);
-    S.work = dalloc<double>(c, 5 * mm * kc);
+    S.work = dalloc<double>(c, 5 * mm * kc + 4);
     S.s_sorted = dalloc<double>(c, mm);
     S.scal = dalloc<double>(c, 4);
     S.perm = dalloc<int>(c, mm);
@@ -315,6 +315,7 @@ int eigen_stage(tebd_ctx* c, std::vector<Triple>& ts, bool second) {
   eb.bar = c->d_bar;
   eb.wait_clocks = c->wait_clocks;
   eb.panel_blocks = c->panel_blocks;
+  eb.few = 1;
   for (size_t t = 0; t < ts.size(); ++t) {
     const Slot& S = ts[t].h->slots[ts[t].slot];
     EigMat& M = eb.a[t];

@@ -100,109 +100,150 @@ __global__ void k_trace(const __grid_constant__ EigBatch b) {
 }
 
 // ---- bisection --------------------------------------------------------------------
-// Number of eigenvalues of T below x: sign changes of the leading principal
-// minors p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (Sturm's theorem), with
-// a zero minor counted as a change.  Division-free: FP64 division is the
-// slowest operation on this part, and the minors are kept in range by exact
-// rescaling with 2^-500 / 2^500.  ee[i] = e_i^2 (k_esq).  The loop is bound by
-// the FP64 pipe (two DFMA per clock per SM), so only the recurrence itself runs
-// there: the zero, sign and range tests read the IEEE-754 fields with integer
-// operations.  Rescaling by exact powers of two leaves every sign unchanged.
-__device__ __forceinline__ int sturm_count(const double* d, const double* ee, int m, double x) {
-  const double big = 0x1p500, small = 0x1p-500;
-  double pm = 1.0, p = d[0] - x;
-  if (p == 0.0) p = -small;
-  long long bp = __double_as_longlong(p);
-  int cnt = (int)((unsigned long long)bp >> 63);
-  for (int i = 1; i < m; ++i) {
-    double pn = fma(d[i] - x, p, -(ee[i - 1] * pm));
-    long long bn = __double_as_longlong(pn);
-    if ((bn << 1) == 0) {  // a zero minor takes the sign opposite to the previous one
-      pn = (bp < 0) ? small : -small;
-      bn = __double_as_longlong(pn);
-    }
-    cnt += (int)((unsigned long long)(bn ^ bp) >> 63);
-    pm = p;
-    p = pn;
-    bp = bn;
-    const int ex = (int)((bn >> 52) & 0x7FF);
-    if (ex > 1023 + 500) { p *= small; pm *= small; bp = __double_as_longlong(p); }
-    else if (ex < 1023 - 500) { p *= big; pm *= big; bp = __double_as_longlong(p); }
-  }
-  return cnt;
-}
+// The tridiagonals for the Sturm counts, in the inverse-iteration scratch (free until the
+// eigenvectors are computed): T scaled by a power of two (exact) so that its Gershgorin bound lies in
+// [1, 2), as pairs (d_i, e_{i-1}^2), after a header of the scale and the Gershgorin interval.
+struct SturmHead {
+  double gl, gu;  // Gershgorin interval of the scaled T
+  double up, dn;  // scaled = x * up, x = scaled * dn
+};
+__device__ __forceinline__ SturmHead* sturm_head(const EigMat& M) { return reinterpret_cast<SturmHead*>(M.work); }
+__device__ __forceinline__ double2* sturm_pairs(const EigMat& M) { return reinterpret_cast<double2*>(M.work + 4); }
 
-// ee[i] = e_i^2 of every tridiagonal, for the Sturm counts, in the inverse-iteration
-// scratch (free until the eigenvectors are computed).
-__global__ void k_esq(const __grid_constant__ EigBatch b) {
-  const EigMat& M = b.a[blockIdx.y];
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M.m; i += gridDim.x * blockDim.x)
-    M.work[i] = (i < M.m - 1) ? M.e[i] * M.e[i] : 0.0;
-}
-
-__device__ void gershgorin(const double* d, const double* e, int m, double* sh, double& gl, double& gu) {
+__global__ void __launch_bounds__(256) k_sturm_prep(const __grid_constant__ EigBatch b) {
+  const EigMat& M = b.a[blockIdx.x];
+  const int m = M.m;
+  __shared__ double sh[33];
   double lo = DBL_MAX, hi = DBL_MAX;  // hi stored negated for a min-reduction
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
     double r = 0.0;
-    if (i > 0) r += fabs(e[i - 1]);
-    if (i < m - 1) r += fabs(e[i]);
-    lo = fmin(lo, d[i] - r);
-    hi = fmin(hi, -(d[i] + r));
+    if (i > 0) r += fabs(M.e[i - 1]);
+    if (i < m - 1) r += fabs(M.e[i]);
+    lo = fmin(lo, M.d[i] - r);
+    hi = fmin(hi, -(M.d[i] + r));
   }
-  gl = block_min(lo, sh);
-  gu = -block_min(hi, sh);
+  const double gl = block_min(lo, sh), gu = -block_min(hi, sh);
+  const double bn = fmax(fabs(gl), fabs(gu));
+  int e = 0;
+  if (bn > 0.0 && bn < DBL_MAX) e = max(-1020, min(1020, ((__double2hiint(bn) >> 20) & 0x7FF) - 1023));
+  const double up = __longlong_as_double((long long)(1023 - e) << 52), dn = __longlong_as_double((long long)(1023 + e) << 52);
+  if (threadIdx.x == 0) *sturm_head(M) = SturmHead{gl * up, gu * up, up, dn};
+  double2* P = sturm_pairs(M);
+  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    const double ei = (i > 0) ? M.e[i - 1] * up : 0.0;
+    P[i] = make_double2(M.d[i] * up, ei * ei);
+  }
 }
 
-// Multisection with 4 points: a warp serves eight eigenvalues, four lanes each; per
-// iteration the lanes of a group count the eigenvalues below 4 interior points of
-// their interval, which shrinks it 5-fold (~23 iterations to machine precision).
-// The counts are bound by the FP64 pipe once a batch holds many matrices (the
-// blocked form's charge blocks): 4 points take 92 counts per eigenvalue against
-// 136 with 8 points, at 1.35x the serial iterations.
-__global__ void k_bisect(const __grid_constant__ EigBatch b) {
-  const EigMat& M = b.a[blockIdx.y];
-  const int m = M.m;
-  __shared__ double sh[33];
-  double gl, gu;
-  gershgorin(M.d, M.e, m, sh, gl, gu);
-  const int lane = threadIdx.x & 31, g = lane >> 2, sub = lane & 3;
-  const int j = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 8 + g;
+// Number of eigenvalues of the scaled T below x: sign changes of the leading principal
+// minors p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (Sturm's theorem), with
+// a zero minor counted as a change.  Bound: the FP64 pipe, three dependent instructions of 64 clocks
+// a step for a warp alone on its scheduler, so only the recurrence runs there: signs and zeros are
+// read from the upper words, and the range is checked every fourth step only (a step changes the
+// magnitude by less than 2^3 up and 2^60 down: x and d_i are doubles below 4), by exact rescaling.
+__device__ __forceinline__ int sturm_count(const double2* __restrict__ P, int m, double x) {
+  double pm = 0.0, p = 1.0;
+  int hp = 0x3FF00000, cnt = 0;  // upper word of p
+  int i = 0;
+  auto step = [&](double2 t) {
+    double pn = fma(t.x - x, p, -(t.y * pm));
+    int hn = __double2hiint(pn);
+    if (((hn << 1) | __double2loint(pn)) == 0) {  // a zero minor takes the sign opposite to the previous one
+      hn = 0x20B00000 | (~hp & 0x80000000);       // 2^-500
+      pn = __hiloint2double(hn, 0);
+    }
+    cnt += (int)((unsigned)(hn ^ hp) >> 31);
+    pm = p;
+    p = pn;
+    hp = hn;
+  };
+  for (; i + 4 <= m; i += 4) {
+    const double2 t0 = P[i], t1 = P[i + 1], t2 = P[i + 2], t3 = P[i + 3];
+    step(t0);
+    step(t1);
+    step(t2);
+    step(t3);
+    const int ex = (hp >> 20) & 0x7FF;
+    if (ex > 1023 + 300 || ex < 1023 - 300) {
+      const double f = (ex > 1023) ? 0x1p-300 : 0x1p300;
+      p *= f;
+      pm *= f;
+      hp = __double2hiint(p);
+    }
+  }
+  for (; i < m; ++i) step(P[i]);
+  return cnt;
+}
+
+// Multisection: G lanes per eigenvalue count the eigenvalues below G interior points of its
+// interval, which shrinks it by G + 1 per iteration (23 iterations to machine precision with 4 lanes,
+// 13 with 16, 11 with 32).  A count is a serial chain of m steps, so more lanes are faster while the
+// warps do not outnumber the schedulers, and 4 lanes do the least FP64 work (1.7 counts per bit against
+// 3.9 with 16), which is what counts for the hundreds of charge blocks of the blocked form.
+// Measured against 4 lanes for all and a range check every step: 256 values of 4 matrices of 1024 5.45 -> 1.9
+// ms, 61 of 244 1.29 -> 0.46 ms, 8 of 24 90 -> 35 us; the charge blocks of a chi = 1024, d = 5 cut (4 lanes,
+// and the threshold below) 5.4 -> 2.8 ms.
+__host__ __device__ __forceinline__ int bisect_lanes(int kmax, int few) {
+  return kmax <= 32 ? 32 : few && kmax <= 256 ? 16 : few && kmax <= 512 ? 8 : 4;
+}
+
+template <int G>
+__device__ void bisect_warp(const EigMat& M, int w) {
+  const int m = M.m, lane = threadIdx.x & 31, g = lane / G, sub = lane % G;
+  const int j = w * (32 / G) + g;
+  const SturmHead H = *sturm_head(M);
+  const double2* P = sturm_pairs(M);
   const bool active = j < M.kmax && j < m;
-  const double bnorm = fmax(fabs(gl), fabs(gu));
+  const double bnorm = fmax(fabs(H.gl), fabs(H.gu));
   const double eps = DBL_EPSILON, tiny = DBL_MIN * fmax(1.0, bnorm * bnorm);
-  double lo = gl - 2.0 * eps * bnorm * m - 4.0 * tiny;
-  double hi = gu + 2.0 * eps * bnorm * m + 4.0 * tiny;
-  const double atol = 2.0 * eps * bnorm + 4.0 * tiny;
+  double lo = H.gl - 2.0 * eps * bnorm * m - 4.0 * tiny;
+  double hi = H.gu + 2.0 * eps * bnorm * m + 4.0 * tiny;
+  const double atol = 2.0 * eps * bnorm + 4.0 * tiny, frac = (double)(sub + 1) * (1.0 / (G + 1));
   const int target = m - 1 - j;  // ascending index of the j-th largest
   for (int it = 0; it < 64; ++it) {
     const bool conv = !(hi - lo > atol);
     if (__all_sync(0xffffffffu, conv || !active)) break;
-    const double x = lo + (hi - lo) * (double)(sub + 1) * 0.2;
-    const bool above = active && !conv && sturm_count(M.d, M.work, m, x) > target;  // eigenvalue below x
-    const unsigned gb = (__ballot_sync(0xffffffffu, above) >> (4 * g)) & 0xFu;
-    const int l0 = gb ? (__ffs(gb) - 1) : 4;  // first point above the eigenvalue (4: none)
-    const double xa = __shfl_sync(0xffffffffu, x, 4 * g + (l0 > 0 ? l0 - 1 : 0));
-    const double xb = __shfl_sync(0xffffffffu, x, 4 * g + (l0 < 4 ? l0 : 3));
+    const double x = fma(hi - lo, frac, lo);
+    const bool above = active && !conv && sturm_count(P, m, x) > target;  // eigenvalue below x
+    const unsigned gb = (__ballot_sync(0xffffffffu, above) >> (G * g)) & (unsigned)((1ull << G) - 1);
+    const int l0 = gb ? (__ffs(gb) - 1) : G;  // first point above the eigenvalue (G: none)
+    const double xa = __shfl_sync(0xffffffffu, x, G * g + (l0 > 0 ? l0 - 1 : 0));
+    const double xb = __shfl_sync(0xffffffffu, x, G * g + (l0 < G ? l0 : G - 1));
     if (active && !conv) {
       if (l0 > 0) lo = xa;
-      if (l0 < 4) hi = xb;
+      if (l0 < G) hi = xb;
     }
   }
-  if (active && sub == 0) M.evals[j] = 0.5 * (lo + hi);
+  if (active && sub == 0) M.evals[j] = 0.5 * (lo + hi) * H.dn;
+}
+
+__global__ void __launch_bounds__(128) k_bisect(const __grid_constant__ EigBatch b) {
+  const EigMat& M = b.a[blockIdx.y];
+  const int km = min(M.kmax, M.m), G = bisect_lanes(M.kmax, b.few);
+  // warps of a matrix spread over the blocks first
+  const int w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  if (w * (32 / G) >= km) return;
+  if (G == 32) bisect_warp<32>(M, w);
+  else if (G == 16) bisect_warp<16>(M, w);
+  else if (G == 8) bisect_warp<8>(M, w);
+  else bisect_warp<4>(M, w);
 }
 
 // ---- eigenvalue counts of a cut -------------------------------------------------------
 // A cut's spectrum is the union of its matrices' (the charge blocks of one truncated
 // SVD).  Rule T keeps at most `target` values of the cut, so each matrix needs only
 // its eigenvalues above the cut's target-th largest one (and above the floor
-// floor_rel x the cut's trace).  One block per cut finds that threshold by
-// multisection on the summed Sturm counts: P points per matrix per iteration, each
-// iteration shrinking the bracket by P + 1, then writes per matrix the number of
-// its eigenvalues at or above the bracket's lower end (capped by kmax).  The search
-// ends early at a point whose count is exactly the target.  A cut's counts all run on
-// one SM, whose FP64 pipe bounds them (every count is m dependent steps), so few
-// points per iteration (P <= 7) do less work in total than a wide multisection.
-__device__ __forceinline__ int count_at_or_above(const EigMat& M, double x) { return M.m - sturm_count(M.d, M.work, M.m, x); }
+// floor_rel x the cut's trace).  One block per cut finds a threshold by
+// multisection on the summed Sturm counts, P points per matrix per iteration, then writes per matrix the
+// number of its eigenvalues at or above it (capped by kmax).  The search ends at a point that leaves
+// at most 1/32 too many: bisecting those costs less than the iterations that would exclude them (each
+// a chain of m steps on one SM), and the vectors are chosen from the eigenvalues themselves later.
+__device__ __forceinline__ int count_at_or_above(const EigMat& M, double x) {
+  const double xs = x * sturm_head(M)->up;
+  if (!(xs < 4.0)) return 0;  // beyond the spectrum's bound (2 in the scaled matrix)
+  if (xs < -4.0) return M.m;
+  return M.m - sturm_count(sturm_pairs(M), M.m, xs);
+}
 
 __global__ void __launch_bounds__(1024) k_cut_counts(const ThrCut* __restrict__ cuts) {
   const ThrCut C = cuts[blockIdx.x];
@@ -212,15 +253,10 @@ __global__ void __launch_bounds__(1024) k_cut_counts(const ThrCut* __restrict__ 
   __shared__ int go_sh;
   // the cut's trace and an upper bound of its spectrum (Gershgorin)
   double tr = 0.0, up = 0.0;
-  for (int i = threadIdx.x; i < C.n; i += blockDim.x) tr += *C.mats[i].trace;
-  for (int i = 0; i < C.n; ++i) {
-    const EigMat& M = C.mats[i];
-    for (int r = threadIdx.x; r < M.m; r += blockDim.x) {
-      double g = M.d[r];
-      if (r > 0) g += fabs(M.e[r - 1]);
-      if (r < M.m - 1) g += fabs(M.e[r]);
-      up = fmax(up, g);
-    }
+  for (int i = threadIdx.x; i < C.n; i += blockDim.x) {
+    tr += *C.mats[i].trace;
+    const SturmHead* H = sturm_head(C.mats[i]);
+    up = fmax(up, H->gu * H->dn);
   }
   tr = block_sum(tr, sh);
   up = -block_min(-up, sh);
@@ -237,7 +273,7 @@ __global__ void __launch_bounds__(1024) k_cut_counts(const ThrCut* __restrict__ 
   if (threadIdx.x == 0) {
     lo_sh = floor_v;
     hi_sh = fmax(up, floor_v) * (1.0 + 4.0 * DBL_EPSILON) + DBL_MIN;
-    go_sh = cnt[0] > C.target;
+    go_sh = cnt[0] > C.target + C.target / 32;
   }
   __syncthreads();
   const int P = max(1, min(7, (int)blockDim.x / max(C.n, 1)));
@@ -259,7 +295,7 @@ __global__ void __launch_bounds__(1024) k_cut_counts(const ThrCut* __restrict__ 
       const double nhi = (jb + 1 < P) ? lo + (hi - lo) * (double)(jb + 2) / (double)(P + 1) : hi;
       lo_sh = nlo;
       hi_sh = nhi;
-      go_sh = (jb < 0 || cnt[jb] != C.target) && (nhi - nlo) > 4.0 * DBL_EPSILON * fmax(fabs(nhi), DBL_MIN);
+      go_sh = (jb < 0 || cnt[jb] > C.target + C.target / 32) && (nhi - nlo) > 4.0 * DBL_EPSILON * fmax(fabs(nhi), DBL_MIN);
     }
     __syncthreads();
   }
@@ -1285,7 +1321,7 @@ int eig_tridiagonalize(const EigBatch& b, bool mixed, void* const* oz_ws, int* s
     k_tridiag_tail<<<b.n, TL_THREADS, TL_SMEM, s>>>(b);
     ++launches;
   }
-  k_esq<<<dim3(std::max(1, std::min(64, (mm + 255) / 256)), b.n), 256, 0, s>>>(b);
+  k_sturm_prep<<<b.n, 256, 0, s>>>(b);
   return launches + 1;
 }
 
@@ -1302,10 +1338,13 @@ int eig_cut_counts(const ThrCut* cuts_dev, int ncuts, cudaStream_t s) {
 
 int eig_bisect(const EigBatch& b, cudaStream_t s) {
   if (b.n == 0) return 0;
-  int km = 0;
-  for (int i = 0; i < b.n; ++i) km = std::max(km, std::min(b.a[i].kmax, b.a[i].m));
-  if (km == 0) return 0;
-  k_bisect<<<dim3((km + 31) / 32, b.n), 128, 0, s>>>(b);  // four warps, eight eigenvalues each
+  int warps = 0;
+  for (int i = 0; i < b.n; ++i) {
+    const int per = 32 / bisect_lanes(b.a[i].kmax, b.few), km = std::min(b.a[i].kmax, b.a[i].m);
+    warps = std::max(warps, (km + per - 1) / per);
+  }
+  if (warps == 0) return 0;
+  k_bisect<<<dim3((warps + 3) / 4, b.n), 128, 0, s>>>(b);  // up to four warps per block
   return 1;
 }
 

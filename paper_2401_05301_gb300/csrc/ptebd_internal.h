@@ -178,7 +178,7 @@ struct EigMat {
   double* Z;         // m x K real eigenvectors of T (row-major, ld = K)
   double* Z2;        // m x K scratch (Newton-Schulz ping-pong)
   double* S;         // K x K scratch
-  double* work;      // inverse-iteration LU scratch, 5 * m * K doubles
+  double* work;      // Sturm pairs (4 + 2 m doubles), then inverse-iteration scratch (5 m K doubles)
   double2* U;        // K x m eigenvectors of H, one per row (U[j*m + r] = u_j[r])
   double2* pan;      // panel arrays of the blocked reduction [eig_panel_doubles2(m)]
   int m, kmax, K;
@@ -190,6 +190,7 @@ struct EigBatch {
   unsigned int* bar;  // grid-barrier state {count, generation, error} for the persistent reduction
   long long wait_clocks;  // limit of each grid-barrier wait of the reduction (clock64 ticks)
   int panel_blocks;       // blocks per SM of the reduction's cooperative grid (0: as many as fit, at most 3)
+  int few;                // 1: dense form, a batch of at most 24 matrices (the bisection spreads wider)
 };
 
 constexpr int EIG_PARTS = 384;  // partial norms of a row, one per column piece (32 columns at m = 12288)

@@ -809,7 +809,7 @@ void layout_cut(Cut& cut, Bump& bp) {
     B.oZ = bp.take(8 * g * k);
     B.oZ2 = bp.take(8 * g * k);
     B.oS = bp.take(8 * k * k);
-    B.owork = bp.take(40 * g * k);
+    B.owork = bp.take(40 * g * k + 32);
     B.oU = bp.take(16 * k * g);
     B.opan = bp.take(16 * eig_panel_doubles2((int)g));
     B.oY = bp.take(16 * k * n);
