@@ -211,8 +211,11 @@ __device__ __forceinline__ double2 job_elem(const OzPackJob& J, int r, int k) {
 }
 
 __device__ __forceinline__ int find_job(const OzPackBatch& pb, int blk) {
-  int j = 0;
-  while (j + 1 < pb.njob && blk >= pb.block_start[j + 1]) ++j;
+  int j = 0, hi = pb.njob - 1;
+  while (j < hi) {
+    const int mid = (j + hi + 1) >> 1;
+    if (pb.block_start[mid] <= blk) j = mid; else hi = mid - 1;
+  }
   return j;
 }
 
@@ -400,7 +403,10 @@ __global__ void __launch_bounds__(OZ_NT, 1) k_oz_gemm(const __grid_constant__ Oz
 
   const int tile = blockIdx.x;
   int pi = 0;
-  while (pi + 1 < gb.nprob && tile >= gb.tile_start[pi + 1]) ++pi;
+  for (int hi = gb.nprob - 1; pi < hi;) {
+    const int mid = (pi + hi + 1) >> 1;
+    if (gb.tile_start[mid] <= tile) pi = mid; else hi = mid - 1;
+  }
   const OzTile& P = gb.p[pi];
   int mt, nt;
   tile_of(P, tile - gb.tile_start[pi], mt, nt);
@@ -646,13 +652,31 @@ Geo geometry(int M, int N, int K, bool gram) {
 
 }  // namespace
 
-static_assert(sizeof(OzGemmBatch) < 4000, "kernel parameter block too large");
-static_assert(sizeof(OzPackBatch) < 4000, "kernel parameter block too large");
+static_assert(sizeof(OzGemmBatch) < 32000, "kernel parameter block too large (32 KB on sm_70 and later)");
+static_assert(sizeof(OzPackBatch) < 32000, "kernel parameter block too large");
 static_assert(bf16_idesc(128, 64) == ((1u << 4) | (1u << 7) | (1u << 10) | (8u << 17) | (8u << 24)), "idesc");
 
 size_t oz_workspace_bytes(int M, int N, int K, bool gram) {
   if (M <= 0 || N <= 0 || K <= 0) return 0;
   return geometry(M, N, K, gram).total;
+}
+
+int oz_gemm_pooled(std::vector<OzProb>& probs, void* pool, size_t bytes, int* status, cudaStream_t s) {
+  int launches = 0;
+  std::vector<OzProb> group;
+  size_t used = 0;
+  for (OzProb& q : probs) {
+    const size_t need = (oz_workspace_bytes(q.M, q.N, q.K, q.gram != 0) + 255) & ~size_t(255);
+    if (group.size() == (size_t)OZ_MAXP || used + need > bytes) {
+      launches += oz_gemm_launch(group, status, s);
+      group.clear();
+      used = 0;
+    }
+    q.ws = static_cast<char*>(pool) + used;
+    used += need;
+    group.push_back(q);
+  }
+  return launches + oz_gemm_launch(group, status, s);
 }
 
 int oz_gemm_launch(const std::vector<OzProb>& probs, int* status, cudaStream_t s) {

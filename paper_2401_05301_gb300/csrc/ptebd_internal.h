@@ -99,7 +99,7 @@ struct OzProb {
   double* Creal;  // if set, the real part of the result goes here (ldc in doubles) instead of C
   void* ws;  // oz_workspace_bytes(M, N, K, gram) bytes, 256-byte aligned, owned by the caller
 };
-constexpr int OZ_MAXP = 16;
+constexpr int OZ_MAXP = 64;  // problems per launch: the blocked form has hundreds of small products at a time
 struct OzPackJob {
   const double2* X;
   long long rs, ks;
@@ -138,6 +138,9 @@ struct OzGemmBatch {
 };
 size_t oz_workspace_bytes(int M, int N, int K, bool gram);
 int oz_gemm_launch(const std::vector<OzProb>& probs, int* status, cudaStream_t s);
+// The same with the digit workspaces taken from one pool (bytes >= the largest problem's need): as many
+// problems share a launch as the pool holds, at most OZ_MAXP.
+int oz_gemm_pooled(std::vector<OzProb>& probs, void* pool, size_t bytes, int* status, cudaStream_t s);
 
 class Gemm {
  public:

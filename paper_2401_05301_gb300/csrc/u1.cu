@@ -48,10 +48,12 @@ struct U1Slot {
 
 struct U1Work {
   std::vector<U1Slot> slots;
-  // digit workspaces of the exact-digit engine, one per problem of a launch: OZ_MAXP for
-  // the block products (sized for the largest), EIG_MAXP for the eigen-solver's products
-  std::vector<void*> ring, ering;
-  size_t ring_bytes = 0, ering_bytes = 0;
+  // digit workspaces of the exact-digit engine: one pool for the block products (POOL times the
+  // largest one's), and one workspace per matrix of a batch for the eigen-solver's products
+  void* pool = nullptr;
+  size_t pool_bytes = 0;
+  std::vector<void*> ering;
+  size_t ering_bytes = 0;
   char* h_stage[2] = {nullptr, nullptr};  // pinned staging of descriptors, by chunk parity
   char* d_stage[2] = {nullptr, nullptr};
   size_t stage_cap[2] = {0, 0};
@@ -68,7 +70,7 @@ struct U1Work {
 
 namespace {
 
-constexpr int RING = OZ_MAXP;    // problems of one exact-digit launch
+constexpr int POOL = 16;         // the digit pool holds 16 of the largest products, or up to OZ_MAXP small ones
 constexpr int ERING = EIG_MAXP;  // matrices of one eigen-solver batch
 constexpr int MV_TILE = 4096;   // elements per block of the move kernel
 constexpr int TR_THREADS = 1024;
@@ -523,7 +525,34 @@ int grow_ring(tebd_ctx* c, std::vector<void*>& ring, size_t& have, int count, si
   return TEBD_OK;
 }
 
-int ensure_ring(tebd_ctx* c, size_t bytes) { return grow_ring(c, c->u1w->ring, c->u1w->ring_bytes, RING, bytes); }
+// A pool for products whose largest needs `bytes`.
+int ensure_pool(tebd_ctx* c, size_t bytes) {
+  U1Work& w = *c->u1w;
+  if (w.pool_bytes >= POOL * bytes) return TEBD_OK;
+  if (w.pool) {
+    if (cudaStreamSynchronize(c->stream) != cudaSuccess) return fail_cuda(c);
+    cudaFree(w.pool);
+  }
+  w.pool = nullptr;
+  w.pool_bytes = 0;
+  const size_t want = POOL * align256(bytes + bytes / 4);
+  if (cudaMalloc(&w.pool, want) != cudaSuccess) {
+    cudaGetLastError();
+    return TEBD_ERR_OOM;
+  }
+  w.pool_bytes = want;
+  return TEBD_OK;
+}
+
+// The products on the exact-digit engine with pooled workspaces.
+int run_oz(tebd_ctx* c, std::vector<OzProb>& oz) {
+  size_t need = 0;
+  for (const OzProb& q : oz) need = std::max(need, oz_workspace_bytes(q.M, q.N, q.K, q.gram != 0));
+  if (need == 0) return TEBD_OK;
+  if (int r = ensure_pool(c, need)) return r;
+  c->launches += oz_gemm_pooled(oz, c->u1w->pool, c->u1w->pool_bytes, c->d_status, c->stream);
+  return check_launch(c);
+}
 int ensure_ering(tebd_ctx* c, size_t bytes) { return grow_ring(c, c->u1w->ering, c->u1w->ering_bytes, ERING, bytes); }
 
 int ensure_back(tebd_ctx* c, size_t n) {
@@ -673,8 +702,6 @@ struct Prod {
   int accumulate;
 };
 
-size_t oz_bytes(const Prod& p) { return oz_workspace_bytes(p.M, p.N, p.K, false); }
-
 void check_prod(Checker& ck, const char* what, const Prod& p, const Span& sa, const Span& sb, const Span& sc) {
   ck.need(fits(p.A, 16, p.M, p.K, p.lda, 1, sa), what);
   ck.need(p.opB == OP_C ? fits(p.B, 16, p.N, p.K, p.ldb, 1, sb) : fits(p.B, 16, p.K, p.N, p.ldb, 1, sb), what);
@@ -685,9 +712,6 @@ void check_prod(Checker& ck, const char* what, const Prod& p, const Span& sa, co
 int run_prods(tebd_ctx* c, const std::vector<Prod>& ps, int engine) {
   if (ps.empty()) return TEBD_OK;
   if (engine == 2) {
-    size_t need = 0;
-    for (const Prod& p : ps) need = std::max(need, oz_bytes(p));
-    if (int r = ensure_ring(c, need)) return r;
     std::vector<OzProb> oz;
     for (const Prod& p : ps) {
       OzProb q{};
@@ -695,11 +719,9 @@ int run_prods(tebd_ctx* c, const std::vector<Prod>& ps, int engine) {
       q.b = p.opB == OP_C ? OzOperand{p.B, p.ldb, 1, nullptr, 1, 1} : OzOperand{p.B, 1, p.ldb, nullptr, 1, 0};
       q.M = p.M; q.N = p.N; q.K = p.K; q.C = p.C; q.ldc = p.ldc; q.alpha = p.alpha; q.beta = p.accumulate;
       q.row_div = q.col_div = 1;
-      q.ws = c->u1w->ring[oz.size() % OZ_MAXP];
       oz.push_back(q);
     }
-    c->launches += oz_gemm_launch(oz, c->d_status, c->stream);
-    return check_launch(c);
+    return run_oz(c, oz);
   }
   // (an accumulating product is not eligible for the 3xTF32 kernel: Gemm::launch then keeps FP64)
   Gemm gn(true, OP_N, OP_N), gc(true, OP_N, OP_C);
@@ -845,14 +867,12 @@ int decompose(tebd_ctx* c, std::vector<Cut*>& cuts, std::vector<char*>& bases, s
     double w = 0.0;
     Gemm g(true, OP_N, OP_C), gr(true, OP_C, OP_N);
     std::vector<OzProb> oz;
-    size_t need = 0;
     for (size_t t = 0; t < nc; ++t)
       for (CutBlk& B : cuts[t]->blk) {
         char* a = bases[t];
         if (B.right()) {  // H[i][j] = sum_r lam_r^2 conj(P[r][i]) P[r][j], n x n
           w += 4.0 * (double)B.n * B.n * B.b;
           if (mixed) {
-            need = std::max(need, oz_workspace_bytes(B.n, B.n, B.b, true));
             OzProb q{};
             q.a = OzOperand{at<double2>(a, B.oP), 1, B.n, at<double>(a, B.oLam), 1, 1};
             q.M = q.N = B.n; q.K = B.b; q.C = at<double2>(a, B.oH); q.ldc = B.n; q.alpha = 1.0;
@@ -869,7 +889,6 @@ int decompose(tebd_ctx* c, std::vector<Cut*>& cuts, std::vector<char*>& bases, s
         }
         w += 4.0 * (double)B.b * B.b * B.n;
         if (mixed) {
-          need = std::max(need, oz_workspace_bytes(B.b, B.b, B.n, true));
           OzProb q{};
           q.a = OzOperand{at<double2>(a, B.oP), B.n, 1, nullptr, 1, 0};
           q.M = q.N = B.b; q.K = B.n; q.C = at<double2>(a, B.oH); q.ldc = B.b; q.alpha = 1.0;
@@ -886,9 +905,7 @@ int decompose(tebd_ctx* c, std::vector<Cut*>& cuts, std::vector<char*>& bases, s
       }
     ProfScope ps(c, TEBD_PROF_GRAM, w);
     if (mixed) {
-      if (int r = ensure_ring(c, need)) return r;
-      for (size_t j = 0; j < oz.size(); ++j) oz[j].ws = c->u1w->ring[j % OZ_MAXP];
-      c->launches += oz_gemm_launch(oz, c->d_status, c->stream);
+      if (int r = run_oz(c, oz)) return r;
     } else {
       c->launches += g.launch(c->stream);
       c->launches += gr.launch(c->stream);
@@ -1120,7 +1137,6 @@ int decompose(tebd_ctx* c, std::vector<Cut*>& cuts, std::vector<char*>& bases, s
     std::vector<OzProb> oz;
     std::vector<RightRows> rr;
     int rmaxK = 0;
-    size_t need = 0;
     for (size_t t = 0; t < nc; ++t)
       for (CutBlk& B : cuts[t]->blk) {
         if (B.K == 0) continue;
@@ -1130,7 +1146,6 @@ int decompose(tebd_ctx* c, std::vector<Cut*>& cuts, std::vector<char*>& bases, s
           rr.push_back(RightRows{at<double2>(a, B.oU), at<double2>(a, B.oY), at<double2>(a, B.oOut), B.K, B.n, B.b});
           rmaxK = std::max(rmaxK, B.K);
           if (mixed) {
-            need = std::max(need, oz_workspace_bytes(B.b, B.K, B.n, false));
             OzProb q{};
             q.a = OzOperand{at<double2>(a, B.oP), B.n, 1, nullptr, 1, 0};
             q.b = OzOperand{at<double2>(a, B.oY), B.n, 1, nullptr, 1, 1};
@@ -1146,7 +1161,6 @@ int decompose(tebd_ctx* c, std::vector<Cut*>& cuts, std::vector<char*>& bases, s
           continue;
         }
         if (mixed) {
-          need = std::max(need, oz_workspace_bytes(B.K, B.n, B.b, false));
           OzProb q{};
           q.a = OzOperand{at<double2>(a, B.oU), B.b, 1, at<double>(a, B.oLam), 1, 1};
           q.b = OzOperand{at<double2>(a, B.oP), 1, B.n, nullptr, 1, 0};
@@ -1173,9 +1187,7 @@ int decompose(tebd_ctx* c, std::vector<Cut*>& cuts, std::vector<char*>& bases, s
       }
     }
     if (mixed) {
-      if (int r = ensure_ring(c, need)) return r;
-      for (size_t j = 0; j < oz.size(); ++j) oz[j].ws = c->u1w->ring[j % OZ_MAXP];
-      c->launches += oz_gemm_launch(oz, c->d_status, c->stream);
+      if (int r = run_oz(c, oz)) return r;
     } else {
       c->launches += g.launch(c->stream);
       c->launches += gt.launch(c->stream);
@@ -1926,11 +1938,7 @@ void prod_with_M(tebd_ctx* c, Gemm& gN, Gemm& gC, std::vector<OzProb>& oz, const
 int run_M_prods(tebd_ctx* c, Gemm& gN, Gemm& gC, std::vector<OzProb>& oz, double w) {
   ProfScope ps(c, TEBD_PROF_PROJECT, w);
   if (c->precision >= 1) {
-    size_t need = 0;
-    for (const OzProb& q : oz) need = std::max(need, oz_workspace_bytes(q.M, q.N, q.K, false));
-    if (int r = ensure_ring(c, need)) return r;
-    for (size_t j = 0; j < oz.size(); ++j) oz[j].ws = c->u1w->ring[j % OZ_MAXP];
-    c->launches += oz_gemm_launch(oz, c->d_status, c->stream);
+    if (int r = run_oz(c, oz)) return r;
   } else {
     c->launches += gN.launch(c->stream);
     c->launches += gC.launch(c->stream);
@@ -2173,7 +2181,6 @@ int correlators_body(tebd_ctx* h, double2* out) {
   const bool tc = h->precision >= 1;
   Gemm gx(true, OP_C, OP_N), gy(true, OP_N, OP_C);
   std::vector<OzProb> oz;
-  size_t need = 0;
   std::vector<TraceBlk> tb;
   std::vector<TraceBond> bonds;
   for (size_t i = 0; i < vb.size(); ++i) {
@@ -2195,7 +2202,6 @@ int correlators_body(tebd_ctx* h, double2* out) {
       qy.b = OzOperand{at<double2>(a, X.oU), X.Ky, 1, nullptr, 1, 1};
       qy.M = X.nv; qy.N = X.nu; qy.K = X.Ky; qy.C = at<double2>(a, X.oY); qy.ldc = X.nu; qy.alpha = 1.0;
       qy.row_div = qy.col_div = 1;
-      need = std::max({need, oz_workspace_bytes(qx.M, qx.N, qx.K, false), oz_workspace_bytes(qy.M, qy.N, qy.K, false)});
       oz.push_back(qx);
       oz.push_back(qy);
     } else {
@@ -2211,9 +2217,7 @@ int correlators_body(tebd_ctx* h, double2* out) {
     bonds.back().b1 = (int)tb.size();
   }
   if (tc) {
-    if (int r = ensure_ring(h, need)) return r;
-    for (size_t j = 0; j < oz.size(); ++j) oz[j].ws = h->u1w->ring[j % OZ_MAXP];
-    h->launches += oz_gemm_launch(oz, h->d_status, h->stream);
+    if (int r = run_oz(h, oz)) return r;
   } else {
     h->launches += gx.launch(h->stream);
     h->launches += gy.launch(h->stream);
@@ -2271,7 +2275,7 @@ int u1_build_gate_blocks(tebd_ctx* c, const std::vector<std::complex<double>>& G
 
 size_t u1_workspace_bytes(const tebd_ctx* c) {
   if (!c->u1w) return 0;
-  size_t b = c->u1w->ring_bytes * c->u1w->ring.size() + c->u1w->ering_bytes * c->u1w->ering.size() +
+  size_t b = c->u1w->pool_bytes + c->u1w->ering_bytes * c->u1w->ering.size() +
              c->u1w->stage_cap[0] + c->u1w->stage_cap[1];
   for (const U1Slot& s : c->u1w->slots) b += s.a1.cap + s.a2.cap;
   b += c->u1w->meas.cap;
@@ -2285,7 +2289,7 @@ void u1_release(tebd_ctx* c) {
     if (s.a1.base) cudaFree(s.a1.base);
     if (s.a2.base) cudaFree(s.a2.base);
   }
-  for (void* p : w.ring) cudaFree(p);
+  if (w.pool) cudaFree(w.pool);
   for (void* p : w.ering) cudaFree(p);
   if (w.meas.base) cudaFree(w.meas.base);
   for (int p = 0; p < 2; ++p) {
