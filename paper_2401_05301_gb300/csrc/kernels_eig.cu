@@ -624,9 +624,11 @@ __global__ void __launch_bounds__(4 * BT) k_bt_T(const __grid_constant__ EigBatc
 // reductions, magnitudes are compared as integers, and the reflector's scalars (norm, divisions)
 // are one warp's work beside the product, which therefore runs on the unnormalised row.
 // Against three barriers per column with a reflector per block, shuffled row sums and 32 x 256 slabs,
-// the reduction of 4 matrices of 1024 (with its trailing updates and tail) takes 33 instead of 59 ms,
-// of 4 matrices of 244 4.1 instead of 10.8 ms, of the 94 charge blocks (up to 600) of a chi = 1024, d = 5
-// cut of 7 triples 21 instead of 38 ms.
+// the reduction of 4 matrices of 1024 (with its trailing updates and tail) takes 26 instead of 59 ms,
+// of 4 matrices of 244 3.5 instead of 10.8 ms, of the 94 charge blocks (up to 600) of a chi = 1024, d = 5
+// cut of 7 triples 16.5 instead of 38 ms.  A column of 4 x 244 spends 9k clocks in phase A, 12k in phase B and
+// 8k in the barriers.
+
 constexpr int TD_THREADS = 256;
 constexpr int TD_WARPS = TD_THREADS / 32;
 constexpr int TD_NB = 32;      // columns per panel of the blocked reduction
@@ -654,7 +656,9 @@ __host__ __device__ __forceinline__ int tail_start(int m) {
 // at most `limit` clocks (2e9, ~1 s, unless the handle's "wait_limit_clocks"
 // says otherwise); on timeout it records the failure in st[2] and returns
 // false so every block can leave.  The count starts at 0 per launch.
-__device__ bool grid_sync(unsigned int* st, unsigned int& target, long long limit) {
+// `beside` is run by warp 1 while thread 0 waits (it must not touch what other blocks write).
+template <class F>
+__device__ bool grid_sync(unsigned int* st, unsigned int& target, long long limit, F beside) {
   __shared__ int ok_sh;
   __syncthreads();
   target += gridDim.x;
@@ -673,6 +677,8 @@ __device__ bool grid_sync(unsigned int* st, unsigned int& target, long long limi
     }
     __threadfence();
     ok_sh = ok && (*verr == 0);
+  } else if ((threadIdx.x >> 5) == 1) {
+    beside();
   }
   __syncthreads();
   return ok_sh != 0;
@@ -683,14 +689,14 @@ __device__ bool grid_sync(unsigned int* st, unsigned int& target, long long limi
 //   operand of the trailing update); the partial dots of the panel corrections (TD_DOTS x 2 NB); the
 //   partial sums of the Hermitian product, per strip of 32 columns from row blocks (hc) and from
 //   tiles to its right (hr); the partials of u^+ A u, one per tile; the column's scalars.
-// The piece sizes follow the trailing size n only, never the batch: the sums keep their order.
-__host__ __device__ __forceinline__ int td_rows(int n) { return n <= 256 ? 8 : n <= 2048 ? 16 : 32; }   // rows per tile
-__host__ __device__ __forceinline__ int td_cols(int n) { return n <= 256 ? 8 : n <= 512 ? 16 : 32; }    // columns per phase-B piece
-__host__ __device__ __forceinline__ int td_dot(int n) { return n <= 256 ? 16 : n <= 512 ? 32 : 64; }    // rows per partial dot
-constexpr int TD_DOTS = 200;  // partial dots: ceil(12288 / 64) = 192, and 17 for the smaller pieces
+// The piece sizes (as shifts) follow the trailing size n only, never the batch: the sums keep their order.
+__host__ __device__ __forceinline__ int td_rows(int n) { return n <= 256 ? 3 : n <= 2048 ? 4 : 5; }   // rows per tile
+__host__ __device__ __forceinline__ int td_cols(int n) { return n <= 256 ? 3 : n <= 1024 ? 4 : 5; }   // columns per phase-B piece
+__host__ __device__ __forceinline__ int td_dot(int n) { return n <= 256 ? 4 : n <= 512 ? 5 : 6; }     // rows per partial dot
+constexpr int TD_DOTS = 200;  // partial dots: at most ceil(12288 / 64) = 192
 // Strips and row blocks that a trailing set of n can touch (its start is not aligned to them).
 __host__ __device__ __forceinline__ size_t td_strips(int n) { return (size_t)(n + 31) / 32 + 1; }
-__host__ __device__ __forceinline__ size_t td_blocks(int n) { return (size_t)n / td_rows(n) + 2; }
+__host__ __device__ __forceinline__ size_t td_blocks(int n) { return (size_t)(n >> td_rows(n)) + 2; }
 __host__ __device__ __forceinline__ size_t td_tiles(int n) { return td_strips(n) * td_blocks(n); }
 __host__ __device__ inline size_t td_max3(size_t a, size_t b, size_t c) { return a > b ? (a > c ? a : c) : (b > c ? b : c); }
 __host__ __device__ inline size_t td_hc_tiles(int m) {  // the largest of the three piece sizes' needs
@@ -699,37 +705,33 @@ __host__ __device__ inline size_t td_hc_tiles(int m) {  // the largest of the th
 __host__ __device__ __forceinline__ size_t td_hr_tiles(int m) { return td_strips(m) * td_strips(m); }
 __host__ __device__ size_t td_panel_size(int m) {
   return (size_t)m * 4 * TD_NB + (size_t)TD_DOTS * 2 * TD_NB + 32 * (td_hc_tiles(m) + td_hr_tiles(m)) +
-         (td_hc_tiles(m) + 1) / 2 + 8;
+         (td_hc_tiles(m) + 1) / 2 + 8;  // the host lays td_hr, td_q and td_sc out the same way
 }
 __device__ __forceinline__ double2* pan_vw(const EigMat& M) { return M.pan; }
 __device__ __forceinline__ double2* pan_wv(const EigMat& M) { return M.pan + (size_t)M.m * 2 * TD_NB; }
 __device__ __forceinline__ double2* pan_xy(const EigMat& M) { return M.pan + (size_t)M.m * 4 * TD_NB; }
 __device__ __forceinline__ double2* pan_hc(const EigMat& M) { return pan_xy(M) + (size_t)TD_DOTS * 2 * TD_NB; }
-__device__ __forceinline__ double2* pan_hr(const EigMat& M) { return pan_hc(M) + 32 * td_hc_tiles(M.m); }
-__device__ __forceinline__ double* pan_q(const EigMat& M) {
-  return reinterpret_cast<double*>(pan_hr(M) + 32 * td_hr_tiles(M.m));
-}
-__device__ __forceinline__ double2* pan_scal(const EigMat& M) {  // [0] sc, [1] (A(k+1, k+1), 0)
-  return pan_hr(M) + 32 * td_hr_tiles(M.m) + (td_hc_tiles(M.m) + 1) / 2;
-}
+__device__ __forceinline__ double2* pan_hr(const EigMat& M) { return M.td_hr; }
+__device__ __forceinline__ double* pan_q(const EigMat& M) { return M.td_q; }
+__device__ __forceinline__ double2* pan_scal(const EigMat& M) { return M.td_sc; }  // [0] sc, [1] (A(k+1, k+1), 0)
 
 // What a column's pieces are, from m and k alone.
 struct TdGeo {
   int m, k, n;          // trailing set: indices k+1 .. m-1, n of them
-  int rows, cols, dot;  // piece sizes
+  int rows, cols, dot;  // piece sizes (shifts)
   int s0, ns;           // first strip, strips
   int b0, nb;           // first row block, row blocks
   int g0, ng;           // first phase-B piece, pieces
   int nd;               // partial dots
   __device__ TdGeo(int m_, int k_) : m(m_), k(k_), n(m_ - k_ - 1) {
     rows = td_rows(n); cols = td_cols(n); dot = td_dot(n);
-    s0 = (k + 1) / 32; ns = (m - 1) / 32 - s0 + 1;
-    b0 = (k + 1) / rows; nb = (m - 1) / rows - b0 + 1;
-    g0 = (k + 1) / cols; ng = (m - 1) / cols - g0 + 1;
-    nd = (n + dot - 1) / dot;
+    s0 = (k + 1) >> 5; ns = ((m - 1) >> 5) - s0 + 1;
+    b0 = (k + 1) >> rows; nb = ((m - 1) >> rows) - b0 + 1;
+    g0 = (k + 1) >> cols; ng = ((m - 1) >> cols) - g0 + 1;
+    nd = (n + (1 << dot) - 1) >> dot;
   }
   // tiles: row block b of strip S meets the strips S .. end; counted as if the last strip were full
-  __device__ int per() const { return 32 / rows; }
+  __device__ int per() const { return 32 >> rows; }
   __device__ int first_blocks() const { return (s0 + 1) * per() - b0; }  // row blocks of the first strip
   __device__ int tiles() const { return first_blocks() * ns + per() * (ns * (ns - 1) / 2); }
   __device__ int items_a(int j) const { return 1 + (j > 0 ? 2 * nd : 0) + tiles(); }
@@ -743,7 +745,7 @@ struct TdGeo {
     }
     t -= f;
     const int last = per() * (ns * (ns - 1) / 2) - 1 - t;  // counted from the end: strips of 1, 2, ... tiles per row block
-    int D = (int)((sqrtf(8.0f * (float)(last / per()) + 1.0f) + 1.0f) * 0.5f);
+    int D = (int)((sqrtf(8.0f * (float)(last >> (5 - rows)) + 1.0f) + 1.0f) * 0.5f);
     while (per() * (D * (D - 1) / 2) > last) --D;
     while (per() * (D * (D + 1) / 2) <= last) ++D;
     const int rem = last - per() * (D * (D - 1) / 2);  // within the strip that has D strips from itself on
@@ -783,6 +785,9 @@ __device__ __forceinline__ void put_norm(const EigMat& M, int g, double2 x, bool
 __device__ void td_scalars(const EigMat& M, int k) {
   const int m = M.m, lane = threadIdx.x & 31;
   const TdGeo P(m, k - 1);  // the pieces that wrote the partials of row k
+  const double2* row = M.H + (size_t)k * m;
+  const double2 x0 = row[k + 1];
+  const double dk = row[k].x, a00 = M.H[(size_t)(k + 1) * m + k + 1].x;
   int bmax = -4096, emax = 0;
   for (int g = lane; g < P.ng; g += 32) {
     const long long t = __double_as_longlong(M.part[g].y);
@@ -800,30 +805,26 @@ __device__ void td_scalars(const EigMat& M, int k) {
     s += (d == 0) ? t.x : (d < -500 ? 0.0 : t.x * pow2i(2 * d));
   }
   const double xnorm2 = warp_sum(s);
+  const bool flush = emax < 1023 - REFL_FLUSH_EXP;  // every entry below 2^-900
+  const double f = (E == 0) ? 1.0 : pow2i(max(-1022, min(1022, -E)));
+  const double ar = x0.x * f, ai = -x0.y * f;
+  double beta = x0.x;
+  double2 tau = make_double2(0.0, 0.0), sc = tau;
+  if (!flush && !(xnorm2 == 0.0 && ai == 0.0)) {
+    const double bs = -copysign(sqrt(ar * ar + ai * ai + xnorm2), ar), zr = ar - bs;
+    // lane 0: 1 / beta, lane 1: f / |alpha - beta|^2
+    const double r = ((lane & 1) ? f : 1.0) / ((lane & 1) ? fma(zr, zr, ai * ai) : bs);
+    const double inv = __shfl_sync(0xffffffffu, r, 0), iden = __shfl_sync(0xffffffffu, r, 1);
+    tau = make_double2(-zr * inv, -ai * inv);
+    sc = make_double2(zr * iden, -ai * iden);
+    beta = (E == 0) ? bs : bs * pow2i(max(-1022, min(1022, E)));
+  }
   if (lane == 0) {
-    const double2* row = M.H + (size_t)k * m;
-    const double2 x0 = row[k + 1];
-    const bool flush = emax < 1023 - REFL_FLUSH_EXP;  // every entry below 2^-900
-    const double f = (E == 0) ? 1.0 : pow2i(max(-1022, min(1022, -E)));
-    const double ar = x0.x * f, ai = -x0.y * f;
-    double beta;
-    double2 tau, sc;
-    if (flush || (xnorm2 == 0.0 && ai == 0.0)) {
-      beta = x0.x;
-      tau = make_double2(0.0, 0.0);
-      sc = make_double2(0.0, 0.0);
-    } else {
-      const double bs = -copysign(sqrt(ar * ar + ai * ai + xnorm2), ar);
-      const double zr = ar - bs, inv = 1.0 / bs, iden = f / (zr * zr + ai * ai);
-      tau = make_double2(-zr * inv, -ai * inv);
-      sc = make_double2(zr * iden, -ai * iden);
-      beta = (E == 0) ? bs : bs * pow2i(max(-1022, min(1022, E)));
-    }
-    M.d[k] = row[k].x;
+    M.d[k] = dk;
     M.e[k] = beta;
     M.tau[k] = tau;
     pan_scal(M)[0] = sc;
-    pan_scal(M)[1] = make_double2(M.H[(size_t)(k + 1) * m + k + 1].x, 0.0);
+    pan_scal(M)[1] = make_double2(a00, 0.0);
   }
 }
 
@@ -835,13 +836,13 @@ __device__ __forceinline__ double2 td_u(const EigMat& M, int k, int r) {
 // One tile of hraw = A u (one warp): row block b against strip T.  The lanes hold the strip's
 // columns: each row of A is read once, gives its term of the column sums conj(A[r][c]) u_r from
 // registers and, off the diagonal, the row sums A[r][c] u_c through a transposed read of shared
-// memory (st: 16 x 33, us: 32).  Diagonal tiles need only the column sums.
+// memory (st: 16 x 33, us: 64).  Diagonal tiles need only the column sums.
 template <int SUB>
 __device__ void td_tile(const EigMat& M, const TdGeo& G, int t, double2* st, double2* us) {
   const int lane = threadIdx.x & 31, m = G.m, k = G.k;
   int b, T;
   G.tile(t, b, T);
-  const int r0 = (G.b0 + b) * G.rows;
+  const int r0 = (G.b0 + b) << G.rows;
   if (r0 >= m) {  // the last strip's missing row blocks
     if (lane == 0) pan_q(M)[t] = 0.0;
     return;
@@ -849,14 +850,15 @@ __device__ void td_tile(const EigMat& M, const TdGeo& G, int t, double2* st, dou
   const int S = r0 / 32 - G.s0;
   const bool diag = (S == T);
   const int c = 32 * (G.s0 + T) + lane;
-  const double2* x = M.H + (size_t)k * m;
-  const double2 uc = td_u(M, k, c);
-  if (!diag) us[lane] = uc;
+  const double2 uc = td_u(M, k, c), ur = td_u(M, k, r0 + lane);  // (lanes beyond the row block: not used)
+  us[lane] = uc;
+  us[32 + lane] = ur;
   double2 acc = make_double2(0.0, 0.0);
   double2* hr = pan_hr(M) + ((size_t)S * G.ns + T) * 32;
-  for (int sub = r0; sub < r0 + G.rows; sub += SUB) {
+  const bool okc = c < m && c > k;
+  __syncwarp();
+  for (int sub = r0; sub < r0 + (1 << G.rows); sub += SUB) {
     if (sub + SUB <= k + 1 || sub >= m) continue;
-    const bool okc = c < m && c > k;
 #pragma unroll
     for (int h = 0; h < SUB; h += 8) {
       double2 a[8];
@@ -867,9 +869,8 @@ __device__ void td_tile(const EigMat& M, const TdGeo& G, int t, double2* st, dou
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int r = sub + h + u;
-        if (r > k + 1 && r < m) acc = cfma_conj(a[u], cconj(x[r]), acc);
         if (!diag) st[(h + u) * 33 + lane] = a[u];
+        if (sub + h + u > k + 1) acc = cfma_conj(a[u], us[32 + sub - r0 + h + u], acc);  // (rows beyond m hold zeros)
       }
     }
     if (!diag) {
@@ -899,7 +900,7 @@ __device__ void td_tile(const EigMat& M, const TdGeo& G, int t, double2* st, dou
 __device__ void td_dots(const EigMat& M, const TdGeo& G, int j, int p, int which) {
   const int lane = threadIdx.x & 31;
   if (lane >= j) return;
-  const int r0 = max(G.k + 2, G.k + 1 + p * G.dot), r1 = min(G.m, G.k + 1 + (p + 1) * G.dot);
+  const int r0 = max(G.k + 2, G.k + 1 + (p << G.dot)), r1 = min(G.m, G.k + 1 + ((p + 1) << G.dot));
   const double2* col = pan_vw(M) + which * TD_NB + lane;
   const double2* x = M.H + (size_t)G.k * G.m;
   double2 t = make_double2(0.0, 0.0);
@@ -958,44 +959,45 @@ __device__ __forceinline__ void td_prefix(int* pre, int n, F count) {
 //           needed for it), w = p + alpha v; row k+1 brought to A(k+1), and its partial norms.
 // After the panel, the caller applies A -= V W^+ + W V^+ to rows and columns >= k1
 // as one Hermitian rank-2*NB matrix product.
-constexpr int TD_ST = 16 * 33 + 32;  // shared memory of one warp's tile (complex)
+constexpr int TD_ST = 16 * 33 + 64;  // shared memory of one warp's tile (complex)
 constexpr int TD_SMEM = TD_WARPS * TD_ST * (int)sizeof(double2);
 __global__ void __launch_bounds__(TD_THREADS, 2) k_tridiag_panel(const __grid_constant__ EigBatch b, int k0, int k1) {
   extern __shared__ double2 td_sh[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __shared__ int pre[EIG_MAXP + 1];
-  __shared__ double2 xyp[TD_THREADS / (2 * TD_NB)][2 * TD_NB];  // partial X', Y' sums
-  __shared__ double2 xy_sh[2 * TD_NB];                          // Y_i = v_i^+ v, then X_i = w_i^+ v
-  __shared__ double2 vk_sh[2 * TD_NB];                          // v_i(k+1), then w_i(k+1)
+  __shared__ int pre_a[EIG_MAXP + 1], pre_b[EIG_MAXP + 1];  // items before each matrix, phase A / B
+  __shared__ double2 xy_sh[2 * TD_NB];                      // Y_i = v_i^+ v, then X_i = w_i^+ v
+  __shared__ double2 vk_sh[2 * TD_NB];                      // v_i(k+1), then w_i(k+1)
   __shared__ double2 pv_sh[TD_WARPS][32], rv_sh[TD_WARPS][32];
-  __shared__ double q_sh[TD_WARPS];
-  __shared__ double2 h0_sh, w0_sh;
+  __shared__ double q_sh[4];
+  __shared__ double2 h0_sh, p0_sh;
   __shared__ double alpha_sh;
   unsigned int target = 0;  // barrier count expected at the next grid_sync
+  auto items_a = [&](int k) {
+    td_prefix(pre_a, b.n, [&](int i) { return k0 < tail_start(b.a[i].m) ? TdGeo(b.a[i].m, k).items_a(k - k0) : 0; });
+  };
+  auto items_b = [&](int k) {
+    td_prefix(pre_b, b.n, [&](int i) { return k0 < tail_start(b.a[i].m) ? TdGeo(b.a[i].m, k).ng : 0; });
+  };
   // the partial norms of the panel's first row
-  if (warp == 0)
-    td_prefix(pre, b.n, [&](int i) { return k0 < tail_start(b.a[i].m) ? TdGeo(b.a[i].m, k0 - 1).ng : 0; });
+  if (warp == 0) items_b(k0 - 1);
   __syncthreads();
-  for (int it = warp * gridDim.x + blockIdx.x; it < pre[b.n]; it += TD_WARPS * gridDim.x) {
-    const int mi = td_find(pre, b.n, it);
+  for (int it = warp * gridDim.x + blockIdx.x; it < pre_b[b.n]; it += TD_WARPS * gridDim.x) {
+    const int mi = td_find(pre_b, b.n, it);
     const EigMat& M = b.a[mi];
     const TdGeo P(M.m, k0 - 1);
-    const int g = it - pre[mi], c = (P.g0 + g) * P.cols + lane;
-    const bool ok = lane < P.cols && c < M.m && c > k0;
+    const int g = it - pre_b[mi], c = ((P.g0 + g) << P.cols) + lane;
+    const bool ok = lane < (1 << P.cols) && c < M.m && c > k0;
     put_norm(M, g, ok ? M.H[(size_t)k0 * M.m + c] : make_double2(0.0, 0.0), c > k0 + 1);
   }
-  if (!grid_sync(b.bar, target, b.wait_clocks)) return;
+  if (!grid_sync(b.bar, target, b.wait_clocks, [&] { items_a(k0); })) return;
   for (int k = k0; k < k1; ++k) {
     const int j = k - k0;
     // ---- phase A
-    if (warp == 0)
-      td_prefix(pre, b.n, [&](int i) { return k0 < tail_start(b.a[i].m) ? TdGeo(b.a[i].m, k).items_a(j) : 0; });
-    __syncthreads();
-    for (int it = warp * gridDim.x + blockIdx.x; it < pre[b.n]; it += TD_WARPS * gridDim.x) {
-      const int mi = td_find(pre, b.n, it);
+    for (int it = warp * gridDim.x + blockIdx.x; it < pre_a[b.n]; it += TD_WARPS * gridDim.x) {
+      const int mi = td_find(pre_a, b.n, it);
       const EigMat& M = b.a[mi];
       const TdGeo G(M.m, k);
-      int rem = it - pre[mi];
+      int rem = it - pre_a[mi];
       if (rem == 0) {
         td_scalars(M, k);
         continue;
@@ -1008,89 +1010,91 @@ __global__ void __launch_bounds__(TD_THREADS, 2) k_tridiag_panel(const __grid_co
         continue;
       }
       double2* st = td_sh + warp * TD_ST;
-      if (G.rows == 8) td_tile<8>(M, G, rem - nd2, st, st + 16 * 33);
+      if (G.rows == 3) td_tile<8>(M, G, rem - nd2, st, st + 16 * 33);
       else td_tile<16>(M, G, rem - nd2, st, st + 16 * 33);
       __syncwarp();
     }
-    if (!grid_sync(b.bar, target, b.wait_clocks)) return;
+    if (!grid_sync(b.bar, target, b.wait_clocks, [&] { items_b(k); })) return;
     // ---- phase B
-    if (warp == 0)
-      td_prefix(pre, b.n, [&](int i) { return k0 < tail_start(b.a[i].m) ? TdGeo(b.a[i].m, k).ng : 0; });
-    __syncthreads();
-    for (int it = blockIdx.x; it < pre[b.n]; it += gridDim.x) {
-      const int mi = td_find(pre, b.n, it);
+    for (int it = blockIdx.x; it < pre_b[b.n]; it += gridDim.x) {
+      const int mi = td_find(pre_b, b.n, it);
       const EigMat& M = b.a[mi];
       const TdGeo G(M.m, k);
-      const int m = M.m, g = it - pre[mi];
+      const int m = M.m, g = it - pre_b[mi];
       const bool nextrow = (k + 1 < k1);
       const double2 sc = pan_scal(M)[0], tau = M.tau[k];
-      // sums over the whole trailing set: X', Y' (a quarter of the partials per 64 threads), u^+ A u, hraw(k+1)
-      {
-        const int v = threadIdx.x & (2 * TD_NB - 1), part = threadIdx.x / (2 * TD_NB);
-        if ((v & (TD_NB - 1)) < j) {
-          double2 t = make_double2(0.0, 0.0);
-          for (int p = part; p < G.nd; p += TD_THREADS / (2 * TD_NB)) t = cadd(t, pan_xy(M)[(size_t)p * 2 * TD_NB + v]);
-          xyp[part][v] = t;
-          if (part == 0) vk_sh[v] = pan_vw(M)[(size_t)(k + 1) * 2 * TD_NB + v];
-        }
-        double q = 0.0;
-        for (int t = threadIdx.x; t < G.tiles(); t += TD_THREADS) q += pan_q(M)[t];
-        q = warp_sum(q);
-        if (lane == 0) q_sh[warp] = q;
-        if (warp == TD_WARPS - 1) {  // hraw(k+1): the first strip's row blocks, then the strips to its right
-          const int e = (k + 1) & 31, nc = min(G.first_blocks(), G.nb);
-          double2 h = make_double2(0.0, 0.0);
-          for (int i = lane; i < nc + G.ns - 1; i += 32)
-            h = cadd(h, i < nc ? pan_hc(M)[(size_t)i * 32 + e] : pan_hr(M)[(size_t)(i - nc + 1) * 32 + e]);
-          h = warp_sum2(h);
-          if (lane == 0) h0_sh = h;
-        }
-      }
-      __syncthreads();
-      if (threadIdx.x < 2 * TD_NB) {
-        const int v = threadIdx.x;
-        if ((v & (TD_NB - 1)) < j) {
-          const double2 t = cadd(cadd(xyp[0][v], xyp[1][v]), cadd(xyp[2][v], xyp[3][v]));
-          xy_sh[v] = cfma(sc, t, cconj(vk_sh[v]));
-        } else {
-          xy_sh[v] = vk_sh[v] = make_double2(0.0, 0.0);
-        }
-      }
-      __syncthreads();
-      const int nc_ = G.cols, grp = 32 / nc_;           // columns of the piece, lane groups
-      const int cl = lane & (nc_ - 1), c = (G.g0 + g) * nc_ + cl;
+      const int nc_ = 1 << G.cols, grp = 32 >> G.cols;  // columns of the piece, lane groups
+      const int cl = lane & (nc_ - 1), c = ((G.g0 + g) << G.cols) + cl;
       const bool ok = c > k && c < m;
-      if (warp == 0) {  // alpha and w(k+1)
-        const double2 X = xy_sh[TD_NB + lane], Y = xy_sh[lane], vi = vk_sh[lane], wi = vk_sh[TD_NB + lane];
-        double gx = fma(Y.x, X.x, Y.y * X.y);
-        double2 c0 = cfma(wi, Y, cmul(vi, X));
-        if (j > 0) {
-          gx = warp_sum(gx);
-          c0 = warp_sum2(c0);
+      double2 h = make_double2(0.0, 0.0);
+      if (warp < 2) {  // X_i = w_i^+ v, Y_i = v_i^+ v over the whole trailing set
+        const int v = threadIdx.x;
+        double2 x = make_double2(0.0, 0.0), vk = x;
+        if ((v & (TD_NB - 1)) < j) {
+          vk = pan_vw(M)[(size_t)(k + 1) * 2 * TD_NB + v];
+          const double2* xy = pan_xy(M) + v;
+          double2 t = make_double2(0.0, 0.0);
+#pragma unroll 8
+          for (int p = 0; p < G.nd; ++p) t = cadd(t, xy[(size_t)p * 2 * TD_NB]);
+          x = cfma(sc, t, cconj(vk));
         }
-        if (lane == 0) {
-          double q = 0.0;
-          for (int w = 0; w < TD_WARPS; ++w) q += q_sh[w];
-          const double a00 = pan_scal(M)[1].x;
-          const double2 s0 = cmul(sc, h0_sh);
-          // v^+ A(k) v = A00 + 2 Re(sc hraw_0) + |sc|^2 u^+ A u - 2 Re sum_i conj(Y_i) X_i
-          const double va = fma(fma(sc.x, sc.x, sc.y * sc.y), q, fma(2.0, s0.x - gx, a00));
-          const double alpha = -0.5 * fma(tau.x, tau.x, tau.y * tau.y) * va;
-          const double2 p0 = cmul(tau, make_double2(a00 + s0.x - c0.x, s0.y - c0.y));
-          alpha_sh = alpha;
-          w0_sh = make_double2(p0.x + alpha, p0.y);
-        }
-      } else {  // the other warps: sc hraw - corrections, and the corrections of row k+1
-        const int slots = (TD_WARPS - 1) * grp, slot = (warp - 1) * grp + lane / nc_;
-        const int S = c / 32 - G.s0, e = c & 31;
-        double2 h = make_double2(0.0, 0.0), rc = make_double2(0.0, 0.0);
+        xy_sh[v] = x;
+        vk_sh[v] = vk;
+      } else {
+        // hraw of the piece's columns: row blocks down to the strip's own, then the strips to its right
+        const int slots = (TD_WARPS - 2) * grp, slot = (warp - 2) * grp + (lane >> G.cols);
         if (ok) {
-          const int n1 = min(G.nb, G.first_blocks() + S * G.per());  // row blocks down to the strip's own
+          const int S = (c >> 5) - G.s0, e = c & 31, n1 = min(G.nb, G.first_blocks() + S * G.per());
           const double2* hc = pan_hc(M) + (size_t)S * G.nb * 32 + e;
           const double2* hr = pan_hr(M) + (size_t)S * G.ns * 32 + e;
+#pragma unroll 4
           for (int i = slot; i < n1; i += slots) h = cadd(h, hc[(size_t)i * 32]);
+#pragma unroll 4
           for (int T = S + 1 + slot; T < G.ns; T += slots) h = cadd(h, hr[(size_t)T * 32]);
           h = cmul(sc, h);
+        }
+        if (warp < 6) {  // u^+ A u
+          double q = 0.0;
+          const int nt = G.tiles();
+#pragma unroll 4
+          for (int t = (warp - 2) * 32 + lane; t < nt; t += 128) q += pan_q(M)[t];
+          q = warp_sum(q);
+          if (lane == 0) q_sh[warp - 2] = q;
+        } else if (warp == 6) {  // hraw(k+1)
+          const int e = (k + 1) & 31, nc = min(G.first_blocks(), G.nb);
+          double2 t = make_double2(0.0, 0.0);
+          for (int i = lane; i < nc + G.ns - 1; i += 32)
+            t = cadd(t, i < nc ? pan_hc(M)[(size_t)i * 32 + e] : pan_hr(M)[(size_t)(i - nc + 1) * 32 + e]);
+          t = warp_sum2(t);
+          if (lane == 0) h0_sh = t;
+        }
+      }
+      __syncthreads();
+      double2 a = make_double2(0.0, 0.0), v = a;
+      if (warp == 0) {  // alpha, and v of the piece
+        if (ok && lane < nc_) {
+          a = M.H[(size_t)(k + 1) * m + c];  // A(k0)(k+1, c): its conjugate is (A e_0)(c)
+          v = M.H[(size_t)k * m + c];
+        }
+        const double2 X = xy_sh[TD_NB + lane], Y = xy_sh[lane], h0 = h0_sh;
+        double gx = fma(Y.x, X.x, Y.y * X.y);
+        if (j > 0) gx = warp_sum(gx);
+        const double q = (q_sh[0] + q_sh[1]) + (q_sh[2] + q_sh[3]);
+        // v^+ A(k) v = A00 + 2 Re(sc hraw_0) + |sc|^2 u^+ A u - 2 Re sum_i conj(Y_i) X_i
+        const double s0 = fma(sc.x, h0.x, -sc.y * h0.y);
+        const double va = fma(fma(sc.x, sc.x, sc.y * sc.y), q, fma(2.0, s0 - gx, pan_scal(M)[1].x));
+        if (lane == 0) alpha_sh = -0.5 * fma(tau.x, tau.x, tau.y * tau.y) * va;
+        v = (c == k + 1) ? make_double2(1.0, 0.0) : cmul(sc, cconj(v));
+      } else if (warp == 1) {  // p(k+1), w(k+1) = p(k+1) + alpha
+        const double2 X = xy_sh[TD_NB + lane], Y = xy_sh[lane], vi = vk_sh[lane], wi = vk_sh[TD_NB + lane];
+        double2 c0 = cfma(wi, Y, cmul(vi, X));
+        if (j > 0) c0 = warp_sum2(c0);
+        const double2 h0 = cfma(sc, h0_sh, pan_scal(M)[1]);
+        if (lane == 0) p0_sh = cmul(tau, csub(h0, c0));
+      } else {  // - corrections of the product, and the corrections of row k+1
+        const int slots = (TD_WARPS - 2) * grp, slot = (warp - 2) * grp + (lane >> G.cols);
+        double2 rc = make_double2(0.0, 0.0);
+        if (ok) {
           const double2* row = pan_vw(M) + (size_t)c * 2 * TD_NB;
           for (int i = slot; i < j; i += slots) {
             const double2 vc = row[i], wc = row[TD_NB + i];
@@ -1108,8 +1112,10 @@ __global__ void __launch_bounds__(TD_THREADS, 2) k_tridiag_panel(const __grid_co
         for (int o = nc_; o < 32; o <<= 1) {
           h.x += __shfl_xor_sync(0xffffffffu, h.x, o);
           h.y += __shfl_xor_sync(0xffffffffu, h.y, o);
-          rc.x += __shfl_xor_sync(0xffffffffu, rc.x, o);
-          rc.y += __shfl_xor_sync(0xffffffffu, rc.y, o);
+          if (j > 0 && nextrow) {
+            rc.x += __shfl_xor_sync(0xffffffffu, rc.x, o);
+            rc.y += __shfl_xor_sync(0xffffffffu, rc.y, o);
+          }
         }
         if (lane < nc_) {
           pv_sh[warp][lane] = h;
@@ -1118,45 +1124,42 @@ __global__ void __launch_bounds__(TD_THREADS, 2) k_tridiag_panel(const __grid_co
       }
       __syncthreads();
       if (warp == 1 && lane < nc_) {  // the row corrections, beside warp 0's product
-        double2 rs = rv_sh[1][lane];
-        for (int w = 2; w < TD_WARPS; ++w) rs = cadd(rs, rv_sh[w][lane]);
+        double2 rs = make_double2(0.0, 0.0);
+        if (j > 0 && nextrow)
+          rs = cadd(cadd(cadd(rv_sh[2][lane], rv_sh[3][lane]), cadd(rv_sh[4][lane], rv_sh[5][lane])),
+                    cadd(rv_sh[6][lane], rv_sh[7][lane]));
         rv_sh[0][lane] = rs;
       }
-      double2 v = make_double2(0.0, 0.0), w = v, a = v;
-      if (warp == 0) {
-        const bool mine = ok && lane < nc_;
-        if (mine) {
-          a = M.H[(size_t)(k + 1) * m + c];  // A(k0)(k+1, c): its conjugate is (A e_0)(c)
-          v = (c == k + 1) ? make_double2(1.0, 0.0) : cmul(sc, cconj(M.H[(size_t)k * m + c]));
-          double2 h = cconj(a);
-          for (int q = 1; q < TD_WARPS; ++q) h = cadd(h, pv_sh[q][lane]);
-          const double alpha = alpha_sh;
-          w = cmul(tau, h);
-          w = make_double2(fma(alpha, v.x, w.x), fma(alpha, v.y, w.y));
-          double2* VW = pan_vw(M) + (size_t)c * 2 * TD_NB;
-          double2* WV = pan_wv(M) + (size_t)c * 2 * TD_NB;
-          VW[j] = v;
-          VW[TD_NB + j] = w;
-          WV[j] = w;
-          WV[TD_NB + j] = v;
-          M.H[(size_t)k * m + c] = v;
-        }
+      double2 w = make_double2(0.0, 0.0);
+      if (warp == 0 && ok && lane < nc_) {
+        const double2 h1 = cadd(cadd(pv_sh[2][lane], pv_sh[3][lane]), cadd(pv_sh[4][lane], pv_sh[5][lane]));
+        const double2 h2 = cadd(cconj(a), cadd(pv_sh[6][lane], pv_sh[7][lane]));
+        const double alpha = alpha_sh;
+        w = cmul(tau, cadd(h1, h2));
+        w = make_double2(fma(alpha, v.x, w.x), fma(alpha, v.y, w.y));
+        double2* VW = pan_vw(M) + (size_t)c * 2 * TD_NB;
+        double2* WV = pan_wv(M) + (size_t)c * 2 * TD_NB;
+        VW[j] = v;
+        VW[TD_NB + j] = w;
+        WV[j] = w;
+        WV[TD_NB + j] = v;
+        M.H[(size_t)k * m + c] = v;
       }
       __syncthreads();
       if (warp == 0 && nextrow) {  // row k+1 of A(k+1) = A(k0) - corrections - conj(w) - w(k+1) conj(v)
         double2 x = make_double2(0.0, 0.0);
         if (ok && lane < nc_) {
           a = csub(csub(a, rv_sh[0][lane]), cconj(w));
-          x = csub(a, cmul(w0_sh, cconj(v)));
+          x = cfma_conj(v, make_double2(-p0_sh.x - alpha_sh, -p0_sh.y), a);
           M.H[(size_t)(k + 1) * m + c] = x;
         }
         const bool off = c > k + 1 && lane < nc_;  // the diagonal is not part of the next reflector
         put_norm(M, g, off ? x : make_double2(0.0, 0.0), c > k + 2);
       }
-      __syncthreads();
+      if (it + (int)gridDim.x < pre_b[b.n]) __syncthreads();  // the shared arrays are free for the next piece
     }
     if (k + 1 < k1)
-      if (!grid_sync(b.bar, target, b.wait_clocks)) return;
+      if (!grid_sync(b.bar, target, b.wait_clocks, [&] { items_a(k + 1); })) return;
   }
 }
 
@@ -1305,8 +1308,15 @@ int eig_trace(const EigBatch& b, cudaStream_t s) {
   return 1;
 }
 
-int eig_tridiagonalize(const EigBatch& b, bool mixed, void* const* oz_ws, int* status, cudaStream_t s) {
-  if (b.n == 0) return 0;
+int eig_tridiagonalize(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status, cudaStream_t s) {
+  if (b0.n == 0) return 0;
+  EigBatch b = b0;
+  for (int i = 0; i < b.n; ++i) {  // where the panel arrays' sized parts start
+    EigMat& M = b.a[i];
+    M.td_hr = M.pan + (size_t)M.m * 4 * TD_NB + (size_t)TD_DOTS * 2 * TD_NB + 32 * td_hc_tiles(M.m);
+    M.td_q = reinterpret_cast<double*>(M.td_hr + 32 * td_hr_tiles(M.m));
+    M.td_sc = M.td_hr + 32 * td_hr_tiles(M.m) + (td_hc_tiles(M.m) + 1) / 2;
+  }
   const int mm = max_m(b);
   static int sms = 0, per_sm = 0;
   if (sms == 0) {
@@ -1322,17 +1332,17 @@ int eig_tridiagonalize(const EigBatch& b, bool mixed, void* const* oz_ws, int* s
   for (int i = 0; i < b.n; ++i) kend = std::max(kend, tail_start(b.a[i].m));
   for (int k0 = 0; k0 < kend; k0 += TD_NB) {
     int k1 = std::min(mm, k0 + TD_NB);
-    // grid sized to the larger of the panel's phases: tiles per warp, pieces per block
+    // a block per tile or piece while SMs are free: the FP64 pipe is per SM, so a tile is faster alone
     long long tiles = 0, pieces = 0;
     for (int i = 0; i < b.n; ++i) {
       if (k0 >= tail_start(b.a[i].m)) continue;
       const int n = b.a[i].m - k0 - 1;
       tiles += (long long)td_tiles(n) / 2 + 1;
-      pieces += n / td_cols(n) + 2;
+      pieces += (n >> td_cols(n)) + 2;
     }
-    const int gsz = (int)std::min<long long>(grid, std::max(pieces, tiles / TD_WARPS + 1));
+    const int gsz = (int)std::min<long long>(grid, std::max(pieces, tiles));
     cudaMemsetAsync(b.bar, 0, sizeof(unsigned int), s);  // arrival count of the grid barrier
-    void* args[] = {const_cast<EigBatch*>(&b), &k0, &k1};
+    void* args[] = {&b, &k0, &k1};
     if (cudaLaunchCooperativeKernel((const void*)k_tridiag_panel, dim3(gsz), dim3(TD_THREADS), args, TD_SMEM,
                                     s) != cudaSuccess)
       return -1;

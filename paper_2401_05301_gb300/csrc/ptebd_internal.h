@@ -184,6 +184,9 @@ struct EigMat {
   double* work;      // Sturm pairs (4 + 2 m doubles), then inverse-iteration scratch (5 m K doubles)
   double2* U;        // K x m eigenvectors of H, one per row (U[j*m + r] = u_j[r])
   double2* pan;      // panel arrays of the blocked reduction [eig_panel_doubles2(m)]
+  double2* td_hr;    // parts of pan, set by the reduction: row sums of its tiles, their u^+ A u, its scalars
+  double* td_q;
+  double2* td_sc;
   int m, kmax, K;
 };
 
