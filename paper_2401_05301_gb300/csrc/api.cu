@@ -116,6 +116,7 @@ int gate_sites(const tebd_ctx* c) { return c->ss ? c->L - 1 : c->L - 2; }
 // projection Y1 (K x n1 over m) and projection Y2 (K x m over m) products.
 double oz_slot_bytes(long long capmax, long long d, long long chi_max, bool two_site = false) {
   const long long mm = capmax * d, n1max = (two_site ? d : d * d) * capmax, kc = std::min<long long>(mm, chi_max);
+  const long long D = two_site ? d * d : d * d * d;
   return (double)std::max({oz_workspace_bytes((int)mm, (int)mm, (int)n1max, true),
                            oz_workspace_bytes((int)kc, (int)n1max, (int)mm, false),
                            oz_workspace_bytes((int)kc, (int)mm, (int)mm, false),
@@ -123,7 +124,10 @@ double oz_slot_bytes(long long capmax, long long d, long long chi_max, bool two_
                            oz_workspace_bytes((int)mm, (int)(d * capmax), (int)capmax, false),
                            oz_workspace_bytes((int)(mm * d), (int)(d * capmax), (int)capmax, false),
                            oz_workspace_bytes((int)mm, (int)kc, (int)n1max, false),
-                           oz_workspace_bytes((int)mm, (int)kc, (int)mm, false)});
+                           oz_workspace_bytes((int)mm, (int)kc, (int)mm, false),
+                           // precision 1: the gate's TF32 planes (those of its other products are smaller
+                           // than the same products' digits)
+                           tc_workspace_bytes((int)D, (int)capmax, (int)D, (int)capmax)});
 }
 
 double slot_bytes_for(long long capmax, long long d, long long chi_max, int precision, bool two_site = false) {
@@ -622,6 +626,9 @@ int update_chunk(tebd_ctx* c, std::vector<Triple>& ts, int tidx) {
     for (auto& T : ts)
       if (int r = ensure_oz(T.h)) return r;
   const bool two = c->ss;  // super sites: theta~ = B_i B_{i+1}, one cut, B_{i+1} = V^+
+  // a triple's workspace for the tensor-core products: digit planes, or the TF32 planes of a contraction
+  std::vector<void*> oz_ws;
+  for (auto& T : ts) oz_ws.push_back(T.h->slots[T.slot].oz);
   for (auto& T : ts) {
     const tebd_ctx* o = T.h;
     T.chl = o->chi[T.i]; T.c1 = o->chi[T.i + 1]; T.c2 = o->chi[T.i + 2];
@@ -676,9 +683,9 @@ int update_chunk(tebd_ctx* c, std::vector<Triple>& ts, int tidx) {
         c->launches += oz_gemm_launch(o2, c->d_status, s);
         c->launches += g3.launch(s);
       } else {
-        c->launches += g1.launch(s, tf32, c->d_status);
-        c->launches += g2.launch(s, tf32, c->d_status);
-        c->launches += g3.launch(s, tf32, c->d_status);
+        c->launches += tf32 ? g1.launch_tf32(s, c->d_status, oz_ws.data()) : g1.launch(s);
+        c->launches += tf32 ? g2.launch_tf32(s, c->d_status, oz_ws.data()) : g2.launch(s);
+        c->launches += tf32 ? g3.launch_tf32(s, c->d_status, oz_ws.data()) : g3.launch(s);
       }
     }
     if (!c->randomized) {  // the randomized cut never forms the Gram matrix of theta'
@@ -763,7 +770,7 @@ int update_chunk(tebd_ctx* c, std::vector<Triple>& ts, int tidx) {
         }
         c->launches += oz_gemm_launch(o6, c->d_status, s);
       } else {
-        c->launches += g6.launch(s, tf32, c->d_status);
+        c->launches += tf32 ? g6.launch_tf32(s, c->d_status, oz_ws.data()) : g6.launch(s);
       }
       if (c->capturing)  // B_i / ||s|| with the norm the truncation left on the device
         for (auto& T : ts)
@@ -844,7 +851,7 @@ int update_chunk(tebd_ctx* c, std::vector<Triple>& ts, int tidx) {
         }
         c->launches += oz_gemm_launch(o9, c->d_status, s);
       } else {
-        c->launches += g9.launch(s, tf32, c->d_status);
+        c->launches += tf32 ? g9.launch_tf32(s, c->d_status, oz_ws.data()) : g9.launch(s);
       }
       if (c->capturing)
         for (auto& T : ts)
@@ -1148,7 +1155,23 @@ int tebd_zgemm(int precision, int opB, int M, int N, int K, double alpha, const 
     Gemm g(true, OP_N, opB ? OP_C : OP_N);
     GemmProb& p = g.add(M, N, K, A, lda, B, ldb, C, ldc);
     p.alpha_re = alpha;
-    g.launch(static_cast<cudaStream_t>(cuda_stream), precision == 1, nullptr);
+    if (precision == 1) {
+      cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+      void* ws = nullptr;
+      if (cudaMallocAsync(&ws, tc_workspace_bytes(M, N, K, 1), st) != cudaSuccess) {
+        cudaGetLastError();
+        return TEBD_ERR_OOM;
+      }
+      try {
+        g.launch_tf32(st, nullptr, &ws);
+      } catch (...) {
+        cudaFreeAsync(ws, st);
+        return TEBD_ERR_OOM;
+      }
+      cudaFreeAsync(ws, st);
+    } else {
+      g.launch(static_cast<cudaStream_t>(cuda_stream));
+    }
   } catch (...) {
     return TEBD_ERR_OOM;
   }

@@ -300,28 +300,29 @@ int gemm_launch_single(bool complex_, int opA, int opB, const GemmProb& p, cudaS
   return launches;
 }
 
-int Gemm::launch(cudaStream_t s, bool mixed, int* status) {
-  if (mixed && cplx_ && opA_ == OP_N && (opB_ == OP_N || opB_ == OP_C)) {
-    std::vector<TcGemmProb> tp;
-    bool eligible = true;
-    for (const GemmProb& p : probs_) {
-      if (p.s_red || p.s_red_b || p.s_row || p.s_col || p.accumulate || p.herm || p.alpha_im != 0.0)
-        eligible = false;
-      TcGemmProb q{};
-      q.A = static_cast<const double2*>(p.A);
-      q.B = static_cast<const double2*>(p.B);
-      q.C = static_cast<double2*>(p.C);
-      q.lda = p.lda; q.ldb = p.ldb; q.ldc = p.ldc;
-      q.sA = p.sA; q.sB = p.sB; q.sC = p.sC;
-      q.alpha = p.alpha_re;
-      q.M = p.M; q.N = p.N; q.K = p.K; q.batch = p.batch; q.opB = opB_;
-      tp.push_back(q);
-    }
-    if (eligible) {
-      probs_.clear();
-      return tc_gemm_launch(tp, status, s);
-    }
+int Gemm::launch_tf32(cudaStream_t s, int* status, void* const* ws) {
+  std::vector<TcGemmProb> tp;
+  for (size_t i = 0; i < probs_.size(); ++i) {
+    const GemmProb& p = probs_[i];
+    if (!cplx_ || opA_ != OP_N || opB_ == OP_CJ || p.s_red || p.s_red_b || p.s_row || p.s_col || p.accumulate || p.herm ||
+        p.alpha_im != 0.0 || (p.batch > 1 && p.sA != 0))
+      throw std::runtime_error("not a 3xTF32 product");
+    TcGemmProb q{};
+    q.A = static_cast<const double2*>(p.A);
+    q.B = static_cast<const double2*>(p.B);
+    q.C = static_cast<double2*>(p.C);
+    q.lda = p.lda; q.ldb = p.ldb; q.ldc = p.ldc;
+    q.sB = p.sB; q.sC = p.sC;
+    q.alpha = p.alpha_re;
+    q.M = p.M; q.N = p.N; q.K = p.K; q.batch = p.batch; q.opB = opB_;
+    q.ws = ws[i];
+    tp.push_back(q);
   }
+  probs_.clear();
+  return tc_gemm_launch(tp, status, s);
+}
+
+int Gemm::launch(cudaStream_t s) {
   int launches = 0;
   for (size_t i = 0; i < probs_.size();)
     i = launch_batch(cplx_, opA_, opB_, probs_.data(), i, probs_.size(), launches, s);

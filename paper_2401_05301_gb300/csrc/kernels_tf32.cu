@@ -22,14 +22,18 @@
 // accumulators into FP32 registers with round-to-nearest adds (measured bias
 // ~4e-8 relative, independent of K).
 //
-// Kernel: one CTA (256 threads) per 128 x 128 tile of the real product.
-// All threads load and split a K-slab of A and B into 128-byte-swizzled,
-// K-major shared-memory tiles (the canonical layout of tcgen05 matrix
-// descriptors), two slabs double-buffered; one thread issues
-// tcgen05.mma.kind::tf32 (M = 128, N = 128, K = 8) and commits each slab to an
-// mbarrier; the next slab is loaded while the current one multiplies.  Every mbarrier
-// wait is bounded (~1 s); on timeout the CTA flags an error, drains its issued
-// MMAs (bounded), frees its tensor memory and returns.
+// Data path.  A packing kernel cuts every operand element once and writes the hi and lo planes in
+// the 128-byte-swizzled K-major image that the tensor core reads (blocks of 32 rows x 32 reals, 4 KB,
+// ordered [plane][slab][row block]), so a tile of a slab is one contiguous bulk copy per plane.  The
+// product kernel (one 128 x 128 real tile per CTA) is warp-specialised: one thread issues the
+// copies into a ring of three slabs, one thread issues tcgen05.mma.kind::tf32 (M = 128, N = 128,
+// K = 8), and eight warps drain each accumulator as soon as its three products are done and hand
+// it back, so the products of the next slab overlap the drains.  Tiles leave through shared memory
+// in whole rows.
+// Bound: the drains (64 KB of tensor memory and 128 x 128 adds per k-step).  Measured against
+// splitting both operands again in every CTA (same bits): 4096 x 1024 x 256 complex 683 -> 132 us.
+// Every mbarrier wait is bounded (~1 s); on timeout the CTA flags an error, drains its issued
+// copies and MMAs (bounded), frees its tensor memory and returns.
 #include "ptebd_internal.h"
 
 #include <algorithm>
@@ -42,15 +46,19 @@ namespace {
 constexpr int TM = 128;               // rows of the real product per CTA (UMMA M)
 constexpr int TN = 128;               // columns of the real product per CTA (UMMA N) = 64 complex
 constexpr int TK = 32;                // reals of K per slab (one 128-byte swizzle row of fp32)
-constexpr int NT = 256;               // threads per CTA
+constexpr int DW = 8;                 // drain warps: 4 lane groups x 2 column halves
+constexpr int NT = 32 * (DW + 2);     // + one copy warp + one MMA warp
+constexpr int BLK = 4096;             // one packed block: 32 rows x 32 fp32
 constexpr int A_BYTES = TM * TK * 4;  // 16 KB per plane
 constexpr int B_BYTES = TN * TK * 4;  // 16 KB per plane
 constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;  // hi and lo planes of A and B: 64 KB
 constexpr int NACC = TK / 8;          // one accumulator per k-step of a slab
 constexpr int TMEM_COLS = NACC * TN;  // 512: the whole tensor memory of the SM
-constexpr int STAGES = 2;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 128;
+constexpr int STAGES = 3;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+constexpr int OUT_LD = TN / 2 + 1;    // staged output row (complex), padded
 constexpr long long WAIT_CLOCKS = 2000000000LL;  // ~1 s at 2 GHz
+static_assert(TM * OUT_LD * 16 <= STAGES * STAGE_BYTES, "the staged tile must fit the stages");
 
 // ---- small PTX wrappers ---------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -59,11 +67,11 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
 }
 
-// Bounded wait for the phase with the given parity; false on timeout.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+// Bounded wait for the phase with the given parity; false on timeout or once another role failed.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* fail) {
   const uint32_t a = smem_u32(bar);
   const long long t0 = clock64();
-  while (true) {
+  for (int it = 0;; ++it) {
     uint32_t done;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -71,11 +79,28 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
         : "r"(a), "r"(parity)
         : "memory");
     if (done) return true;
-    if (clock64() - t0 > WAIT_CLOCKS) return false;
+    if ((it & 63) == 63) {
+      if (fail && *fail) return false;
+      if (clock64() - t0 > WAIT_CLOCKS) return false;
+    }
   }
 }
 
-__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
+               : "memory");
+}
+// Bulk copy global -> shared (TMA engine), completion counted on bar.
+__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -147,110 +172,127 @@ __device__ __forceinline__ uint32_t swz(int row, int k) {
   return (uint32_t)(row * 128 + ((((k >> 2) ^ (row & 7)) & 7) << 4) + ((k & 3) << 2));
 }
 
-__device__ __forceinline__ double2 load_c(const double2* p) { return __ldg(p); }
+// ---- packing ----------------------------------------------------------------------
 
-// Fill one slab (real K offset k0) of the hi/lo planes of A and B.
-__device__ void fill_slab(const TcGemmProb& P, const double2* A, const double2* B, int row0, int col0, int k0,
-                          uint8_t* st) {
-  uint8_t* Ahi = st;
-  uint8_t* Alo = st + A_BYTES;
-  uint8_t* Bhi = st + 2 * A_BYTES;
-  uint8_t* Blo = st + 2 * A_BYTES + B_BYTES;
-  const int kc0 = k0 >> 1;  // complex K offset of the slab
-  // A: 128 rows x 16 complex; thread t handles (row = t/2, 8 complex per thread)
-  for (int idx = threadIdx.x; idx < TM * 16; idx += NT) {
-    const int r = idx >> 4, q = idx & 15;
-    const int gr = row0 + r, gk = kc0 + q;
-    double2 v = make_double2(0.0, 0.0);
-    if (gr < P.M && gk < P.K) v = load_c(A + (long long)gr * P.lda + gk);
-    uint32_t h0, l0, h1, l1;
-    split_tf32(v.x, h0, l0);
-    split_tf32(v.y, h1, l1);
-    *reinterpret_cast<uint32_t*>(Ahi + swz(r, 2 * q)) = h0;
-    *reinterpret_cast<uint32_t*>(Ahi + swz(r, 2 * q + 1)) = h1;
-    *reinterpret_cast<uint32_t*>(Alo + swz(r, 2 * q)) = l0;
-    *reinterpret_cast<uint32_t*>(Alo + swz(r, 2 * q + 1)) = l1;
+// One operand's planes: rows x K complex; A: element (r, k) at X[r * rs + k]; B: row r is column r of
+// op(B), element (k, r) at X[(r / per) * sb + (r % per) * rs + k * ks] (conjugated for op = C).  A row of A is one row of
+// reals (re, im); a column of B is two: (br, -bi) and (bi, br).
+struct TfPackJob {
+  const double2* X;
+  long long rs, ks, sb;
+  uint8_t* P;      // hi plane, then lo plane
+  size_t plane;    // bytes of a plane
+  int rows, K, per, b, conj, nrb, nkt;
+};
+struct TfPackBatch {
+  TfPackJob job[2 * TC_MAXP];
+  int block_start[2 * TC_MAXP + 1];
+  int njob;
+};
+
+// One block per packed block: 32 rows x 16 complex (A) or 16 columns x 16 complex (B).
+__global__ void __launch_bounds__(256) k_tf_pack(const __grid_constant__ TfPackBatch pb) {
+  int j = 0;
+  for (int hi = pb.njob - 1; j < hi;) {
+    const int mid = (j + hi + 1) >> 1;
+    if (pb.block_start[mid] <= (int)blockIdx.x) j = mid; else hi = mid - 1;
   }
-  // B': rows 2j, 2j+1 (j = complex column) x 32 reals of K; element b = op(B)(k, j)
-  //   row 2j   : ( br, -bi ) at k' = 2k, 2k+1     row 2j+1 : ( bi, br )
-  for (int idx = threadIdx.x; idx < (TN / 2) * 16; idx += NT) {
-    int jj, q;
-    if (P.opB == OP_N) { jj = idx & (TN / 2 - 1); q = idx / (TN / 2); } else { q = idx & 15; jj = idx >> 4; }
-    const int gj = (col0 >> 1) + jj, gk = kc0 + q;
-    double2 v = make_double2(0.0, 0.0);
-    if (gj < P.N && gk < P.K) {
-      if (P.opB == OP_N) {
-        v = load_c(B + (long long)gk * P.ldb + gj);
-      } else {
-        v = load_c(B + (long long)gj * P.ldb + gk);
-        v.y = -v.y;
-      }
+  const TfPackJob& J = pb.job[j];
+  const int local = blockIdx.x - pb.block_start[j];
+  const int rb = local % J.nrb, kt = local / J.nrb;
+  uint8_t* hi_p = J.P + ((size_t)kt * J.nrb + rb) * BLK;
+  uint8_t* lo_p = hi_p + J.plane;
+  if (!J.b) {
+    for (int idx = threadIdx.x; idx < 32 * 16; idx += 256) {
+      const int r = idx >> 4, q = idx & 15;
+      const int gr = rb * 32 + r, gk = kt * 16 + q;
+      double2 v = make_double2(0.0, 0.0);
+      if (gr < J.rows && gk < J.K) v = __ldg(J.X + (long long)gr * J.rs + gk);
+      uint32_t h0, l0, h1, l1;
+      split_tf32(v.x, h0, l0);
+      split_tf32(v.y, h1, l1);
+      const uint32_t at = swz(r, 2 * q);  // an even k: both words in one 8-byte slot
+      *reinterpret_cast<uint2*>(hi_p + at) = make_uint2(h0, h1);
+      *reinterpret_cast<uint2*>(lo_p + at) = make_uint2(l0, l1);
     }
-    uint32_t hr, lr, hi_, li_;
+    return;
+  }
+  {
+    int jj, q;
+    if (J.ks == 1) { q = threadIdx.x & 15; jj = threadIdx.x >> 4; } else { jj = threadIdx.x & 15; q = threadIdx.x >> 4; }
+    const int gj = rb * 16 + jj, gk = kt * 16 + q;
+    double2 v = make_double2(0.0, 0.0);
+    if (gj < J.rows && gk < J.K) {
+      v = __ldg(J.X + (long long)(gj / J.per) * J.sb + (long long)(gj % J.per) * J.rs + (long long)gk * J.ks);
+      if (J.conj) v.y = -v.y;
+    }
+    uint32_t hr, lr, hm, lm;
     split_tf32(v.x, hr, lr);
-    split_tf32(v.y, hi_, li_);
+    split_tf32(v.y, hm, lm);
     const uint32_t sign = 0x80000000u;
-    const int r0 = 2 * jj, r1 = 2 * jj + 1, ka = 2 * q, kb = 2 * q + 1;
-    *reinterpret_cast<uint32_t*>(Bhi + swz(r0, ka)) = hr;
-    *reinterpret_cast<uint32_t*>(Bhi + swz(r0, kb)) = hi_ ^ (hi_ ? sign : 0u);
-    *reinterpret_cast<uint32_t*>(Bhi + swz(r1, ka)) = hi_;
-    *reinterpret_cast<uint32_t*>(Bhi + swz(r1, kb)) = hr;
-    *reinterpret_cast<uint32_t*>(Blo + swz(r0, ka)) = lr;
-    *reinterpret_cast<uint32_t*>(Blo + swz(r0, kb)) = li_ ^ (li_ ? sign : 0u);
-    *reinterpret_cast<uint32_t*>(Blo + swz(r1, ka)) = li_;
-    *reinterpret_cast<uint32_t*>(Blo + swz(r1, kb)) = lr;
+    const uint32_t a0 = swz(2 * jj, 2 * q), a1 = swz(2 * jj + 1, 2 * q);
+    *reinterpret_cast<uint2*>(hi_p + a0) = make_uint2(hr, hm ^ (hm ? sign : 0u));
+    *reinterpret_cast<uint2*>(lo_p + a0) = make_uint2(lr, lm ^ (lm ? sign : 0u));
+    *reinterpret_cast<uint2*>(hi_p + a1) = make_uint2(hm, hr);
+    *reinterpret_cast<uint2*>(lo_p + a1) = make_uint2(lm, lr);
   }
 }
 
-// Add the 64 accumulator columns this thread owns (row 32g + lane, columns
-// [64h, 64h + 64) of accumulator `which`) into acc[] with round-to-nearest adds.
-__device__ __forceinline__ void drain(uint32_t tmem, int which, int g, int h, float (&acc)[64]) {
-#pragma unroll
-  for (int c0 = 0; c0 < 64; c0 += 16) {
-    uint32_t v[16];
-    const uint32_t taddr = tmem + ((uint32_t)(32 * g) << 16) + (uint32_t)(which * TN + h * 64 + c0);
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) acc[c0 + i] = __fadd_rn(acc[c0 + i], __uint_as_float(v[i]));
-  }
+// ---- the product ------------------------------------------------------------------
+
+struct TfTile {
+  const uint8_t* A;   // hi plane, lo plane planeA further
+  const uint8_t* B;
+  size_t planeA, planeB;
+  double2* C;
+  long long ldc, sC;
+  double alpha;
+  int M, N, per, nkt, nrbA, nrbB, tiles_n;
+};
+struct TfBatch {
+  TfTile p[TC_MAXP];
+  int tile_start[TC_MAXP + 1];
+  int nprob;
+  int* status;
+};
+
+// An FP32 value as FP64, on the integer pipe (the FP64 pipe takes a warp-wide conversion every 16 to 19 clocks).
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t b = __float_as_uint(f), e = (b >> 23) & 0xFF;
+  if (e == 0 || e == 0xFF) return (double)f;  // zero, subnormal, Inf, NaN
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(b << 29));
 }
 
-__global__ void __launch_bounds__(NT, 1) k_tf32x3(const __grid_constant__ TcGemmBatch gb) {
+__global__ void __launch_bounds__(NT, 1) k_tf32x3(const __grid_constant__ TfBatch gb) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* slab_bar = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
-  uint64_t* done_bar = slab_bar + STAGES;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done_bar + 1);
-  int* fail_sh = reinterpret_cast<int*>(tmem_slot + 1);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+  uint64_t* full = bars;                     // [STAGES] a slab has arrived
+  uint64_t* empty = bars + STAGES;           // [STAGES] its products are done
+  uint64_t* accfull = bars + 2 * STAGES;     // [NACC]
+  uint64_t* accempty = accfull + NACC;       // [NACC]
+  uint64_t* done = accempty + NACC;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  volatile int* fail_sh = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  // locate the problem, batch entry and tile of this CTA
-  const int tile = blockIdx.x;
   int pi = 0;
-  while (pi + 1 < gb.nprob && tile >= gb.tile_start[pi + 1]) ++pi;
-  const TcGemmProb& P = gb.p[pi];
-  const int local = tile - gb.tile_start[pi];
-  const int tn = (2 * P.N + TN - 1) / TN, tm = (P.M + TM - 1) / TM;
-  const int bidx = local / (tm * tn), rr = local % (tm * tn);
-  const int row0 = (rr / tn) * TM, col0 = (rr % tn) * TN;
-  const double2* A = P.A + (long long)bidx * P.sA;
-  const double2* B = P.B + (long long)bidx * P.sB;
-  double2* C = P.C + (long long)bidx * P.sC;
-
+  for (int hi = gb.nprob - 1; pi < hi;) {
+    const int mid = (pi + hi + 1) >> 1;
+    if (gb.tile_start[mid] <= (int)blockIdx.x) pi = mid; else hi = mid - 1;
+  }
+  const TfTile& P = gb.p[pi];
+  const int local = blockIdx.x - gb.tile_start[pi];
+  const int mt = local / P.tiles_n, nt = local - mt * P.tiles_n;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = warp & 3, h = warp >> 2;  // TMEM lane group and column half drained by this warp
-  if (warp == 0) {
+  if (warp == DW + 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
-  if (threadIdx.x == 32) {
-    for (int q = 0; q < STAGES; ++q) mbar_init(&slab_bar[q], 1);
-    mbar_init(done_bar, 1);
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    for (int i = 0; i < NACC; ++i) { mbar_init(&accfull[i], 1); mbar_init(&accempty[i], DW); }
+    mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *fail_sh = 0;
   }
@@ -258,78 +300,150 @@ __global__ void __launch_bounds__(NT, 1) k_tf32x3(const __grid_constant__ TcGemm
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const uint32_t idesc = tf32_idesc(TM, TN);
-  const int nk = (2 * P.K + TK - 1) / TK;  // slabs of 32 reals of K
+  const int nk = P.nkt;
 
-  float acc[64];
-#pragma unroll
-  for (int i = 0; i < 64; ++i) acc[i] = 0.0f;
-
-  fill_slab(P, A, B, row0, col0, 0, smem);
-  fence_async_shared();
-  __syncthreads();
-  bool ok = true;
-  for (int kb = 0; kb < nk; ++kb) {
-    const int s = kb & 1;
-    if (threadIdx.x == 0) {  // slab kb: k-step kk into accumulator kk, from a fresh start
-      tc_fence_after();
-      uint8_t* st = smem + s * STAGE_BYTES;
-      const uint32_t a_hi = smem_u32(st), a_lo = smem_u32(st + A_BYTES);
-      const uint32_t b_hi = smem_u32(st + 2 * A_BYTES), b_lo = smem_u32(st + 2 * A_BYTES + B_BYTES);
-#pragma unroll
-      for (int kk = 0; kk < NACC; ++kk) {
-        const uint32_t off = kk * 32;  // 8 tf32 = 32 bytes along K inside the swizzled row
-        const uint32_t d = tmem + (uint32_t)(kk * TN);
-        mma_tf32(d, smem_desc(a_hi + off), smem_desc(b_lo + off), idesc, 0u);
-        mma_tf32(d, smem_desc(a_lo + off), smem_desc(b_hi + off), idesc, 1u);
-        mma_tf32(d, smem_desc(a_hi + off), smem_desc(b_hi + off), idesc, 1u);
+  if (warp == DW) {
+    // ---- copies: the four planes of a slab
+    if (lane == 0) {
+      int issued = 0;
+      bool ok = true;
+      for (int kt = 0; kt < nk; ++kt) {
+        const int st = kt % STAGES;
+        if (kt >= STAGES && !mbar_wait(&empty[st], (uint32_t)((kt / STAGES - 1) & 1), fail_sh)) { ok = false; break; }
+        uint8_t* dst = smem + st * STAGE_BYTES;
+        const uint8_t* a = P.A + ((size_t)kt * P.nrbA + 4 * mt) * BLK;
+        const uint8_t* b = P.B + ((size_t)kt * P.nrbB + 4 * nt) * BLK;
+        mbar_expect_tx(&full[st], STAGE_BYTES);
+        ++issued;
+        bulk_copy(dst, a, A_BYTES, &full[st]);
+        bulk_copy(dst + A_BYTES, a + P.planeA, A_BYTES, &full[st]);
+        bulk_copy(dst + 2 * A_BYTES, b, B_BYTES, &full[st]);
+        bulk_copy(dst + 2 * A_BYTES + B_BYTES, b + P.planeB, B_BYTES, &full[st]);
       }
-      mma_commit(&slab_bar[s]);
-    }
-    if (kb + 1 < nk) {  // buffer s^1 was released when slab kb-1 finished (waited below)
-      fill_slab(P, A, B, row0, col0, (kb + 1) * TK, smem + (s ^ 1) * STAGE_BYTES);
-      fence_async_shared();
-    }
-    if (mbar_wait(&slab_bar[s], (uint32_t)((kb >> 1) & 1))) {
-#pragma unroll
-      for (int q = 0; q < NACC; ++q) drain(tmem, q, g, h, acc);
-    } else {
-      atomicExch(fail_sh, 1);
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (*fail_sh) { ok = false; break; }
-  }
-  if (!ok) {  // let every issued MMA finish (bounded) before the tensor memory is freed
-    if (threadIdx.x == 0) mma_commit(done_bar);
-    mbar_wait(done_bar, 0);
-  }
-  tc_fence_before();
-  if (ok) {
-    const int row = row0 + 32 * g + lane;
-    if (row < P.M) {
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const int j = (col0 + h * 64) / 2 + i;
-        if (j < P.N)
-          C[(long long)row * P.ldc + j] =
-              make_double2((double)acc[2 * i] * P.alpha, (double)acc[2 * i + 1] * P.alpha);
+      if (!ok) {  // let the copies already issued land before the CTA's shared memory is released
+        *fail_sh = 1;
+        for (int kt = max(0, issued - STAGES); kt < issued; ++kt)
+          mbar_wait(&full[kt % STAGES], (uint32_t)((kt / STAGES) & 1), nullptr);
       }
     }
-  } else if (threadIdx.x == 0 && gb.status) {
-    atomicExch(gb.status, -6);  // TEBD_ERR_TIMEOUT: a bounded mbarrier wait ran out
+  } else if (warp == DW + 1) {
+    // ---- products: k-step kk of every slab into accumulator kk, from a fresh start
+    if (lane == 0) {
+      const uint32_t idesc = tf32_idesc(TM, TN);
+      bool ok = true;
+      for (int kt = 0; kt < nk && ok; ++kt) {
+        const int st = kt % STAGES;
+        if (!mbar_wait(&full[st], (uint32_t)((kt / STAGES) & 1), fail_sh)) { ok = false; break; }
+        const uint32_t base = smem_u32(smem + st * STAGE_BYTES);
+        const uint32_t a_hi = base, a_lo = base + A_BYTES, b_hi = base + 2 * A_BYTES, b_lo = b_hi + B_BYTES;
+        for (int kk = 0; kk < NACC; ++kk) {
+          if (kt > 0 && !mbar_wait(&accempty[kk], (uint32_t)((kt - 1) & 1), fail_sh)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t off = kk * 32;  // 8 tf32 = 32 bytes along K inside the swizzled row
+          const uint32_t d = tmem + (uint32_t)(kk * TN);
+          mma_tf32(d, smem_desc(a_hi + off), smem_desc(b_lo + off), idesc, 0u);
+          mma_tf32(d, smem_desc(a_lo + off), smem_desc(b_hi + off), idesc, 1u);
+          mma_tf32(d, smem_desc(a_hi + off), smem_desc(b_hi + off), idesc, 1u);
+          mma_commit(&accfull[kk]);
+        }
+        if (ok) mma_commit(&empty[st]);
+      }
+      if (!ok) {
+        *fail_sh = 1;
+        mma_commit(done);  // all MMAs issued so far complete before tensor memory is freed
+        mbar_wait(done, 0, nullptr);
+      }
+    }
+  } else {
+    // ---- drain: warp (g, h) owns TMEM lanes 32g.. and columns 64h.. of every accumulator, which it adds
+    // into FP32 registers with round-to-nearest adds, k-step by k-step
+    const int g = warp & 3, h = warp >> 2;
+    float acc[64];
+#pragma unroll
+    for (int i = 0; i < 64; ++i) acc[i] = 0.0f;
+    bool ok = true;
+    for (int kt = 0; kt < nk && ok; ++kt) {
+      for (int q = 0; q < NACC; ++q) {
+        if (!mbar_wait(&accfull[q], (uint32_t)(kt & 1), fail_sh)) { ok = false; break; }
+        tc_fence_after();
+        uint32_t v[64];
+        const uint32_t taddr = tmem + ((uint32_t)(32 * g) << 16) + (uint32_t)(q * TN + h * 64);
+#pragma unroll
+        for (int c0 = 0; c0 < 64; c0 += 16)
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+              "[%16];"
+              : "=r"(v[c0]), "=r"(v[c0 + 1]), "=r"(v[c0 + 2]), "=r"(v[c0 + 3]), "=r"(v[c0 + 4]), "=r"(v[c0 + 5]),
+                "=r"(v[c0 + 6]), "=r"(v[c0 + 7]), "=r"(v[c0 + 8]), "=r"(v[c0 + 9]), "=r"(v[c0 + 10]),
+                "=r"(v[c0 + 11]), "=r"(v[c0 + 12]), "=r"(v[c0 + 13]), "=r"(v[c0 + 14]), "=r"(v[c0 + 15])
+              : "r"(taddr + c0));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&accempty[q]);  // the values are in registers
+#pragma unroll
+        for (int i = 0; i < 64; ++i) acc[i] = __fadd_rn(acc[i], __uint_as_float(v[i]));
+      }
+    }
+    if (!ok) *fail_sh = 1;
+    // every drain warp takes the same branch; when all drained everything, all copies and MMAs are done
+    int any_bad;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.s32 %0, 1, 0, q;\n}\n"
+        : "=r"(any_bad)
+        : "r"(ok ? 0 : 1), "r"(32 * DW)
+        : "memory");
+    if (!any_bad) {
+      double2* out = reinterpret_cast<double2*>(smem);
+      double2* mine = out + (size_t)(32 * g + lane) * OUT_LD + 32 * h;
+      const double al = P.alpha;
+      if (al == 1.0) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) mine[i] = make_double2(widen(acc[2 * i]), widen(acc[2 * i + 1]));
+      } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) mine[i] = make_double2(widen(acc[2 * i]) * al, widen(acc[2 * i + 1]) * al);
+      }
+      asm volatile("bar.sync 1, %0;" ::"r"(32 * DW) : "memory");
+      for (int e = threadIdx.x; e < TM * (TN / 2); e += 32 * DW) {
+        const int r = e / (TN / 2), cc = e - r * (TN / 2);
+        const int i = mt * TM + r, jj = nt * (TN / 2) + cc;
+        if (i < P.M && jj < P.N) P.C[(long long)(jj / P.per) * P.sC + (long long)i * P.ldc + jj % P.per] = out[(size_t)r * OUT_LD + cc];
+      }
+    }
   }
   __syncthreads();
-  if (warp == 0) {
+  if (*fail_sh && threadIdx.x == 0 && gb.status) atomicExch(gb.status, -6);  // TEBD_ERR_TIMEOUT: a bounded wait ran out
+  if (warp == DW + 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
   }
 }
 
+struct Geo {
+  int nkt, nrbA, nrbB;
+  size_t planeA, planeB;
+};
+Geo geometry(int M, long long N, int K) {
+  Geo g{};
+  g.nkt = (K + 15) / 16;
+  g.nrbA = 4 * ((M + TM - 1) / TM);
+  g.nrbB = (int)(4 * ((N + TN / 2 - 1) / (TN / 2)));
+  g.planeA = (size_t)g.nkt * g.nrbA * BLK;
+  g.planeB = (size_t)g.nkt * g.nrbB * BLK;
+  return g;
+}
+
 }  // namespace
 
-static_assert(sizeof(TcGemmBatch) < 4000, "kernel parameter block too large");
+static_assert(sizeof(TfBatch) < 32000 && sizeof(TfPackBatch) < 32000, "kernel parameter block too large (32 KB on sm_70 and later)");
 static_assert(tf32_idesc(128, 128) == ((1u << 4) | (2u << 7) | (2u << 10) | (16u << 17) | (8u << 24)), "idesc");
+
+size_t tc_workspace_bytes(int M, int N, int K, int batch) {
+  if (M <= 0 || N <= 0 || K <= 0 || batch <= 0) return 0;
+  const Geo g = geometry(M, (long long)N * batch, K);
+  return 2 * (g.planeA + g.planeB);
+}
 
 int tc_gemm_launch(const std::vector<TcGemmProb>& probs, int* status, cudaStream_t s) {
   static bool attr = false;
@@ -338,25 +452,63 @@ int tc_gemm_launch(const std::vector<TcGemmProb>& probs, int* status, cudaStream
     attr = true;
   }
   int launches = 0;
-  size_t i = 0;
-  while (i < probs.size()) {
-    TcGemmBatch gb{};
+  for (size_t i = 0; i < probs.size();) {
+    TfBatch gb{};
+    TfPackBatch pk{};
     gb.status = status;
-    int tiles = 0;
-    while (i < probs.size() && gb.nprob < TC_MAXP) {
-      const TcGemmProb& p = probs[i++];
+    int tiles = 0, blocks = 0;
+    for (; i < probs.size() && gb.nprob < TC_MAXP; ++i) {
+      const TcGemmProb& p = probs[i];
       if (p.M <= 0 || p.N <= 0 || p.batch <= 0) continue;
-      gb.p[gb.nprob] = p;
-      gb.tile_start[gb.nprob] = tiles;
-      tiles += p.batch * ((p.M + TM - 1) / TM) * ((2 * p.N + TN - 1) / TN);
-      gb.nprob++;
+      // the columns of all batch entries side by side: A is shared (sA = 0) or there is one entry
+      const int N = p.N * p.batch;
+      const Geo g = geometry(p.M, N, p.K);
+      uint8_t* ws = static_cast<uint8_t*>(p.ws);
+      auto job = [&](const TfPackJob& J) {
+        pk.job[pk.njob] = J;
+        pk.block_start[pk.njob++] = blocks;
+        blocks += J.nrb * J.nkt;
+      };
+      job(TfPackJob{p.A, p.lda, 1, 0, ws, g.planeA, p.M, p.K, 1, 0, 0, g.nrbA, g.nkt});
+      const bool c = p.opB == OP_C;
+      job(TfPackJob{p.B, c ? p.ldb : 1, c ? 1 : p.ldb, p.sB, ws + 2 * g.planeA, g.planeB, N, p.K, p.N, 1, c ? 1 : 0,
+                    g.nrbB, g.nkt});
+      TfTile& t = gb.p[gb.nprob];
+      t.A = ws; t.B = ws + 2 * g.planeA; t.planeA = g.planeA; t.planeB = g.planeB;
+      t.C = p.C; t.ldc = p.ldc; t.sC = p.sC; t.alpha = p.alpha; t.M = p.M; t.N = N; t.per = p.N;
+      t.nkt = g.nkt; t.nrbA = g.nrbA; t.nrbB = g.nrbB; t.tiles_n = g.nrbB / 4;
+      gb.tile_start[gb.nprob++] = tiles;
+      tiles += (g.nrbA / 4) * t.tiles_n;
     }
     gb.tile_start[gb.nprob] = tiles;
+    pk.block_start[pk.njob] = blocks;
     if (tiles == 0) continue;
+    if (blocks > 0) {
+      k_tf_pack<<<blocks, 256, 0, s>>>(pk);
+      ++launches;
+    }
     k_tf32x3<<<tiles, NT, SMEM_BYTES, s>>>(gb);
     ++launches;
   }
   return launches;
+}
+
+int tc_gemm_pooled(std::vector<TcGemmProb>& probs, void* pool, size_t bytes, int* status, cudaStream_t s) {
+  int launches = 0;
+  std::vector<TcGemmProb> group;
+  size_t used = 0;
+  for (TcGemmProb& q : probs) {
+    const size_t need = tc_workspace_bytes(q.M, q.N, q.K, q.batch);
+    if (group.size() == (size_t)TC_MAXP || used + need > bytes) {
+      launches += tc_gemm_launch(group, status, s);
+      group.clear();
+      used = 0;
+    }
+    q.ws = static_cast<char*>(pool) + used;
+    used += need;
+    group.push_back(q);
+  }
+  return launches + tc_gemm_launch(group, status, s);
 }
 
 }  // namespace ptebd

@@ -51,7 +51,7 @@ struct GemmProb {
 struct GemmBatch {
   GemmProb p[GEMM_MAXP];
   int tile_start[GEMM_MAXP + 1];
-  int nprob, opA, opB, mixed;
+  int nprob, opA, opB;
 };
 
 // ---- complex GEMM as split 3xTF32 on tcgen05 tensor cores (kernels_tf32.cu) ------
@@ -61,18 +61,16 @@ struct TcGemmProb {
   const double2* A;
   const double2* B;
   double2* C;
-  long long lda, ldb, ldc, sA, sB, sC;
+  long long lda, ldb, ldc, sB, sC;
   double alpha;
-  int M, N, K, batch, opB;
+  int M, N, K, batch, opB;  // batch > 1: entries sB / sC apart that share A
+  void* ws;  // tc_workspace_bytes(M, N, K, batch) bytes, 256-byte aligned, owned by the caller
 };
-constexpr int TC_MAXP = 24;
-struct TcGemmBatch {
-  TcGemmProb p[TC_MAXP];
-  int tile_start[TC_MAXP + 1];
-  int nprob;
-  int* status;  // set to TEBD_ERR_TIMEOUT if a bounded wait runs out
-};
+constexpr int TC_MAXP = 64;
+size_t tc_workspace_bytes(int M, int N, int K, int batch);
 int tc_gemm_launch(const std::vector<TcGemmProb>& probs, int* status, cudaStream_t s);
+// The same with the workspaces taken from one pool (bytes >= the largest problem's need).
+int tc_gemm_pooled(std::vector<TcGemmProb>& probs, void* pool, size_t bytes, int* status, cudaStream_t s);
 
 // ---- FP64-accurate complex GEMM on bf16 tensor cores, exact digit splitting (kernels_ozaki.cu)
 // C[i][j] = alpha * s_row[i / row_div] * s_col[j / col_div] * sum_k a(i, k) b(j, k)
@@ -148,9 +146,10 @@ class Gemm {
   GemmProb& add(int M, int N, int K, const void* A, long long lda, const void* B, long long ldb, void* C,
                 long long ldc);
   // Launch everything added so far (in chunks of GEMM_MAXP) on stream; returns launches issued.
-  // mixed: complex problems with op(A) = N, op(B) in {N, C}, real alpha and no
-  // scalings run as split 3xTF32 on the tensor cores instead of FP64.
-  int launch(cudaStream_t s, bool mixed = false, int* status = nullptr);
+  int launch(cudaStream_t s);
+  // The problems as split 3xTF32 on the tensor cores instead (complex, op(A) = N, op(B) in {N, C}, real
+  // alpha, no scalings, no accumulation, one entry or a shared A); ws[i]: the i-th problem's workspace.
+  int launch_tf32(cudaStream_t s, int* status, void* const* ws);
   size_t size() const { return probs_.size(); }
 
  private:

@@ -723,16 +723,27 @@ int run_prods(tebd_ctx* c, const std::vector<Prod>& ps, int engine) {
     }
     return run_oz(c, oz);
   }
-  // (an accumulating product is not eligible for the 3xTF32 kernel: Gemm::launch then keeps FP64)
+  if (engine == 1) {
+    std::vector<TcGemmProb> tp;
+    size_t need = 0;
+    for (const Prod& p : ps) {
+      if (p.accumulate) return TEBD_ERR_STATE;  // the contractions never accumulate
+      tp.push_back(TcGemmProb{p.A, p.B, p.C, p.lda, p.ldb, p.ldc, 0, 0, p.alpha, p.M, p.N, p.K, 1, p.opB, nullptr});
+      need = std::max(need, tc_workspace_bytes(p.M, p.N, p.K, 1));
+    }
+    if (need == 0) return TEBD_OK;
+    if (int r = ensure_pool(c, need)) return r;
+    c->launches += tc_gemm_pooled(tp, c->u1w->pool, c->u1w->pool_bytes, c->d_status, c->stream);
+    return check_launch(c);
+  }
   Gemm gn(true, OP_N, OP_N), gc(true, OP_N, OP_C);
   for (const Prod& p : ps) {
     GemmProb& g = (p.opB == OP_C ? gc : gn).add(p.M, p.N, p.K, p.A, p.lda, p.B, p.ldb, p.C, p.ldc);
     g.alpha_re = p.alpha;
     g.accumulate = p.accumulate;
   }
-  const bool tf32 = engine == 1;
-  c->launches += gn.launch(c->stream, tf32, c->d_status);
-  c->launches += gc.launch(c->stream, tf32, c->d_status);
+  c->launches += gn.launch(c->stream);
+  c->launches += gc.launch(c->stream);
   return check_launch(c);
 }
 
