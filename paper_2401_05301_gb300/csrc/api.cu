@@ -1138,7 +1138,7 @@ int tebd_zgemm(int precision, int opB, int M, int N, int K, double alpha, const 
     q.ldc = ldc;
     q.alpha = alpha;
     q.row_div = q.col_div = 1;
-    if (cudaMallocAsync(&q.ws, oz_workspace_bytes(M, N, K, false), st) != cudaSuccess) {
+    if (ws_alloc(&q.ws, oz_workspace_bytes(M, N, K, false), st) != cudaSuccess) {
       cudaGetLastError();
       return TEBD_ERR_OOM;
     }
@@ -1158,17 +1158,18 @@ int tebd_zgemm(int precision, int opB, int M, int N, int K, double alpha, const 
     if (precision == 1) {
       cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
       void* ws = nullptr;
-      if (cudaMallocAsync(&ws, tc_workspace_bytes(M, N, K, 1), st) != cudaSuccess) {
+      const size_t bytes = tc_workspace_bytes(M, N, K, 1);
+      if (bytes > 0 && ws_alloc(&ws, bytes, st) != cudaSuccess) {
         cudaGetLastError();
         return TEBD_ERR_OOM;
       }
       try {
         g.launch_tf32(st, nullptr, &ws);
       } catch (...) {
-        cudaFreeAsync(ws, st);
+        if (ws) cudaFreeAsync(ws, st);
         return TEBD_ERR_OOM;
       }
-      cudaFreeAsync(ws, st);
+      if (ws) cudaFreeAsync(ws, st);
     } else {
       g.launch(static_cast<cudaStream_t>(cuda_stream));
     }

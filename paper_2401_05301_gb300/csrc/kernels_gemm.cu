@@ -98,8 +98,8 @@ __device__ __forceinline__ double2 peer_value(const double2* mine, unsigned rank
   return make_double2(peer_load(m, rank), peer_load(m + 1, rank));
 }
 
-template <class A_, int OPA, int OPB>
-__global__ void __launch_bounds__(NT) gemm_kernel(const __grid_constant__ GemmBatch gb) {
+template <class A_, int OPA, int OPB, int CAP>
+__global__ void __launch_bounds__(NT) gemm_kernel(const __grid_constant__ GemmBatch<CAP> gb) {
   using T = typename A_::T;
   __shared__ T As[BK][TB + 1];
   __shared__ T Bs[BK][TB + 1];
@@ -219,10 +219,10 @@ __global__ void __launch_bounds__(NT) gemm_kernel(const __grid_constant__ GemmBa
   }
 }
 
-template <class A_, int OPA, int OPB>
-void launch_one(const GemmBatch& gb, int ctas, bool clustered, cudaStream_t s) {
+template <class A_, int OPA, int OPB, int CAP>
+void launch_one(const GemmBatch<CAP>& gb, int ctas, bool clustered, cudaStream_t s) {
   if (!clustered) {
-    gemm_kernel<A_, OPA, OPB><<<ctas, NT, 0, s>>>(gb);
+    gemm_kernel<A_, OPA, OPB, CAP><<<ctas, NT, 0, s>>>(gb);
     return;
   }
   cudaLaunchConfig_t cfg{};
@@ -235,15 +235,15 @@ void launch_one(const GemmBatch& gb, int ctas, bool clustered, cudaStream_t s) {
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, gemm_kernel<A_, OPA, OPB>, gb);  // a failure stays pending for the caller's check
+  cudaLaunchKernelEx(&cfg, gemm_kernel<A_, OPA, OPB, CAP>, gb);  // a failure stays pending for the caller's check
 }
 
-template <class A_>
-void dispatch(const GemmBatch& gb, int ctas, bool clustered, cudaStream_t s) {
-  const int key = gb.opA * 3 + gb.opB;
+template <class A_, int CAP>
+void dispatch(int opA, int opB, const GemmBatch<CAP>& gb, int ctas, bool clustered, cudaStream_t s) {
+  const int key = opA * 3 + opB;
   switch (key) {
 #define CASE(a, b) \
-  case a * 3 + b: launch_one<A_, a, b>(gb, ctas, clustered, s); break;
+  case a * 3 + b: launch_one<A_, a, b, CAP>(gb, ctas, clustered, s); break;
     CASE(0, 0) CASE(0, 1) CASE(0, 2) CASE(1, 0) CASE(1, 1) CASE(1, 2) CASE(2, 0) CASE(2, 1) CASE(2, 2)
 #undef CASE
     default: throw std::runtime_error("bad gemm op");
@@ -251,14 +251,14 @@ void dispatch(const GemmBatch& gb, int ctas, bool clustered, cudaStream_t s) {
 }
 
 // Launches the problems [i, n) that fit one batch; returns the index after the last one taken.
-size_t launch_batch(bool cplx, int opA, int opB, const GemmProb* p, size_t i, size_t n, int& launches, cudaStream_t s) {
-  GemmBatch gb{};
-  gb.opA = opA;
-  gb.opB = opB;
+template <int CAP>
+size_t launch_some(bool cplx, int opA, int opB, const GemmProb* p, size_t i, size_t n, int& launches, cudaStream_t s) {
+  GemmBatch<CAP> gb;
+  gb.nprob = 0;
   long long ctas = 0;
   bool clustered = false;
   const size_t first = i;
-  for (; i < n && gb.nprob < GEMM_MAXP; ++i) {
+  for (; i < n && gb.nprob < CAP; ++i) {
     const GemmProb& q = p[i];
     if (q.M <= 0 || q.N <= 0 || q.batch <= 0) continue;
     const int split = split_of(q);
@@ -273,14 +273,20 @@ size_t launch_batch(bool cplx, int opA, int opB, const GemmProb* p, size_t i, si
   }
   if (ctas == 0) return std::max(i, first + 1);
   gb.tile_start[gb.nprob] = (int)ctas;
-  if (cplx) dispatch<C>(gb, (int)ctas, clustered, s); else dispatch<R>(gb, (int)ctas, clustered, s);
+  if (cplx) dispatch<C, CAP>(opA, opB, gb, (int)ctas, clustered, s);
+  else dispatch<R, CAP>(opA, opB, gb, (int)ctas, clustered, s);
   ++launches;
   return i;
 }
 
+size_t launch_batch(bool cplx, int opA, int opB, const GemmProb* p, size_t i, size_t n, int& launches, cudaStream_t s) {
+  return n - i <= (size_t)FEW_MAXP ? launch_some<FEW_MAXP>(cplx, opA, opB, p, i, n, launches, s)
+                                   : launch_some<GEMM_MAXP>(cplx, opA, opB, p, i, n, launches, s);
+}
+
 }  // namespace
 
-static_assert(sizeof(GemmBatch) < 32000, "kernel parameter block too large (32 KB on sm_70 and later)");
+static_assert(sizeof(GemmBatch<GEMM_MAXP>) < 32000, "kernel parameter block too large (32 KB on sm_70 and later)");
 
 GemmProb& Gemm::add(int M, int N, int K, const void* A, long long lda, const void* B, long long ldb, void* C,
                     long long ldc) {

@@ -53,6 +53,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <mutex>
 
 namespace ptebd {
 
@@ -210,7 +211,8 @@ __device__ __forceinline__ double2 job_elem(const OzPackJob& J, int r, int k) {
   return x;
 }
 
-__device__ __forceinline__ int find_job(const OzPackBatch& pb, int blk) {
+template <int CAP>
+__device__ __forceinline__ int find_job(const OzPackBatch<CAP>& pb, int blk) {
   int j = 0, hi = pb.njob - 1;
   while (j < hi) {
     const int mid = (j + hi + 1) >> 1;
@@ -263,7 +265,8 @@ __device__ __forceinline__ void row_magnitudes(const OzPackJob& J, int rb, int (
 }
 
 // Row exponents: one block per 32 rows of a job.
-__global__ void __launch_bounds__(256) k_oz_exp(const __grid_constant__ OzPackBatch pb) {
+template <int CAP>
+__global__ void __launch_bounds__(256) k_oz_exp(const __grid_constant__ OzPackBatch<CAP> pb) {
   const int j = find_job(pb, blockIdx.x);
   const OzPackJob& J = pb.job[j];
   const int rb = blockIdx.x - pb.block_start[j];
@@ -274,7 +277,8 @@ __global__ void __launch_bounds__(256) k_oz_exp(const __grid_constant__ OzPackBa
 
 // Digits: one block per (row block, k-step) of a job; writes one or two planes.  A job with few
 // k-steps (J.own_exp) finds its row exponents here, reading its rows once more from cache.
-__global__ void __launch_bounds__(256) k_oz_pack(const __grid_constant__ OzPackBatch pb) {
+template <int CAP>
+__global__ void __launch_bounds__(256) k_oz_pack(const __grid_constant__ OzPackBatch<CAP> pb) {
   const int j = find_job(pb, blockIdx.x);
   const OzPackJob& J = pb.job[j];
   const int local = blockIdx.x - pb.block_start[j];
@@ -385,7 +389,8 @@ __device__ __forceinline__ double oz_value(long long Phi, long long Plo, int x) 
   return __longlong_as_double((long long)bits);
 }
 
-__global__ void __launch_bounds__(OZ_NT, 1) k_oz_gemm(const __grid_constant__ OzGemmBatch gb) {
+template <int CAP>
+__global__ void __launch_bounds__(OZ_NT, 1) k_oz_gemm(const __grid_constant__ OzGemmBatch<CAP> gb) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* Bst = smem;                       // two stages of all B slices
@@ -577,36 +582,40 @@ __global__ void __launch_bounds__(OZ_NT, 1) k_oz_gemm(const __grid_constant__ Oz
       asm volatile("bar.sync 1, %0;" ::"r"(32 * OZ_DW) : "memory");
       const int tid = threadIdx.x;
       const bool scaled = P.s_row || P.s_col || fabs(P.alpha) != 1.0;  // +-1 takes no FP64 multiply
-      for (int e = tid; e < OZ_TM * OZ_TNC; e += 32 * OZ_DW) {
-        const int r = e / OZ_TNC, cc = e % OZ_TNC;
-        const int i = mt * OZ_TM + r, jj = nt * OZ_TNC + cc;
-        if (i >= P.M || jj >= P.N || (P.herm && jj > i)) continue;
-        double2 val = make_double2(stage[r * OZ_STAGE_LD + cc], stage[r * OZ_STAGE_LD + OZ_TNC + cc]);
-        if (scaled) {
-          double f = P.alpha;
-          if (P.s_row) f *= P.s_row[i / P.row_div];
-          if (P.s_col) f *= P.s_col[jj / P.col_div];
-          val.x *= f;
-          val.y *= f;
-        } else if (P.alpha < 0.0) {
-          val.x = -val.x;
-          val.y = -val.y;
-        }
-        if (P.Creal) {  // real result (real operands): only the real part is stored
-          double* dst = P.Creal + (long long)i * P.ldc + jj;
-          if (P.beta) val.x += *dst;
-          *dst = val.x;
-        } else {
-          double2* dst = P.C + (long long)i * P.ldc + jj;
-          if (P.beta) {
-            const double2 old = *dst;
-            val.x += old.x;
-            val.y += old.y;
+      const int cc = tid & (OZ_TNC - 1), jj = nt * OZ_TNC + cc;  // a thread keeps its column
+      if (jj < P.N) {
+        const double fc = scaled ? (P.s_col ? P.alpha * P.s_col[jj / P.col_div] : P.alpha) : 1.0;
+        const int rows = min(OZ_TM, P.M - mt * OZ_TM);
+        for (int r = tid / OZ_TNC; r < rows; r += 32 * OZ_DW / OZ_TNC) {
+          const int i = mt * OZ_TM + r;
+          if (P.herm && jj > i) continue;
+          double2 val = make_double2(stage[r * OZ_STAGE_LD + cc], stage[r * OZ_STAGE_LD + OZ_TNC + cc]);
+          if (scaled) {
+            const double f = P.s_row ? (P.s_col ? P.alpha * P.s_row[i / P.row_div] * P.s_col[jj / P.col_div]
+                                                : fc * P.s_row[i / P.row_div])
+                                     : fc;
+            val.x *= f;
+            val.y *= f;
+          } else if (P.alpha < 0.0) {
+            val.x = -val.x;
+            val.y = -val.y;
           }
-          *dst = val;
+          if (P.Creal) {  // real result (real operands): only the real part is stored
+            double* dst = P.Creal + (long long)i * P.ldc + jj;
+            if (P.beta) val.x += *dst;
+            *dst = val.x;
+          } else {
+            double2* dst = P.C + (long long)i * P.ldc + jj;
+            if (P.beta) {
+              const double2 old = *dst;
+              val.x += old.x;
+              val.y += old.y;
+            }
+            *dst = val;
+          }
+          stage[r * OZ_STAGE_LD + cc] = val.x;  // the final value, for the mirror below
+          stage[r * OZ_STAGE_LD + OZ_TNC + cc] = val.y;
         }
-        stage[r * OZ_STAGE_LD + cc] = val.x;  // the final value, for the mirror below
-        stage[r * OZ_STAGE_LD + OZ_TNC + cc] = val.y;
       }
       if (P.herm) {  // mirror the strictly lower part: C[j][i] = conj(C[i][j])
         asm volatile("bar.sync 1, %0;" ::"r"(32 * OZ_DW) : "memory");
@@ -652,9 +661,46 @@ Geo geometry(int M, int N, int K, bool gram) {
 
 }  // namespace
 
-static_assert(sizeof(OzGemmBatch) < 32000, "kernel parameter block too large (32 KB on sm_70 and later)");
-static_assert(sizeof(OzPackBatch) < 32000, "kernel parameter block too large");
+static_assert(sizeof(OzGemmBatch<OZ_MAXP>) < 32000, "kernel parameter block too large (32 KB on sm_70 and later)");
+static_assert(sizeof(OzPackBatch<OZ_MAXP>) < 32000, "kernel parameter block too large");
 static_assert(bf16_idesc(128, 64) == ((1u << 4) | (1u << 7) | (1u << 10) | (8u << 17) | (8u << 24)), "idesc");
+
+namespace {
+constexpr int WS_DEVICES = 64;
+std::mutex ws_mutex;
+cudaMemPool_t ws_pools[WS_DEVICES] = {};
+cudaMemPool_t ws_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= WS_DEVICES) return nullptr;
+  std::lock_guard<std::mutex> lock(ws_mutex);
+  if (!ws_pools[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    unsigned long long keep = 128ull << 20;
+    cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+    ws_pools[dev] = p;
+  }
+  return ws_pools[dev];
+}
+}  // namespace
+
+cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s) {
+  cudaMemPool_t pool = ws_pool();
+  return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+}
+
+void ws_trim() {
+  if (cudaMemPool_t pool = ws_pool()) cudaMemPoolTrimTo(pool, 0);
+  cudaGetLastError();
+}
 
 size_t oz_workspace_bytes(int M, int N, int K, bool gram) {
   if (M <= 0 || N <= 0 || K <= 0) return 0;
@@ -679,22 +725,26 @@ int oz_gemm_pooled(std::vector<OzProb>& probs, void* pool, size_t bytes, int* st
   return launches + oz_gemm_launch(group, status, s);
 }
 
-int oz_gemm_launch(const std::vector<OzProb>& probs, int* status, cudaStream_t s) {
+namespace {
+template <int CAP>
+int launch_all(const std::vector<OzProb>& probs, int* status, cudaStream_t s) {
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
+    cudaFuncSetAttribute(k_oz_gemm<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
     attr = true;
   }
   int launches = 0;
   size_t i0 = 0;
   while (i0 < probs.size()) {
-    const size_t i1 = std::min(probs.size(), i0 + (size_t)OZ_MAXP);
+    const size_t i1 = std::min(probs.size(), i0 + (size_t)CAP);
     // row exponents and digits of every operand
-    OzPackBatch eb{}, pk{};
-    OzGemmBatch gb{};
+    OzPackBatch<CAP> eb, pk;
+    eb.njob = pk.njob = 0;
+    OzGemmBatch<CAP> gb;
+    gb.nprob = 0;
     gb.status = status;
     int eblocks = 0, pblocks = 0, tiles = 0;
-    auto add_job = [&](OzPackBatch& b, int& blocks, const OzPackJob& J, int per_job_blocks) {
+    auto add_job = [&](OzPackBatch<CAP>& b, int& blocks, const OzPackJob& J, int per_job_blocks) {
       b.job[b.njob] = J;
       b.block_start[b.njob] = blocks;
       blocks += per_job_blocks;
@@ -732,6 +782,7 @@ int oz_gemm_launch(const std::vector<OzProb>& probs, int* status, cudaStream_t s
         add_job(pk, pblocks, jb, g.nrbB * g.nkt);
       }
       OzTile& t = gb.p[gb.nprob];
+      t = OzTile{};
       t.DA = DA; t.D1 = gram ? DA : D1; t.D2 = D2; t.eA = eA; t.eB = eB;
       t.C = p.C; t.Creal = p.Creal; t.ldc = p.ldc; t.alpha = p.alpha; t.s_row = p.s_row; t.s_col = p.s_col;
       t.row_div = std::max(1, p.row_div); t.col_div = std::max(1, p.col_div);
@@ -753,16 +804,21 @@ int oz_gemm_launch(const std::vector<OzProb>& probs, int* status, cudaStream_t s
     gb.tile_start[gb.nprob] = tiles;
     if (tiles > 0) {
       if (eblocks > 0) {
-        k_oz_exp<<<eblocks, 256, 0, s>>>(eb);
+        k_oz_exp<CAP><<<eblocks, 256, 0, s>>>(eb);
         ++launches;
       }
-      k_oz_pack<<<pblocks, 256, 0, s>>>(pk);
-      k_oz_gemm<<<tiles, OZ_NT, OZ_SMEM, s>>>(gb);
+      k_oz_pack<CAP><<<pblocks, 256, 0, s>>>(pk);
+      k_oz_gemm<CAP><<<tiles, OZ_NT, OZ_SMEM, s>>>(gb);
       launches += 2;
     }
     i0 = i1;
   }
   return launches;
+}
+}  // namespace
+
+int oz_gemm_launch(const std::vector<OzProb>& probs, int* status, cudaStream_t s) {
+  return probs.size() <= (size_t)FEW_MAXP ? launch_all<FEW_MAXP>(probs, status, s) : launch_all<OZ_MAXP>(probs, status, s);
 }
 
 }  // namespace ptebd

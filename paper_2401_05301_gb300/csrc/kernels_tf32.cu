@@ -184,14 +184,44 @@ struct TfPackJob {
   size_t plane;    // bytes of a plane
   int rows, K, per, b, conj, nrb, nkt;
 };
+template <int CAP>
 struct TfPackBatch {
-  TfPackJob job[2 * TC_MAXP];
-  int block_start[2 * TC_MAXP + 1];
+  TfPackJob job[2 * CAP];
+  int block_start[2 * CAP + 1];
   int njob;
 };
 
+// Element (local row r, local k q) of packed block (rb, kt) of A into the two planes.
+__device__ __forceinline__ void put_a(const TfPackJob& J, int gr, int gk, uint8_t* hi_p, uint8_t* lo_p, uint32_t at) {
+  double2 v = make_double2(0.0, 0.0);
+  if (gr < J.rows && gk < J.K) v = __ldg(J.X + (long long)gr * J.rs + gk);
+  uint32_t h0, l0, h1, l1;
+  split_tf32(v.x, h0, l0);
+  split_tf32(v.y, h1, l1);
+  *reinterpret_cast<uint2*>(hi_p + at) = make_uint2(h0, h1);  // an even k: both words in one 8-byte slot
+  *reinterpret_cast<uint2*>(lo_p + at) = make_uint2(l0, l1);
+}
+// Column gj, element gk of op(B): rows 2 jj and 2 jj + 1 of the block, words 2 q and 2 q + 1.
+__device__ __forceinline__ void put_b(const TfPackJob& J, int gj, int gk, uint8_t* hi_p, uint8_t* lo_p, int jj, int q) {
+  double2 v = make_double2(0.0, 0.0);
+  if (gj < J.rows && gk < J.K) {
+    v = __ldg(J.X + (long long)(gj / J.per) * J.sb + (long long)(gj % J.per) * J.rs + (long long)gk * J.ks);
+    if (J.conj) v.y = -v.y;
+  }
+  uint32_t hr, lr, hm, lm;
+  split_tf32(v.x, hr, lr);
+  split_tf32(v.y, hm, lm);
+  const uint32_t sign = 0x80000000u;
+  const uint32_t a0 = swz(2 * jj, 2 * q), a1 = swz(2 * jj + 1, 2 * q);
+  *reinterpret_cast<uint2*>(hi_p + a0) = make_uint2(hr, hm ^ (hm ? sign : 0u));
+  *reinterpret_cast<uint2*>(lo_p + a0) = make_uint2(lr, lm ^ (lm ? sign : 0u));
+  *reinterpret_cast<uint2*>(hi_p + a1) = make_uint2(hm, hr);
+  *reinterpret_cast<uint2*>(lo_p + a1) = make_uint2(lm, lr);
+}
+
 // One block per packed block: 32 rows x 16 complex (A) or 16 columns x 16 complex (B).
-__global__ void __launch_bounds__(256) k_tf_pack(const __grid_constant__ TfPackBatch pb) {
+template <int CAP>
+__global__ void __launch_bounds__(256) k_tf_pack(const __grid_constant__ TfPackBatch<CAP> pb) {
   int j = 0;
   for (int hi = pb.njob - 1; j < hi;) {
     const int mid = (j + hi + 1) >> 1;
@@ -205,36 +235,28 @@ __global__ void __launch_bounds__(256) k_tf_pack(const __grid_constant__ TfPackB
   if (!J.b) {
     for (int idx = threadIdx.x; idx < 32 * 16; idx += 256) {
       const int r = idx >> 4, q = idx & 15;
-      const int gr = rb * 32 + r, gk = kt * 16 + q;
-      double2 v = make_double2(0.0, 0.0);
-      if (gr < J.rows && gk < J.K) v = __ldg(J.X + (long long)gr * J.rs + gk);
-      uint32_t h0, l0, h1, l1;
-      split_tf32(v.x, h0, l0);
-      split_tf32(v.y, h1, l1);
-      const uint32_t at = swz(r, 2 * q);  // an even k: both words in one 8-byte slot
-      *reinterpret_cast<uint2*>(hi_p + at) = make_uint2(h0, h1);
-      *reinterpret_cast<uint2*>(lo_p + at) = make_uint2(l0, l1);
+      put_a(J, rb * 32 + r, kt * 16 + q, hi_p, lo_p, swz(r, 2 * q));
     }
-    return;
+  } else {
+    const bool k_first = J.ks == 1;  // lanes along the contiguous index
+    const int q = k_first ? threadIdx.x & 15 : threadIdx.x >> 4, jj = k_first ? threadIdx.x >> 4 : threadIdx.x & 15;
+    put_b(J, rb * 16 + jj, kt * 16 + q, hi_p, lo_p, jj, q);
   }
-  {
-    int jj, q;
-    if (J.ks == 1) { q = threadIdx.x & 15; jj = threadIdx.x >> 4; } else { jj = threadIdx.x & 15; q = threadIdx.x >> 4; }
-    const int gj = rb * 16 + jj, gk = kt * 16 + q;
-    double2 v = make_double2(0.0, 0.0);
-    if (gj < J.rows && gk < J.K) {
-      v = __ldg(J.X + (long long)(gj / J.per) * J.sb + (long long)(gj % J.per) * J.rs + (long long)gk * J.ks);
-      if (J.conj) v.y = -v.y;
+}
+
+// A direct tile's slabs (at most STAGES) by the drain warps themselves.
+__device__ void fill_direct(const TfPackJob& A, const TfPackJob& B, int mt, int nt, int nk, uint8_t* smem) {
+  for (int kt = 0; kt < nk; ++kt) {
+    uint8_t* st = smem + kt * STAGE_BYTES;
+    for (int idx = threadIdx.x; idx < TM * 16; idx += 32 * DW) {
+      const int r = idx >> 4, q = idx & 15;
+      put_a(A, mt * TM + r, kt * 16 + q, st, st + A_BYTES, swz(r, 2 * q));
     }
-    uint32_t hr, lr, hm, lm;
-    split_tf32(v.x, hr, lr);
-    split_tf32(v.y, hm, lm);
-    const uint32_t sign = 0x80000000u;
-    const uint32_t a0 = swz(2 * jj, 2 * q), a1 = swz(2 * jj + 1, 2 * q);
-    *reinterpret_cast<uint2*>(hi_p + a0) = make_uint2(hr, hm ^ (hm ? sign : 0u));
-    *reinterpret_cast<uint2*>(lo_p + a0) = make_uint2(lr, lm ^ (lm ? sign : 0u));
-    *reinterpret_cast<uint2*>(hi_p + a1) = make_uint2(hm, hr);
-    *reinterpret_cast<uint2*>(lo_p + a1) = make_uint2(lm, lr);
+    for (int idx = threadIdx.x; idx < (TN / 2) * 16; idx += 32 * DW) {
+      const bool k_first = B.ks == 1;
+      const int q = k_first ? idx & 15 : idx / (TN / 2), jj = k_first ? idx >> 4 : idx % (TN / 2);
+      put_b(B, nt * (TN / 2) + jj, kt * 16 + q, st + 2 * A_BYTES, st + 2 * A_BYTES + B_BYTES, jj, q);
+    }
   }
 }
 
@@ -248,10 +270,13 @@ struct TfTile {
   long long ldc, sC;
   double alpha;
   int M, N, per, nkt, nrbA, nrbB, tiles_n;
+  TfPackJob da, db;   // direct: the operands, cut by the CTA itself (no planes)
+  int direct;
 };
+template <int CAP>
 struct TfBatch {
-  TfTile p[TC_MAXP];
-  int tile_start[TC_MAXP + 1];
+  TfTile p[CAP];
+  int tile_start[CAP + 1];
   int nprob;
   int* status;
 };
@@ -263,7 +288,8 @@ __device__ __forceinline__ double widen(float f) {
   return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(b << 29));
 }
 
-__global__ void __launch_bounds__(NT, 1) k_tf32x3(const __grid_constant__ TfBatch gb) {
+template <int CAP>
+__global__ void __launch_bounds__(NT, 1) k_tf32x3(const __grid_constant__ TfBatch<CAP> gb) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
@@ -304,7 +330,7 @@ __global__ void __launch_bounds__(NT, 1) k_tf32x3(const __grid_constant__ TfBatc
 
   if (warp == DW) {
     // ---- copies: the four planes of a slab
-    if (lane == 0) {
+    if (lane == 0 && !P.direct) {
       int issued = 0;
       bool ok = true;
       for (int kt = 0; kt < nk; ++kt) {
@@ -358,6 +384,13 @@ __global__ void __launch_bounds__(NT, 1) k_tf32x3(const __grid_constant__ TfBatc
     // ---- drain: warp (g, h) owns TMEM lanes 32g.. and columns 64h.. of every accumulator, which it adds
     // into FP32 registers with round-to-nearest adds, k-step by k-step
     const int g = warp & 3, h = warp >> 2;
+    if (P.direct) {
+      fill_direct(P.da, P.db, mt, nt, nk, smem);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("bar.sync 1, %0;" ::"r"(32 * DW) : "memory");
+      if (threadIdx.x == 0)
+        for (int kt = 0; kt < nk; ++kt) mbar_arrive(&full[kt]);
+    }
     float acc[64];
 #pragma unroll
     for (int i = 0; i < 64; ++i) acc[i] = 0.0f;
@@ -393,7 +426,18 @@ __global__ void __launch_bounds__(NT, 1) k_tf32x3(const __grid_constant__ TfBatc
         : "=r"(any_bad)
         : "r"(ok ? 0 : 1), "r"(32 * DW)
         : "memory");
-    if (!any_bad) {
+    if (!any_bad && P.direct) {  // few rows: straight from the registers
+      const int row = mt * TM + 32 * g + lane;
+      if (row < P.M) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          const int jj = nt * (TN / 2) + 32 * h + i;
+          if (jj < P.N)
+            P.C[(long long)(jj / P.per) * P.sC + (long long)row * P.ldc + jj % P.per] =
+                make_double2(widen(acc[2 * i]) * P.alpha, widen(acc[2 * i + 1]) * P.alpha);
+        }
+      }
+    } else if (!any_bad) {
       double2* out = reinterpret_cast<double2*>(smem);
       double2* mine = out + (size_t)(32 * g + lane) * OUT_LD + 32 * h;
       const double al = P.alpha;
@@ -405,10 +449,12 @@ __global__ void __launch_bounds__(NT, 1) k_tf32x3(const __grid_constant__ TfBatc
         for (int i = 0; i < 32; ++i) mine[i] = make_double2(widen(acc[2 * i]) * al, widen(acc[2 * i + 1]) * al);
       }
       asm volatile("bar.sync 1, %0;" ::"r"(32 * DW) : "memory");
-      for (int e = threadIdx.x; e < TM * (TN / 2); e += 32 * DW) {
-        const int r = e / (TN / 2), cc = e - r * (TN / 2);
-        const int i = mt * TM + r, jj = nt * (TN / 2) + cc;
-        if (i < P.M && jj < P.N) P.C[(long long)(jj / P.per) * P.sC + (long long)i * P.ldc + jj % P.per] = out[(size_t)r * OUT_LD + cc];
+      const int cc = threadIdx.x & (TN / 2 - 1), jj = nt * (TN / 2) + cc;  // a thread keeps its column
+      if (jj < P.N) {
+        double2* dst = P.C + (long long)(jj / P.per) * P.sC + jj % P.per;
+        const int rows = min(TM, P.M - mt * TM);
+        for (int r = threadIdx.x / (TN / 2); r < rows; r += 32 * DW / (TN / 2))
+          dst[(long long)(mt * TM + r) * P.ldc] = out[(size_t)r * OUT_LD + cc];
       }
     }
   }
@@ -436,28 +482,42 @@ Geo geometry(int M, long long N, int K) {
 
 }  // namespace
 
-static_assert(sizeof(TfBatch) < 32000 && sizeof(TfPackBatch) < 32000, "kernel parameter block too large (32 KB on sm_70 and later)");
+static_assert(sizeof(TfBatch<TC_MAXP>) < 32000 && sizeof(TfPackBatch<TC_MAXP>) < 32000, "kernel parameter block too large (32 KB on sm_70 and later)");
 static_assert(tf32_idesc(128, 128) == ((1u << 4) | (2u << 7) | (2u << 10) | (16u << 17) | (8u << 24)), "idesc");
+
+namespace {
+// One slab and one wave of tiles: each CTA cuts its own operands, which is cheaper than a launch and a
+// workspace for the planes (32 x 16 x 16 complex 15 us a call against 24 with planes; with two slabs,
+// 250 x 100 x 30, 31 against 24).
+bool tc_direct(int M, long long N, int K) {
+  return K <= 16 && (long long)((M + TM - 1) / TM) * ((N + TN / 2 - 1) / (TN / 2)) <= 152;
+}
+}  // namespace
 
 size_t tc_workspace_bytes(int M, int N, int K, int batch) {
   if (M <= 0 || N <= 0 || K <= 0 || batch <= 0) return 0;
+  if (tc_direct(M, (long long)N * batch, K)) return 0;
   const Geo g = geometry(M, (long long)N * batch, K);
   return 2 * (g.planeA + g.planeB);
 }
 
-int tc_gemm_launch(const std::vector<TcGemmProb>& probs, int* status, cudaStream_t s) {
+namespace {
+template <int CAP>
+int launch_all(const std::vector<TcGemmProb>& probs, int* status, cudaStream_t s) {
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_tf32x3, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    cudaFuncSetAttribute(k_tf32x3<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     attr = true;
   }
   int launches = 0;
   for (size_t i = 0; i < probs.size();) {
-    TfBatch gb{};
-    TfPackBatch pk{};
+    TfBatch<CAP> gb;
+    gb.nprob = 0;
+    TfPackBatch<CAP> pk;
+    pk.njob = 0;
     gb.status = status;
     int tiles = 0, blocks = 0;
-    for (; i < probs.size() && gb.nprob < TC_MAXP; ++i) {
+    for (; i < probs.size() && gb.nprob < CAP; ++i) {
       const TcGemmProb& p = probs[i];
       if (p.M <= 0 || p.N <= 0 || p.batch <= 0) continue;
       // the columns of all batch entries side by side: A is shared (sA = 0) or there is one entry
@@ -469,11 +529,20 @@ int tc_gemm_launch(const std::vector<TcGemmProb>& probs, int* status, cudaStream
         pk.block_start[pk.njob++] = blocks;
         blocks += J.nrb * J.nkt;
       };
-      job(TfPackJob{p.A, p.lda, 1, 0, ws, g.planeA, p.M, p.K, 1, 0, 0, g.nrbA, g.nkt});
       const bool c = p.opB == OP_C;
-      job(TfPackJob{p.B, c ? p.ldb : 1, c ? 1 : p.ldb, p.sB, ws + 2 * g.planeA, g.planeB, N, p.K, p.N, 1, c ? 1 : 0,
-                    g.nrbB, g.nkt});
+      const TfPackJob ja{p.A, p.lda, 1, 0, ws, g.planeA, p.M, p.K, 1, 0, 0, g.nrbA, g.nkt};
+      const TfPackJob jb{p.B, c ? p.ldb : 1, c ? 1 : p.ldb, p.sB, ws + 2 * g.planeA, g.planeB, N, p.K, p.N, 1,
+                         c ? 1 : 0, g.nrbB, g.nkt};
       TfTile& t = gb.p[gb.nprob];
+      t = TfTile{};
+      t.direct = tc_direct(p.M, N, p.K);
+      if (t.direct) {
+        t.da = ja;
+        t.db = jb;
+      } else {
+        job(ja);
+        job(jb);
+      }
       t.A = ws; t.B = ws + 2 * g.planeA; t.planeA = g.planeA; t.planeB = g.planeB;
       t.C = p.C; t.ldc = p.ldc; t.sC = p.sC; t.alpha = p.alpha; t.M = p.M; t.N = N; t.per = p.N;
       t.nkt = g.nkt; t.nrbA = g.nrbA; t.nrbB = g.nrbB; t.tiles_n = g.nrbB / 4;
@@ -484,13 +553,18 @@ int tc_gemm_launch(const std::vector<TcGemmProb>& probs, int* status, cudaStream
     pk.block_start[pk.njob] = blocks;
     if (tiles == 0) continue;
     if (blocks > 0) {
-      k_tf_pack<<<blocks, 256, 0, s>>>(pk);
+      k_tf_pack<CAP><<<blocks, 256, 0, s>>>(pk);
       ++launches;
     }
-    k_tf32x3<<<tiles, NT, SMEM_BYTES, s>>>(gb);
+    k_tf32x3<CAP><<<tiles, NT, SMEM_BYTES, s>>>(gb);
     ++launches;
   }
   return launches;
+}
+}  // namespace
+
+int tc_gemm_launch(const std::vector<TcGemmProb>& probs, int* status, cudaStream_t s) {
+  return probs.size() <= (size_t)FEW_MAXP ? launch_all<FEW_MAXP>(probs, status, s) : launch_all<TC_MAXP>(probs, status, s);
 }
 
 int tc_gemm_pooled(std::vector<TcGemmProb>& probs, void* pool, size_t bytes, int* status, cudaStream_t s) {

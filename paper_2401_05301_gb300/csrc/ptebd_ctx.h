@@ -168,7 +168,11 @@ T* dalloc(tebd_ctx* c, size_t count) {
   if (count == 0) count = 1;
   if (cudaMalloc(&p, count * sizeof(T)) != cudaSuccess) {
     cudaGetLastError();
-    return nullptr;
+    ws_trim();
+    if (cudaMalloc(&p, count * sizeof(T)) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
   }
   c->allocs.push_back(p);
   c->alloc_bytes += count * sizeof(T);

@@ -48,10 +48,14 @@ struct GemmProb {
   int split;  // CTAs of a cluster that share a tile's reduction (set by the launch)
 };
 
+// Launches of few problems take a small parameter block: filling and sending 12 to 30 KB costs the host
+// 1 to 3 us a launch.
+constexpr int FEW_MAXP = 4;
+template <int CAP>
 struct GemmBatch {
-  GemmProb p[GEMM_MAXP];
-  int tile_start[GEMM_MAXP + 1];
-  int nprob, opA, opB;
+  GemmProb p[CAP];
+  int tile_start[CAP + 1];
+  int nprob;
 };
 
 // ---- complex GEMM as split 3xTF32 on tcgen05 tensor cores (kernels_tf32.cu) ------
@@ -109,9 +113,10 @@ struct OzPackJob {
   int own_exp;  // the packing blocks find the row exponents themselves
   int* e;  // row exponents [nrb * 32]
 };
+template <int CAP>
 struct OzPackBatch {
-  OzPackJob job[2 * OZ_MAXP];
-  int block_start[2 * OZ_MAXP + 1];
+  OzPackJob job[2 * CAP];
+  int block_start[2 * CAP + 1];
   int njob;
 };
 struct OzTile {
@@ -128,9 +133,10 @@ struct OzTile {
   const double* s_col;
   int row_div, col_div, M, N, nkt, nrbA, nrbB, herm, tiles_n, beta;
 };
+template <int CAP>
 struct OzGemmBatch {
-  OzTile p[OZ_MAXP];
-  int tile_start[OZ_MAXP + 1];
+  OzTile p[CAP];
+  int tile_start[CAP + 1];
   int nprob;
   int* status;  // set to TEBD_ERR_TIMEOUT if a bounded wait runs out
 };
@@ -139,6 +145,13 @@ int oz_gemm_launch(const std::vector<OzProb>& probs, int* status, cudaStream_t s
 // The same with the digit workspaces taken from one pool (bytes >= the largest problem's need): as many
 // problems share a launch as the pool holds, at most OZ_MAXP.
 int oz_gemm_pooled(std::vector<OzProb>& probs, void* pool, size_t bytes, int* status, cudaStream_t s);
+
+// Workspace of a product without a handle (tebd_zgemm), stream-ordered, freed with cudaFreeAsync.  It comes
+// from a memory pool of the device that keeps at most 128 MB between calls (the default pool gives
+// everything back at each synchronisation: 200 us a call); ws_trim gives that back too, when an
+// allocation of a handle fails.
+cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s);
+void ws_trim();
 
 class Gemm {
  public:

@@ -731,8 +731,7 @@ int run_prods(tebd_ctx* c, const std::vector<Prod>& ps, int engine) {
       tp.push_back(TcGemmProb{p.A, p.B, p.C, p.lda, p.ldb, p.ldc, 0, 0, p.alpha, p.M, p.N, p.K, 1, p.opB, nullptr});
       need = std::max(need, tc_workspace_bytes(p.M, p.N, p.K, 1));
     }
-    if (need == 0) return TEBD_OK;
-    if (int r = ensure_pool(c, need)) return r;
+    if (int r = ensure_pool(c, std::max<size_t>(need, 256))) return r;
     c->launches += tc_gemm_pooled(tp, c->u1w->pool, c->u1w->pool_bytes, c->d_status, c->stream);
     return check_launch(c);
   }
