@@ -1077,20 +1077,25 @@ int graph_step(tebd_ctx* c, const std::vector<tebd_ctx*>& hs, const std::vector<
 }
 
 int ensure_measure_ws(tebd_ctx* c) {
-  if (!c->mN) {  // super sites: two physical densities per site, 2L - 1 physical bonds
-    c->mC = dalloc<double2>(c, c->ss ? 2 * c->L : c->L);
-    c->mN = dalloc<double>(c, c->ss ? 2 * c->L : c->L);
+  if (!c->mN) {  // super sites: two physical densities per site, 2L - 1 physical bonds; then partial sums
+    const size_t n = c->ss ? 2 * (size_t)c->L : (size_t)c->L;
+    c->mC = dalloc<double2>(c, n + MEAS_CHUNK * TRACE_PARTS);
+    c->mN = dalloc<double>(c, n * (1 + DENSITY_PARTS));
     if (!c->mC || !c->mN) return TEBD_ERR_OOM;
   }
   if (c->u1 && c->have_charges) return TEBD_OK;  // the blocked correlators use their own arena
-  if (!c->mP) {
+  if (!c->mX) {
     const long long capmax = std::max<long long>(1, *std::max_element(c->cap.begin(), c->cap.end()));
     const long long big = capmax * c->d * capmax;
-    c->mP = dalloc<double2>(c, MEAS_CHUNK * big);
-    c->mQ = dalloc<double2>(c, MEAS_CHUNK * big);
-    c->mX = dalloc<double2>(c, MEAS_CHUNK * capmax * capmax);
+    if (c->ss) {  // super sites shift one position of a pair: the shifted factors are formed
+      c->mP = dalloc<double2>(c, MEAS_CHUNK * big);
+      c->mQ = dalloc<double2>(c, MEAS_CHUNK * big);
+    } else {      // weights of the products' reductions
+      c->mW = dalloc<double>(c, MEAS_CHUNK * (capmax + 1) * (c->d - 1));
+    }
     c->mY = dalloc<double2>(c, MEAS_CHUNK * capmax * capmax);
-    if (!c->mP || !c->mQ || !c->mX || !c->mY) return TEBD_ERR_OOM;
+    c->mX = dalloc<double2>(c, MEAS_CHUNK * capmax * capmax);
+    if ((c->ss ? !c->mP || !c->mQ : !c->mW) || !c->mX || !c->mY) return TEBD_ERR_OOM;
   }
   return TEBD_OK;
 }
@@ -1542,7 +1547,8 @@ int tebd_estimate_bytes(int L, int n_max, int chi_max, int max_slots, int precis
   int slots = std::min(max_triples_per_layer(L), MAX_SLOTS);
   if (max_slots > 0) slots = std::min(slots, max_slots);
   b += slots * slot_bytes_for(capmax, d, chi_max, precision);
-  b += 16.0 * MEAS_CHUNK * (2.0 * capmax * d * capmax + 2.0 * capmax * capmax) + 24.0 * L;  // measurement
+  b += MEAS_CHUNK * (32.0 * capmax * capmax + 8.0 * (capmax + 1) * (d - 1) + 16.0 * TRACE_PARTS) +
+       (24.0 + 8.0 * DENSITY_PARTS) * L;  // measurement
   *bytes = b;
   return TEBD_OK;
 }
@@ -1636,7 +1642,7 @@ int measure_supersite(tebd_ctx* h, double* n_out, double* cur_out) {
   for (int k = 0; k < L; ++k)
     for (int pos = 0; pos < 2; ++pos)
       da[2 * k + pos] = DensityArgs{h->B[k], h->lam[k], h->mN + 2 * k + pos, h->chi[k], d, h->chi[k + 1], 1 + pos, dp};
-  h->launches += launch_densities(da.data(), Lp, h->stream);
+  h->launches += launch_densities(da.data(), Lp, h->mN + Lp, h->stream);
   for (int k = 0; k < L; ++k)
     h->launches += launch_pair_hop(h->B[k], h->lam[k], h->chi[k], d, h->chi[k + 1], dp, h->mC + 2 * k, h->stream);
   const long long capmax = std::max<long long>(1, *std::max_element(h->cap.begin(), h->cap.end()));
@@ -1657,11 +1663,12 @@ int measure_supersite(tebd_ctx* h, double* n_out, double* cur_out) {
     }
     h->launches += gx.launch(h->stream);
     h->launches += gy.launch(h->stream);
+    std::vector<TraceArgs> tr;
     for (int k = k0; k < k1; ++k) {
       const int q = k - k0;
-      h->launches += launch_trace_product(h->mX + q * capmax * capmax, h->mY + q * capmax * capmax, h->chi[k + 1],
-                                          h->mC + 2 * k + 1, h->stream);
+      tr.push_back(TraceArgs{h->mX + q * capmax * capmax, h->mY + q * capmax * capmax, h->mC + 2 * k + 1, h->chi[k + 1]});
     }
+    h->launches += launch_trace_products(tr.data(), (int)tr.size(), h->mC + Lp, h->stream);
   }
   if (int r = check_launch(h)) return r;
   if (int r = ensure_pinned(h, 3 * (size_t)Lp + 8)) return r;
@@ -1690,9 +1697,8 @@ int tebd_measure(tebd_handle h, double* n_out, double* cur_out) {
     ProfScope ps(h, TEBD_PROF_MEASURE, mbytes);
     std::vector<DensityArgs> da(L);
     for (int k = 0; k < L; ++k) da[k] = DensityArgs{h->B[k], h->lam[k], h->mN + k, h->chi[k], d, h->chi[k + 1]};
-    h->launches += launch_densities(da.data(), L, h->stream);
+    h->launches += launch_densities(da.data(), L, h->mN + L, h->stream);
     const long long capmax = std::max<long long>(1, *std::max_element(h->cap.begin(), h->cap.end()));
-    const long long big = capmax * d * capmax;
     if (h->u1 && h->have_charges) {  // the correlators from the charge blocks
       if (!h->u1w)
         if (int r = u1_alloc_slots(h, 0)) return r;
@@ -1700,24 +1706,30 @@ int tebd_measure(tebd_handle h, double* n_out, double* cur_out) {
     }
     for (int k0 = 0; k0 < (h->u1 && h->have_charges ? 0 : L - 1); k0 += MEAS_CHUNK) {
       const int k1 = std::min(L - 1, k0 + MEAS_CHUNK);
+      // C_k = sum_{c,c'} X[c,c'] Y[c',c]: the raised and lowered factors are the site tensors themselves, one
+      // value of s further, with lam_a^2 sqrt(s+1) and sqrt(t+1) along the reductions (s, t < d - 1)
       Gemm gx(true, OP_C, OP_N), gy(true, OP_N, OP_C);
+      std::vector<HopArgs> hop;
+      std::vector<TraceArgs> tr;
       for (int k = k0; k < k1; ++k) {
         const int q = k - k0;
         const int cl = h->chi[k], cm = h->chi[k + 1], cr = h->chi[k + 2];
-        double2* P = h->mP + q * big;
-        double2* Q = h->mQ + q * big;
-        h->launches += launch_shift_left(h->B[k], h->lam[k], P, cl, d, cm, h->stream);
-        h->launches += launch_shift_right(h->B[k + 1], Q, cm, d, cr, h->stream);
-        gx.add(cm, cm, cl * d, P, cm, h->B[k], cm, h->mX + q * capmax * capmax, cm);
-        gy.add(cm, cm, d * cr, Q, (long long)d * cr, h->B[k + 1], (long long)d * cr, h->mY + q * capmax * capmax, cm);
+        double* w = h->mW + q * (capmax + 1) * (d - 1);
+        double2 *X = h->mX + q * capmax * capmax, *Y = h->mY + q * capmax * capmax;
+        hop.push_back(HopArgs{h->lam[k], w, cl, d});
+        GemmProb& px = gx.add(cm, cm, cl * (d - 1), h->B[k] + cm, cm, h->B[k], cm, X, cm);
+        px.s_red = w;
+        px.red_grp = d - 1;
+        GemmProb& py = gy.add(cm, cm, (d - 1) * cr, h->B[k + 1] + cr, (long long)d * cr, h->B[k + 1], (long long)d * cr, Y,
+                              cm);
+        py.s_red = w + (size_t)cl * (d - 1);
+        py.red_div = cr;
+        tr.push_back(TraceArgs{X, Y, h->mC + k, cm});
       }
+      h->launches += launch_hop_weights(hop.data(), (int)hop.size(), h->stream);
       h->launches += gx.launch(h->stream);
       h->launches += gy.launch(h->stream);
-      for (int k = k0; k < k1; ++k) {
-        const int q = k - k0;
-        h->launches += launch_trace_product(h->mX + q * capmax * capmax, h->mY + q * capmax * capmax, h->chi[k + 1],
-                                            h->mC + k, h->stream);
-      }
+      h->launches += launch_trace_products(tr.data(), (int)tr.size(), h->mC + L, h->stream);
     }
     if (int r = check_launch(h)) return r;
     if (int r = ensure_pinned(h, 3 * (size_t)L + 8)) return r;

@@ -148,9 +148,10 @@ __global__ void __launch_bounds__(NT) gemm_kernel(const __grid_constant__ GemmBa
     T v = A_::zero();
     const int gi = m0 + ai, gk = k0 + ak;
     if (ai < mt && gk < ke) {
-      if (OPA == OP_N) v = A[(long long)gi * P.lda + gk];
-      else if (OPA == OP_C) v = A_::cj(A[(long long)gk * P.lda + gi]);
-      else v = A_::cj(A[(long long)gi * P.lda + gk]);
+      const int kr = P.red_grp > 0 ? gk + gk / P.red_grp : gk;
+      if (OPA == OP_N) v = A[(long long)gi * P.lda + kr];
+      else if (OPA == OP_C) v = A_::cj(A[(long long)kr * P.lda + gi]);
+      else v = A_::cj(A[(long long)gi * P.lda + kr]);
       if (P.s_red) v = A_::scale(v, P.s_red[gk / P.red_div]);
     }
     return v;
@@ -159,9 +160,10 @@ __global__ void __launch_bounds__(NT) gemm_kernel(const __grid_constant__ GemmBa
     T v = A_::zero();
     const int gj = n0 + bj, gk = k0 + bk;
     if (bj < nt && gk < ke) {
-      if (OPB == OP_N) v = B[(long long)gk * P.ldb + gj];
-      else if (OPB == OP_C) v = A_::cj(B[(long long)gj * P.ldb + gk]);
-      else v = A_::cj(B[(long long)gk * P.ldb + gj]);
+      const int kr = P.red_grp > 0 ? gk + gk / P.red_grp : gk;
+      if (OPB == OP_N) v = B[(long long)kr * P.ldb + gj];
+      else if (OPB == OP_C) v = A_::cj(B[(long long)gj * P.ldb + kr]);
+      else v = A_::cj(B[(long long)kr * P.ldb + gj]);
       if (P.s_red_b) v = A_::scale(v, P.s_red_b[gk / P.red_div]);
     }
     return v;

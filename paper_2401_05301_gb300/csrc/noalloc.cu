@@ -72,26 +72,29 @@ extern "C" int tebd_bond_correlator_noalloc(const double* B_left, const double* 
   const double2* Bl = reinterpret_cast<const double2*>(B_left);
   const double2* Br = reinterpret_cast<const double2*>(B_right);
   // Every scratch element read below is first written by this call, so the
-  // contents left by an earlier call never leak into the result.
-  double2* P = scratch;                       // [chi_l * d][chi_m]
-  double2* Q = scratch + NA_BIG;              // [chi_m][d * chi_r]
-  double2* X = scratch + 2 * NA_BIG;          // [chi_m][chi_m]
+  // contents left by an earlier call never leak into the result.  The shifted factors b+ B and b B are
+  // read in place (a row or a column block further) with weights along the reduction.
+  double* w = reinterpret_cast<double*>(scratch);  // chi_l (d - 1) weights, then sqrt(1 .. d - 1)
+  double2* X = scratch + 2 * NA_BIG;               // [chi_m][chi_m]
   double2* Yt = scratch + 2 * NA_BIG + NA_SMALL;
-  launch_shift_left(Bl, lam_left, P, chi_l, d, chi_m, s);
-  launch_shift_right(Br, Q, chi_m, d, chi_r, s);
+  const HopArgs hop{lam_left, w, chi_l, d};
+  launch_hop_weights(&hop, 1, s);
   GemmProb px{};
-  px.A = P; px.B = Bl; px.C = X;
+  px.A = Bl + chi_m; px.B = Bl; px.C = X;
   px.lda = chi_m; px.ldb = chi_m; px.ldc = chi_m;
-  px.M = chi_m; px.N = chi_m; px.K = chi_l * d; px.batch = 1;
+  px.M = chi_m; px.N = chi_m; px.K = chi_l * (d - 1); px.batch = 1;
+  px.s_red = w; px.red_grp = d - 1;
   px.red_div = px.row_div = px.col_div = 1;
   px.alpha_re = 1.0;
   gemm_launch_single(true, OP_C, OP_N, px, s);
   GemmProb py = px;
-  py.A = Q; py.B = Br; py.C = Yt;
+  py.A = Br + chi_r; py.B = Br; py.C = Yt;
   py.lda = (long long)d * chi_r; py.ldb = (long long)d * chi_r; py.ldc = chi_m;
-  py.K = d * chi_r;
+  py.K = (d - 1) * chi_r;
+  py.s_red = w + (size_t)chi_l * (d - 1); py.red_div = chi_r; py.red_grp = 0;
   gemm_launch_single(true, OP_N, OP_C, py, s);
-  launch_trace_product(X, Yt, chi_m, reinterpret_cast<double2*>(C_out), s);
+  const TraceArgs tr{X, Yt, reinterpret_cast<double2*>(C_out), chi_m};
+  launch_trace_products(&tr, 1, nullptr, s);
   // only this call's launches can have set the error read here
   if (cudaGetLastError() != cudaSuccess) return TEBD_ERR_CUDA;
   return TEBD_OK;

@@ -73,7 +73,7 @@ struct tebd_ctx {
   double* h_pinned = nullptr;
   size_t h_pinned_n = 0;
   double2 *mP = nullptr, *mQ = nullptr, *mX = nullptr, *mY = nullptr, *mC = nullptr;
-  double* mN = nullptr;
+  double *mN = nullptr, *mW = nullptr;
   double w_total = 0.0;
   long long steps = 0, gate_updates = 0, launches = 0;
   std::vector<void*> allocs;

@@ -45,6 +45,7 @@ struct GemmProb {
   int red_div, row_div, col_div, accumulate;
   int herm;  // result is Hermitian (M == N, B = A^+): only lower tiles are computed, then mirrored
   const double* s_red_b;  // optional factor of B along the reduction index (red_div as s_red)
+  int red_grp;  // > 0: reduction index k stands for row k + k / red_grp of both operands (one row in red_grp + 1 is left out)
   int split;  // CTAs of a cluster that share a tile's reduction (set by the launch)
 };
 
@@ -288,13 +289,17 @@ struct DensityArgs {
   int chl, d, chr;
   int wmode, wd;  // occupation of local state s: s (0), s / wd (1, first site of a pair), s % wd (2)
 };
-int launch_densities(const DensityArgs* a, int n, cudaStream_t s);
+constexpr int DENSITY_PARTS = 32;  // partial sums per density (part: n * DENSITY_PARTS doubles)
+int launch_densities(const DensityArgs* a, int n, double* part, cudaStream_t s);
 
-// P'[(a,s),c] = lam_a^2 sqrt(s+1) B[a,s+1,c] (s < d-1), 0 for s = d-1
-int launch_shift_left(const double2* B, const double* lam, double2* out, int chl, int d, int chr,
-                      cudaStream_t s);
-// Q'[c,(t,b)] = sqrt(t+1) B[c,t+1,b] (t < d-1), 0 for t = d-1
-int launch_shift_right(const double2* B, double2* out, int chl, int d, int chr, cudaStream_t s);
+// Weights of a bond's correlator products: w[a (d-1) + s] = lam_a^2 sqrt(s+1) for the left one,
+// sq[t] = sqrt(t+1) for the right one (s, t < d - 1).
+struct HopArgs {
+  const double* lam;
+  double* w;   // chl (d - 1), then sq (d - 1)
+  int chl, d;
+};
+int launch_hop_weights(const HopArgs* a, int n, cudaStream_t s);
 // out[(a,s),c] = f lam_a^2 sqrt(w(s)+1) B[a, s+shift, c] where w(s) < wd - 1, else 0, with
 // w(s) = s % wd (mode 1) or s / wd (mode 2); f = 1 and lam optional (NULL: no lam^2).  The
 // raising operator of one site of a super site (pairs of sites, sigma = s_a wd + s_b).
@@ -303,8 +308,15 @@ int launch_shift_pair(const double2* B, const double* lam, double2* out, int chl
 // out = sum_{a,b} lam_a^2 sum_sigma' sqrt(s'_a + 1) sqrt(s'_b) conj(B[a, sigma' + wd - 1, b]) B[a, sigma', b]
 // over s'_a < wd - 1, s'_b >= 1: <b+_(2k-1) b_(2k)> inside super site k.
 int launch_pair_hop(const double2* B, const double* lam, int chl, int d, int chr, int wd, double2* out, cudaStream_t s);
-// out = sum_{c,c'} X[c,c'] Yt[c',c]
-int launch_trace_product(const double2* X, const double2* Yt, int chi, double2* out, cudaStream_t s);
+// out = sum_{c,c'} X[c,c'] Yt[c',c].  part: TRACE_PARTS complex per product, or null (one block each).
+constexpr int TRACE_PARTS = 32;
+struct TraceArgs {
+  const double2* X;
+  const double2* Yt;
+  double2* out;
+  int chi;
+};
+int launch_trace_products(const TraceArgs* a, int n, double2* part, cudaStream_t s);
 
 int launch_check_finite(const double* x, int n, int* status, cudaStream_t s);
 

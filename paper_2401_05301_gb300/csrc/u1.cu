@@ -24,6 +24,7 @@
 // is applied once to the merged spectrum of all blocks of a cut (ties: block
 // order, then index), and the kept vectors are ordered by charge.
 #include "ptebd_ctx.h"
+#include "truncation.cuh"
 
 #include <algorithm>
 #include <cfloat>
@@ -162,6 +163,25 @@ __device__ void bitonic(double* s, int* key, int P, bool desc_s) {
   }
 }
 
+// ||Y_g|| of every candidate g of every cut, a warp per row, into s_out.
+__global__ void __launch_bounds__(256) k_cand_norms(const TruncCut* __restrict__ cuts) {
+  const TruncCut& A = cuts[blockIdx.y];
+  const int g = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (g >= A.ncand) return;
+  int b = 0, o = 0;
+  while (o + A.blk[b].K <= g) o += A.blk[b++].K;
+  const TruncBlk T = A.blk[b];
+  const double2* y = T.Y + (size_t)(g - o) * T.n;
+  double acc = 0.0;
+#pragma unroll 4
+  for (int c = lane; c < T.n; c += 32) {
+    const double2 v = y[c];
+    acc = fma(v.x, v.x, fma(v.y, v.y, acc));
+  }
+  acc = warp_sum_d(acc);
+  if (lane == 0) A.s_out[g] = sqrt(acc);
+}
+
 // Rule T (the tolerances of Sec. II B) on the merged spectrum of one cut:
 // p_k = s_k^2 / total, chi_w = smallest k with sum_{i>k} p_i <= w_cut,
 // chi_eps = #{p_k > eps_rel}, chi' = max(1, min(chi_max, chi_w, chi_eps, K)); the
@@ -176,76 +196,28 @@ __global__ void __launch_bounds__(TR_THREADS) k_trunc_u1(const TruncCut* __restr
   int* key = reinterpret_cast<int*>(s + P);
   __shared__ int off[1025];
   __shared__ int cnt_sh[1024];
-  __shared__ int chi_sh;
-  __shared__ double norm_sh;
+  __shared__ double red[33];
   if (threadIdx.x == 0) {
     int o = 0;
     for (int b = 0; b < A.nb; ++b) { off[b] = o; o += A.blk[b].K; }
     off[A.nb] = o;
   }
   for (int b = threadIdx.x; b < A.nb; b += blockDim.x) cnt_sh[b] = 0;
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int g = warp; g < A.ncand; g += nw) {
-    int b = 0;
-    while (off[b + 1] <= g) ++b;
-    const TruncBlk& T = A.blk[b];
-    const double2* y = T.Y + (size_t)(g - off[b]) * T.n;
-    double acc = 0.0;
-    for (int c = lane; c < T.n; c += 32) acc = fma(y[c].x, y[c].x, fma(y[c].y, y[c].y, acc));
-    acc = warp_sum_d(acc);
-    if (lane == 0) { s[g] = sqrt(acc); key[g] = g; }
+  for (int g = threadIdx.x; g < P; g += blockDim.x) {
+    s[g] = g < A.ncand ? A.s_out[g] : -1.0;
+    key[g] = g < A.ncand ? g : 0x7fffffff;
   }
-  for (int g = A.ncand + threadIdx.x; g < P; g += blockDim.x) { s[g] = -1.0; key[g] = 0x7fffffff; }
   __syncthreads();
   bitonic(s, key, P, true);
-  if (threadIdx.x == 0) {
-    const double total = A.total;
-    const int K = A.ncand;
-    bool bad = !(total > 0.0) || !isfinite(total);
-    double sumK = 0.0;
-    for (int i = 0; i < K; ++i) {
-      if (!isfinite(s[i])) bad = true;
-      sumK += s[i] * s[i];
-    }
-    int chi = 1;
-    double w = 0.0, kept = (K > 0) ? s[0] * s[0] : 0.0;
-    if (!bad) {
-      const double tailK = fmax(0.0, total - sumK);
-      int chi_eps = 0;
-      for (int i = 0; i < K; ++i) chi_eps += (s[i] * s[i] / total > A.eps_rel);
-      chi_eps = max(chi_eps, 1);
-      const double thr = A.w_cut * total;
-      int chi_w = K;
-      double tail = tailK;
-      for (int k = K; k >= 1; --k) {
-        if (tail <= thr) chi_w = k; else break;
-        tail += s[k - 1] * s[k - 1];
-      }
-      chi = max(1, min(min(A.chi_max, chi_w), min(chi_eps, K)));
-      double tc = tailK;
-      for (int i = K - 1; i >= chi; --i) tc += s[i] * s[i];
-      w = tc / total;
-      kept = 0.0;
-      for (int i = 0; i < chi; ++i) kept += s[i] * s[i];
-    } else {
-      atomicExch(A.status, TEBD_ERR_NONFINITE);
-    }
-    chi_sh = chi;
-    norm_sh = sqrt(kept);
-    *A.chi_out = chi;
-    *A.norm_out = norm_sh;
-    *A.w_out = w;
-  }
-  __syncthreads();
-  const int chi = chi_sh;
+  const int chi = truncation_rule(s, A.ncand, A.total, A.chi_max, A.w_cut, A.eps_rel, red, A.chi_out, A.norm_out,
+                                  A.w_out, A.status);
   // the kept entries by (block, row): sort the first chi entries by key
   int P2 = 1;
   while (P2 < chi) P2 <<= 1;
   for (int g = chi + threadIdx.x; g < P2; g += blockDim.x) { s[g] = -1.0; key[g] = 0x7fffffff; }
   __syncthreads();
   bitonic(s, key, P2, false);
-  const double inv = (norm_sh > 0.0) ? 1.0 / norm_sh : 0.0;
+  const double norm = *A.norm_out, inv = (norm > 0.0) ? 1.0 / norm : 0.0;
   for (int k = threadIdx.x; k < chi; k += blockDim.x) {
     const int g = key[k];
     int b = 0;
@@ -1266,8 +1238,11 @@ int decompose(tebd_ctx* c, std::vector<Cut*>& cuts, std::vector<char*>& bases, s
       cudaFuncSetAttribute(k_trunc_u1, cudaFuncAttributeMaxDynamicSharedMemorySize, 16384 * 12);
       attr = true;
     }
+    int most = 1;
+    for (const TruncCut& T : tc) most = std::max(most, T.ncand);
+    k_cand_norms<<<dim3((most + 7) / 8, (unsigned)nc), 256, 0, c->stream>>>(dtc);
     k_trunc_u1<<<(unsigned)nc, TR_THREADS, smem, c->stream>>>(dtc);
-    c->launches += 1;
+    c->launches += 2;
     if (int r = check_launch(c)) return r;
   }
   // read back chi', norms, weights, per-block counts and the status
