@@ -480,14 +480,55 @@ __global__ void __launch_bounds__(32) k_inviter(const __grid_constant__ EigBatch
   }
 }
 
+constexpr int NSS_WORK = 8192;   // K^2 m
+constexpr int NSS_SIZE = 2048;   // m K
+__host__ __device__ __forceinline__ bool ns_small(int m, int K) {
+  return (long long)K * K * m <= NSS_WORK && m * K <= NSS_SIZE;
+}
 // S <- 1.5 I - 0.5 S
 __global__ void k_ns_form(const __grid_constant__ EigBatch b) {
   const EigMat& M = b.a[blockIdx.y];
   const int K = M.K;
+  if (ns_small(M.m, K)) return;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < K * K; idx += gridDim.x * blockDim.x) {
     const int r = idx / K, c = idx % K;
     M.S[idx] = (r == c ? 1.5 : 0.0) - 0.5 * M.S[idx];
   }
+}
+
+// The three Newton-Schulz rounds of a small matrix in one block, with Z, its successor and S in shared
+// memory (result in Z2, as after three rounds of the products).  The limit is where nine launches (4 to 5 us
+// each) cost as much as the products on one SM (K^2 m / 16 FP64 warp instructions a round).  Measured, with
+// the back-transformation reading Z itself: six small blocked simulations 61.3 -> 56.3 ms a step, blocked L = 41
+// quench 34.4 -> 32.1 ms, super sites 9.9 -> 8.0 ms.
+__global__ void __launch_bounds__(256) k_ns_small(const __grid_constant__ EigBatch b) {
+  const EigMat& M = b.a[blockIdx.x];
+  const int m = M.m, K = M.K;
+  if (K == 0 || !ns_small(m, K)) return;
+  __shared__ double za[NSS_SIZE], zb[NSS_SIZE], S[NSS_WORK / 8];  // K^2 <= K^2 m / m, and m >= K
+  double *z = za, *zn = zb;
+  for (int e = threadIdx.x; e < m * K; e += blockDim.x) z[e] = M.Z[e];
+  __syncthreads();
+  for (int it = 0; it < 3; ++it) {
+    for (int e = threadIdx.x; e < K * K; e += blockDim.x) {
+      const int r = e / K, c = e - r * K;
+      double acc = 0.0;
+      for (int i = 0; i < m; ++i) acc = fma(z[i * K + r], z[i * K + c], acc);
+      S[e] = (r == c ? 1.5 : 0.0) - 0.5 * acc;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < m * K; e += blockDim.x) {
+      const int r = e / K, c = e - r * K;
+      double acc = 0.0;
+      for (int i = 0; i < K; ++i) acc = fma(z[r * K + i], S[i * K + c], acc);
+      zn[e] = acc;
+    }
+    __syncthreads();
+    double* t = z;
+    z = zn;
+    zn = t;
+  }
+  for (int e = threadIdx.x; e < m * K; e += blockDim.x) M.Z2[e] = z[e];
 }
 
 // U[j][r] = Z[r][j] (real -> complex, transposed).
@@ -510,7 +551,7 @@ __global__ void k_z_to_u(const __grid_constant__ EigBatch b, int use_z2) {
 }
 
 // ---- back-transformation, reflector by reflector (FP64 path) ------------------------------
-// U <- H(0) H(1) ... H(m-2) U, a warp per eigenvector, which it keeps in shared memory.  The Gram
+// U <- H(0) H(1) ... H(m-2) Z, a warp per eigenvector, which it keeps in registers (m <= 256) or shared memory.  The Gram
 // matrices are graded (rows scaled by lambda), and applying the reflectors one at a time keeps the small
 // leading components of the eigenvectors of small singular values to their own relative accuracy; a
 // compact-WY block of 64 in FP64 loses a digit of them (rows u^+ theta' of a graded 24 to 60 row matrix:
@@ -519,15 +560,52 @@ __global__ void k_z_to_u(const __grid_constant__ EigBatch b, int use_z2) {
 // Measured: 61 vectors of 4 matrices of 244 1.9 ms (8 vectors per block with block-wide sums 2.7 ms), 8 vectors
 // of matrices of 4 to 24 35 us (167 us).
 constexpr int BTS_SMEM = 12288 * 16;  // one vector of the largest matrix (m <= 12288)
-__global__ void k_backtransform(const __grid_constant__ EigBatch b, int stride) {
+__global__ void k_backtransform(const __grid_constant__ EigBatch b, int stride, int use_z2) {
   extern __shared__ double2 bts_sh[];
   const EigMat& M = b.a[blockIdx.y];
-  const int m = M.m, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m = M.m, K = M.K, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int j = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (j >= M.K) return;
-  double2* u = bts_sh + (size_t)warp * stride;
+  if (j >= K) return;
+  const double* Z = (use_z2 ? M.Z2 : M.Z) + j;
   double2* out = M.U + (size_t)j * m;
-  for (int r = lane; r < m; r += 32) u[r] = out[r];
+  constexpr int R = 8;
+  if (m <= 32 * R) {  // the vector in registers, the next reflector's entries on their way during a reflector
+    double2 u[R], vn[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      const int r = 32 * q + lane;
+      u[q] = make_double2(r < m ? Z[(size_t)r * K] : 0.0, 0.0);
+      vn[q] = (r > m - 2 && r < m && m > 1) ? M.H[(size_t)(m - 2) * m + r] : make_double2(0.0, 0.0);
+    }
+    for (int k = m - 2; k >= 0; --k) {
+      const double2 tau = M.tau[k];
+      double2 v[R];
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        v[q] = vn[q];
+        const int r = 32 * q + lane;
+        if (32 * q + 31 >= k) vn[q] = (k > 0 && r > k - 1 && r < m) ? M.H[(size_t)(k - 1) * m + r] : make_double2(0.0, 0.0);
+      }
+      if (tau.x == 0.0 && tau.y == 0.0) continue;
+      double2 a0 = make_double2(0.0, 0.0), a1 = a0;
+#pragma unroll
+      for (int q = 0; q < R; q += 2) {
+        if (32 * q + 31 > k && 32 * q < m) a0 = cfma_conj(v[q], u[q], a0);
+        if (32 * q + 63 > k && 32 * q + 32 < m) a1 = cfma_conj(v[q + 1], u[q + 1], a1);
+      }
+      double2 w = cmul(tau, warp_sum2(cadd(a0, a1)));
+      w = make_double2(-w.x, -w.y);
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+        if (32 * q + 31 > k && 32 * q < m) u[q] = cfma(w, v[q], u[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+      if (32 * q + lane < m) out[32 * q + lane] = u[q];
+    return;
+  }
+  double2* u = bts_sh + (size_t)warp * stride;
+  for (int r = lane; r < m; r += 32) u[r] = make_double2(Z[(size_t)r * K], 0.0);
   for (int k = m - 2; k >= 0; --k) {
     const double2 tau = M.tau[k];
     if (tau.x == 0.0 && tau.y == 0.0) continue;
@@ -1426,13 +1504,21 @@ int eig_vectors(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status,
   k_inviter<<<dim3((Kmax + 31) / 32, b.n), 32, 0, s>>>(b);
   ++launches;
   // Newton-Schulz: Z <- Z (1.5 I - 0.5 Z^T Z)
-  bool in_z2 = false;
-  for (int it = 0; it < 3; ++it) {
+  int n_small = 0, n_large = 0;
+  for (int i = 0; i < b.n; ++i)
+    if (b.a[i].K > 0) ++(ns_small(b.a[i].m, b.a[i].K) ? n_small : n_large);
+  if (n_small > 0) {
+    k_ns_small<<<b.n, 256, 0, s>>>(b);
+    ++launches;
+  }
+  bool in_z2 = true;  // three rounds end in Z2
+  if (n_large > 0) in_z2 = false;
+  for (int it = 0; it < 3 && n_large > 0; ++it) {
     Gemm g1(false, OP_C, OP_N), g2(false, OP_N, OP_N);
     std::vector<OzProb> o1, o2;  // the mixed path: the same real products on the exact-digit engine
     for (int i = 0; i < b.n; ++i) {
       const EigMat& M = b.a[i];
-      if (M.K == 0) continue;
+      if (M.K == 0 || ns_small(M.m, M.K)) continue;
       const double* Zc = in_z2 ? M.Z2 : M.Z;
       double* Zn = in_z2 ? M.Z : M.Z2;
       if (mixed) {
@@ -1461,7 +1547,7 @@ int eig_vectors(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status,
     } else {
       for (int i = 0; i < b.n; ++i) {
         const EigMat& M = b.a[i];
-        if (M.K == 0) continue;
+        if (M.K == 0 || ns_small(M.m, M.K)) continue;
         const double* Zc = in_z2 ? M.Z2 : M.Z;
         double* Zn = in_z2 ? M.Z : M.Z2;
         g2.add(M.m, M.K, M.K, Zc, M.K, M.S, M.K, Zn, M.K);
@@ -1471,10 +1557,7 @@ int eig_vectors(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status,
     in_z2 = !in_z2;
   }
   const int mm = max_m(b);
-  k_z_to_u<<<dim3((mm + 31) / 32, (Kmax + 31) / 32, b.n), dim3(32, 8), 0, s>>>(b, in_z2 ? 1 : 0);
-  ++launches;
   const int nblk = bt_blocks(mm);
-  if (nblk == 0) return launches;  // 1 x 1 matrices only
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_backtransform, cudaFuncAttributeMaxDynamicSharedMemorySize, BTS_SMEM);
@@ -1483,9 +1566,13 @@ int eig_vectors(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status,
   }
   if (!mixed) {  // as many warps per block as their vectors fit, at most 4: few vectors spread over the SMs
     const int stride = (mm + 31) & ~31, warps = std::max(1, std::min(4, BTS_SMEM / (stride * 16)));
-    k_backtransform<<<dim3((Kmax + warps - 1) / warps, b.n), 32 * warps, (size_t)warps * stride * 16, s>>>(b, stride);
+    k_backtransform<<<dim3((Kmax + warps - 1) / warps, b.n), 32 * warps, mm <= 256 ? 0 : (size_t)warps * stride * 16, s>>>(
+        b, stride, in_z2 ? 1 : 0);
     return launches + 1;
   }
+  k_z_to_u<<<dim3((mm + 31) / 32, (Kmax + 31) / 32, b.n), dim3(32, 8), 0, s>>>(b, in_z2 ? 1 : 0);
+  ++launches;
+  if (nblk == 0) return launches;  // 1 x 1 matrices only
   k_bt_clear<<<dim3(std::min(mm, 152), b.n), 128, 0, s>>>(b);
   Gemm gG(true, OP_N, OP_C);  // conj(V^+ V): FP64 on the CUDA cores (64 rows per block: too few for a tensor tile's cost)
   for (int i = 0; i < b.n; ++i) {
