@@ -681,11 +681,14 @@ int update_chunk(tebd_ctx* c, std::vector<Triple>& ts, int tidx) {
         }
         c->launches += oz_gemm_launch(o1, c->d_status, s);
         c->launches += oz_gemm_launch(o2, c->d_status, s);
-        c->launches += g3.launch(s);
+        if (two) c->launches += g3.launch(s);
+        else if (int r = launch_gate_rows(c, ts, tidx)) return r;
       } else {
         c->launches += tf32 ? g1.launch_tf32(s, c->d_status, oz_ws.data()) : g1.launch(s);
         c->launches += tf32 ? g2.launch_tf32(s, c->d_status, oz_ws.data()) : g2.launch(s);
-        c->launches += tf32 ? g3.launch_tf32(s, c->d_status, oz_ws.data()) : g3.launch(s);
+        if (tf32) c->launches += g3.launch_tf32(s, c->d_status, oz_ws.data());
+        else if (two) c->launches += g3.launch(s);
+        else if (int r = launch_gate_rows(c, ts, tidx)) return r;
       }
     }
     if (!c->randomized) {  // the randomized cut never forms the Gram matrix of theta'

@@ -85,6 +85,7 @@ struct tebd_ctx {
   std::vector<std::vector<int>> q;
   double2* Gblk = nullptr;  // gates restricted to each total-occupation block (u1.cu layout)
   size_t Gblk_n = 0;        // complex elements of Gblk
+  int* d_sigma = nullptr;   // device: the local states of three sites by their total occupation (u1.cu)
   ptebd::U1Work* u1w = nullptr;
   // randomized range finder for the truncated SVDs (option "randomized", dense form)
   bool randomized = false;
@@ -192,6 +193,8 @@ int update_chunk_u1(tebd_ctx* c, std::vector<Triple>& ts, int tidx);
 // Gates restricted to their total-occupation blocks, from the dense table (host,
 // Gall: ngates x D x D); allocates and fills c->Gblk.
 int u1_build_gate_blocks(tebd_ctx* c, const std::vector<std::complex<double>>& Gall, size_t ngates);
+// The gate of every triple of a dense batch, C = G theta~ by total occupation (FP64).
+int launch_gate_rows(tebd_ctx* c, const std::vector<Triple>& ts, int tidx);
 // Device bytes of the blocked workspace now held; releases it.
 size_t u1_workspace_bytes(const tebd_ctx* c);
 void u1_release(tebd_ctx* c);
