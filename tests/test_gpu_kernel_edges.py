@@ -1,9 +1,9 @@
 """GPU kernels at the sizes where their tiles, pieces and variants change.
 
 * tebd_zgemm on every engine around its tile edges, split reductions and direct tiles, against a
-  64-bit product of the same inputs.  Bounds: FP64 and exact digits K 2^-52 |A_i.|_max |B_j.|_max sums to
-  below 4 K eps of max|A| max|B|; 3xTF32 drops products below 2^-22 of each factor pair and adds K
-  terms in FP32, below K 2^-20 of max|A| max|B|.
+  64-bit product of the same inputs.  Bounds: a complex FP64 or exact-digit product of K terms is off by at
+  most 4 K eps max|A| max|B|; 3xTF32 drops 2^-22 of each real product and adds in FP32, below
+  K 2^-20 max|A| max|B|.
 * one Trotter layer of saturated states whose Gram matrices cross the reduction's piece sizes (256, 512,
   1024 trailing indices), its 64-column tail and the lanes of the bisection, against the dense oracle's
   update of the same triple: spectra to 1e-10 and densities to 1e-9, the bounds of single updates in the
