@@ -338,7 +338,6 @@ int eigen_stage(tebd_ctx* c, std::vector<Triple>& ts, bool second) {
     double w = 0.0;
     for (int t = 0; t < eb.n; ++t) w += 16.0 / 3.0 * std::pow((double)eb.a[t].m, 3);
     ProfScope ps(c, TEBD_PROF_TRIDIAG, w);
-    c->launches += eig_trace(eb, c->stream);
     const int nl = eig_tridiagonalize(eb, c->precision >= 1, oz_ws, c->d_status, c->stream);
     if (nl < 0) {
       cudaGetLastError();

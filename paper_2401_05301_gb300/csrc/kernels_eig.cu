@@ -91,14 +91,42 @@ __device__ __forceinline__ double pow2i(int e) { return __longlong_as_double((lo
 
 constexpr int NT = 256;
 
-// ---- trace --------------------------------------------------------------------
-__global__ void k_trace(const __grid_constant__ EigBatch b) {
-  const EigMat& M = b.a[blockIdx.x];
+// ---- trace and range ------------------------------------------------------------
+// The reduction forms A u and u^+ A u with unnormalised rows u and multiplies by the reflector's scale
+// and its square later, so what it holds grows and shrinks like the cube of the entries.  Doubles
+// carry that while the trace lies within 2^+-200 (a normalised state's is about 1) and every reflector's
+// row reaches 2^-340: |scale|^2 stays below 2^680, u^+ A u above 2^-680 |A|, and what is rounded
+// away lies below 2^-394.  The exact-digit trailing update holds v (of order 1) and w (of order A) in one row
+// with one exponent, so there the trace has to be near 1: its rounding is 2^-57 of the larger of the two.
+// A matrix outside is scaled by a power of two (exact) to a trace of [1, 2), and T is scaled back; eight
+// CTAs do it, one cluster per matrix.  Charge blocks of little weight pay that (one pass over them), the
+// matrices of a normalised state's dense form do not.
+constexpr int RANGE_FP64 = 200, RANGE_DIGITS = 8;
+constexpr int TRACE_CTAS = 8;
+// Exponent taken out of a matrix of trace tr (0: none, also for a trace that is zero or not finite).
+__device__ __forceinline__ int range_shift(double tr, int range) {
+  const int ef = (__double2hiint(tr) >> 20) & 0x7FF, e = ef - 1023;
+  if (!(tr > 0.0) || ef == 0x7FF || (e >= -range && e <= range)) return 0;
+  return max(-1022, min(1022, e));  // (pow2i takes no more; a subnormal trace ends in [2^-52, 1))
+}
+
+__global__ void __cluster_dims__(TRACE_CTAS, 1, 1) k_trace(const __grid_constant__ EigBatch b) {
+  const EigMat& M = b.a[blockIdx.y];
   __shared__ double sh[33];
   double s = 0.0;
   for (int r = threadIdx.x; r < M.m; r += blockDim.x) s += M.H[(size_t)r * M.m + r].x;
   s = block_sum(s, sh);
-  if (threadIdx.x == 0) *M.trace = s;
+  if (threadIdx.x == 0 && blockIdx.x == 0) *M.trace = s;
+  const int shift = range_shift(s, b.range);  // the same in all CTAs: each has summed the whole diagonal
+  if (shift == 0) return;
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  const double f = pow2i(-shift);
+  const size_t n = (size_t)M.m * M.m;
+#pragma unroll 4
+  for (size_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += TRACE_CTAS * blockDim.x) {
+    const double2 x = M.H[i];
+    M.H[i] = make_double2(x.x * f, x.y * f);
+  }
 }
 
 // ---- bisection --------------------------------------------------------------------
@@ -116,6 +144,14 @@ __global__ void __launch_bounds__(256) k_sturm_prep(const __grid_constant__ EigB
   const EigMat& M = b.a[blockIdx.x];
   const int m = M.m;
   __shared__ double sh[33];
+  if (const int shift = range_shift(*M.trace, b.range)) {  // T back to the matrix's own scale
+    const double f = pow2i(shift);
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+      M.d[i] *= f;
+      M.e[i] *= f;
+    }
+    __syncthreads();
+  }
   double lo = DBL_MAX, hi = DBL_MAX;  // hi stored negated for a min-reduction
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
     double r = 0.0;
@@ -710,12 +746,12 @@ __global__ void __launch_bounds__(4 * BT) k_bt_T(const __grid_constant__ EigBatc
 constexpr int TD_THREADS = 256;
 constexpr int TD_WARPS = TD_THREADS / 32;
 constexpr int TD_NB = 32;      // columns per panel of the blocked reduction
-// A column whose largest off-diagonal entry lies below 2^-900 is taken as already
-// reduced (tau = 0).  The Gram matrices here have trace ~1, so such entries are far
-// below their rounding; they do arise, as rounding noise that each Gram product
-// squares, in empty regions of the chain, and once subnormal the scale 1/amax of
-// the reflector would overflow and turn the column into NaN.
-constexpr int REFL_FLUSH_EXP = 900;
+// A column whose largest off-diagonal entry lies below 2^-340 is taken as already
+// reduced (tau = 0): with a trace of at least 2^-200 (k_trace) such entries are 2^-140 of it, far
+// below the matrix's rounding.  They do arise, as rounding noise that each Gram product
+// squares, in empty regions of the chain, and the squares and cubes that a column's scalars
+// hold would leave the range of a double (NaN below 2^-512).
+constexpr int REFL_FLUSH_EXP = 340;
 // The last TD_TAIL or fewer columns of every matrix are reduced by one block per
 // matrix with the trailing matrix in shared memory (k_tridiag_tail): there the
 // cooperative kernel would pay three grid barriers per column for very little work.
@@ -839,23 +875,16 @@ __device__ __forceinline__ int expo2(double2 x) {
 }
 
 // Partial norm of row k over one piece: lanes hold its entries (zero where there is none; `in`: counted
-// in the sum, i.e. not the first entry).  {sum |x|^2 2^(-2 bin), bin and largest exponent field}; bin is 0
-// unless the piece's largest exponent is outside +-400, where squares would leave the range.
+// in the sum, i.e. not the first entry).  {sum |x|^2, largest exponent field}: a row that is not
+// flushed has its largest entry within 2^-340 .. 2^200, so the squares that count stay in range.
 __device__ __forceinline__ void put_norm(const EigMat& M, int g, double2 x, bool in) {
   const int ef = __reduce_max_sync(0xffffffffu, expo2(x));
-  const int e = ef - 1023, bin = (e < -400 || e > 400) ? (ef == 2047 ? 0 : e) : 0;
   double s = 0.0;
   if (ef != 0) {
-    if (bin != 0) {
-      const double f = pow2i(max(-1022, min(1022, -bin)));
-      x.x *= f;
-      x.y *= f;
-    }
     s = in ? fma(x.x, x.x, x.y * x.y) : 0.0;
     s = warp_sum(s);
   }
-  if ((threadIdx.x & 31) == 0)
-    M.part[g] = make_double2(s, __longlong_as_double(((long long)(bin + 4096) << 32) | ef));
+  if ((threadIdx.x & 31) == 0) M.part[g] = make_double2(s, __longlong_as_double(ef));
 }
 
 // The scalars of column k's reflector from the partial norms of row k (one warp):
@@ -866,36 +895,27 @@ __device__ void td_scalars(const EigMat& M, int k) {
   const double2* row = M.H + (size_t)k * m;
   const double2 x0 = row[k + 1];
   const double dk = row[k].x, a00 = M.H[(size_t)(k + 1) * m + k + 1].x;
-  int bmax = -4096, emax = 0;
-  for (int g = lane; g < P.ng; g += 32) {
-    const long long t = __double_as_longlong(M.part[g].y);
-    const int ef = (int)(t & 0xffffffffll), bin = (int)(t >> 32) - 4096;
-    emax = max(emax, ef);
-    if (ef != 0) bmax = max(bmax, bin);
-  }
-  emax = __reduce_max_sync(0xffffffffu, emax);
-  bmax = __reduce_max_sync(0xffffffffu, bmax);
-  const int E = (emax == 0) ? 0 : bmax;
+  int emax = 0;
   double s = 0.0;
   for (int g = lane; g < P.ng; g += 32) {
     const double2 t = M.part[g];
-    const int d = (int)(__double_as_longlong(t.y) >> 32) - 4096 - E;
-    s += (d == 0) ? t.x : (d < -500 ? 0.0 : t.x * pow2i(2 * d));
+    emax = max(emax, (int)__double_as_longlong(t.y));
+    s += t.x;
   }
+  emax = __reduce_max_sync(0xffffffffu, emax);
   const double xnorm2 = warp_sum(s);
-  const bool flush = emax < 1023 - REFL_FLUSH_EXP;  // every entry below 2^-900
-  const double f = (E == 0) ? 1.0 : pow2i(max(-1022, min(1022, -E)));
-  const double ar = x0.x * f, ai = -x0.y * f;
+  const bool flush = emax < 1023 - REFL_FLUSH_EXP;  // every entry below 2^-340
+  const double ar = x0.x, ai = -x0.y;
   double beta = x0.x;
   double2 tau = make_double2(0.0, 0.0), sc = tau;
   if (!flush && !(xnorm2 == 0.0 && ai == 0.0)) {
     const double bs = -copysign(sqrt(ar * ar + ai * ai + xnorm2), ar), zr = ar - bs;
-    // lane 0: 1 / beta, lane 1: f / |alpha - beta|^2
-    const double r = ((lane & 1) ? f : 1.0) / ((lane & 1) ? fma(zr, zr, ai * ai) : bs);
+    // lane 0: 1 / beta, lane 1: 1 / |alpha - beta|^2
+    const double r = 1.0 / ((lane & 1) ? fma(zr, zr, ai * ai) : bs);
     const double inv = __shfl_sync(0xffffffffu, r, 0), iden = __shfl_sync(0xffffffffu, r, 1);
     tau = make_double2(-zr * inv, -ai * inv);
     sc = make_double2(zr * iden, -ai * iden);
-    beta = (E == 0) ? bs : bs * pow2i(max(-1022, min(1022, E)));
+    beta = bs;
   }
   if (lane == 0) {
     M.d[k] = dk;
@@ -1279,18 +1299,13 @@ __global__ void __launch_bounds__(TL_THREADS) k_tridiag_tail(const __grid_consta
     if (warp == TL_WARPS) {  // the reflector's scalars (td_scalars' arithmetic)
       const double2 xa = lane < n ? x[lane] : make_double2(0.0, 0.0);
       const double2 xb = lane + 32 < n ? x[lane + 32] : make_double2(0.0, 0.0);
-      const int ef = __reduce_max_sync(0xffffffffu, max(expo2(xa), expo2(xb))), e = ef - 1023;
-      const int E = (ef != 0 && ef != 2047 && (e < -400 || e > 400)) ? e : 0;
-      const double f = (E == 0) ? 1.0 : pow2i(max(-1022, min(1022, -E)));
+      const int ef = __reduce_max_sync(0xffffffffu, max(expo2(xa), expo2(xb)));
       double s = 0.0;
-      {
-        const double ax = xa.x * f, ay = xa.y * f, bx = xb.x * f, by = xb.y * f;
-        if (lane > 0) s = fma(ax, ax, ay * ay);
-        s = fma(bx, bx, fma(by, by, s));
-      }
+      if (lane > 0) s = fma(xa.x, xa.x, xa.y * xa.y);
+      s = fma(xb.x, xb.x, fma(xb.y, xb.y, s));
       const double xnorm2 = warp_sum(s);
       if (lane == 0) {
-        const double ar = xa.x * f, ai = -xa.y * f;
+        const double ar = xa.x, ai = -xa.y;
         double beta;
         double2 tau, sc;
         if (ef < 1023 - REFL_FLUSH_EXP || (xnorm2 == 0.0 && ai == 0.0)) {
@@ -1299,10 +1314,10 @@ __global__ void __launch_bounds__(TL_THREADS) k_tridiag_tail(const __grid_consta
           sc = make_double2(0.0, 0.0);
         } else {
           const double bs = -copysign(sqrt(ar * ar + ai * ai + xnorm2), ar);
-          const double zr = ar - bs, inv = 1.0 / bs, iden = f / (zr * zr + ai * ai);
+          const double zr = ar - bs, inv = 1.0 / bs, iden = 1.0 / (zr * zr + ai * ai);
           tau = make_double2(-zr * inv, -ai * inv);
           sc = make_double2(zr * iden, -ai * iden);
-          beta = (E == 0) ? bs : bs * pow2i(max(-1022, min(1022, E)));
+          beta = bs;
         }
         M.d[k] = As[j * TL_LD + j].x;
         M.e[k] = beta;
@@ -1380,15 +1395,10 @@ int max_m(const EigBatch& b) {
 
 static_assert(sizeof(EigBatch) < 32000, "kernel parameter block too large (32 KB on sm_70 and later)");
 
-int eig_trace(const EigBatch& b, cudaStream_t s) {
-  if (b.n == 0) return 0;
-  k_trace<<<b.n, NT, 0, s>>>(b);
-  return 1;
-}
-
 int eig_tridiagonalize(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status, cudaStream_t s) {
   if (b0.n == 0) return 0;
   EigBatch b = b0;
+  b.range = mixed ? RANGE_DIGITS : RANGE_FP64;
   for (int i = 0; i < b.n; ++i) {  // where the panel arrays' sized parts start
     EigMat& M = b.a[i];
     M.td_hr = M.pan + (size_t)M.m * 4 * TD_NB + (size_t)TD_DOTS * 2 * TD_NB + 32 * td_hc_tiles(M.m);
@@ -1405,7 +1415,8 @@ int eig_tridiagonalize(const EigBatch& b0, bool mixed, void* const* oz_ws, int* 
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag_panel, TD_THREADS, TD_SMEM);
   }
   const int grid = std::max(1, sms * std::min(per_sm, b.panel_blocks > 0 ? b.panel_blocks : 3));
-  int launches = 0;
+  k_trace<<<dim3(TRACE_CTAS, b.n), NT, 0, s>>>(b);
+  int launches = 1;
   int kend = 0;  // panels run while any matrix has columns before its tail
   for (int i = 0; i < b.n; ++i) kend = std::max(kend, tail_start(b.a[i].m));
   for (int k0 = 0; k0 < kend; k0 += TD_NB) {

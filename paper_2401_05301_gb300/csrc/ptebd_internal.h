@@ -209,13 +209,14 @@ struct EigBatch {
   unsigned int* bar;  // grid-barrier state {count, generation, error} for the persistent reduction
   long long wait_clocks;  // limit of each grid-barrier wait of the reduction (clock64 ticks)
   int panel_blocks;       // blocks per SM of the reduction's cooperative grid (0: as many as fit, at most 3)
+  int range;              // traces outside 2^+-range are scaled for the reduction (set by eig_tridiagonalize)
   int few;                // 1: dense form, a batch of at most 24 matrices (the bisection spreads wider)
 };
 
 constexpr int EIG_PARTS = 384;  // partial norms of a row, one per column piece (32 columns at m = 12288)
 
 // Each returns the number of kernel launches issued.
-int eig_trace(const EigBatch& b, cudaStream_t s);
+// Writes the trace, scales the matrix if that is far from 1, and reduces it to T.
 // Blocked (panels of 32 columns): one cooperative launch per panel plus the
 // trailing rank-64 update, on the exact-digit tensor-core engine when mixed
 // (oz_ws[i]: a digit workspace per matrix) or the FP64 GEMM otherwise.

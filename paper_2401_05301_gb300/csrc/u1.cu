@@ -986,7 +986,6 @@ int decompose(tebd_ctx* c, std::vector<Cut*>& cuts, std::vector<char*>& bases, s
       eb.wait_clocks = c->wait_clocks;
       eb.panel_blocks = c->panel_blocks;
       for (size_t j = g0; j < std::min(jobs.size(), g0 + EIG_MAXP); ++j) eb.a[eb.n++] = mat(jobs[j]);
-      c->launches += eig_trace(eb, c->stream);
       const int nl = eig_tridiagonalize(eb, mixed, ozw, c->d_status, c->stream);
       if (nl < 0) {
         cudaGetLastError();
