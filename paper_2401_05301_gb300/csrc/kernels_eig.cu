@@ -1406,14 +1406,17 @@ int eig_tridiagonalize(const EigBatch& b0, bool mixed, void* const* oz_ws, int* 
     M.td_sc = M.td_hr + 32 * td_hr_tiles(M.m) + (td_hc_tiles(M.m) + 1) / 2;
   }
   const int mm = max_m(b);
-  static int sms = 0, per_sm = 0;
-  if (sms == 0) {
-    int dev = 0;
+  static PerDevice panel_shape;  // SMs, and blocks of the panel kernel that fit one (low byte)
+  const int shape = panel_shape([] {
+    int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(k_tridiag_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, TD_SMEM);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag_panel, TD_THREADS, TD_SMEM);
-  }
+    if (!allow_smem(k_tridiag_panel, TD_SMEM) ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag_panel, TD_THREADS, TD_SMEM) != cudaSuccess)
+      return 0;
+    return sms << 8 | per_sm;
+  });
+  const int sms = shape >> 8, per_sm = shape & 255;
   const int grid = std::max(1, sms * std::min(per_sm, b.panel_blocks > 0 ? b.panel_blocks : 3));
   k_trace<<<dim3(TRACE_CTAS, b.n), NT, 0, s>>>(b);
   int launches = 1;
@@ -1471,11 +1474,8 @@ int eig_tridiagonalize(const EigBatch& b0, bool mixed, void* const* oz_ws, int* 
   }
   {
     constexpr int TL_SMEM = (TD_TAIL * TL_LD + 2 * TD_TAIL) * (int)sizeof(double2);
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(k_tridiag_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, TL_SMEM);
-      attr = true;
-    }
+    static PerDevice smem;
+    smem([] { return allow_smem(k_tridiag_tail, TL_SMEM); });
     k_tridiag_tail<<<b.n, TL_THREADS, TL_SMEM, s>>>(b);
     ++launches;
   }
@@ -1569,12 +1569,8 @@ int eig_vectors(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status,
   }
   const int mm = max_m(b);
   const int nblk = bt_blocks(mm);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_backtransform, cudaFuncAttributeMaxDynamicSharedMemorySize, BTS_SMEM);
-    cudaFuncSetAttribute(k_bt_T, cudaFuncAttributeMaxDynamicSharedMemorySize, BT * (BT + 1) * 16);
-    attr = true;
-  }
+  static PerDevice smem;
+  smem([] { return allow_smem(k_backtransform, BTS_SMEM) & allow_smem(k_bt_T, BT * (BT + 1) * 16); });
   if (!mixed) {  // as many warps per block as their vectors fit, at most 4: few vectors spread over the SMs
     const int stride = (mm + 31) & ~31, warps = std::max(1, std::min(4, BTS_SMEM / (stride * 16)));
     k_backtransform<<<dim3((Kmax + warps - 1) / warps, b.n), 32 * warps, mm <= 256 ? 0 : (size_t)warps * stride * 16, s>>>(

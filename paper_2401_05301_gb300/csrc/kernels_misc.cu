@@ -219,11 +219,8 @@ int launch_truncate(const TruncBatch& b, cudaStream_t s) {
   int P = 1;
   while (P < Kmax) P <<= 1;
   const size_t smem = (size_t)P * (sizeof(double) + sizeof(int));
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_truncate, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr = true;
-  }
+  static PerDevice allowed;
+  allowed([] { return allow_smem(k_truncate, 200 * 1024); });
   k_row_norms<<<dim3((Kmax + 7) / 8, b.n), 256, 0, s>>>(b);
   k_truncate<<<b.n, 512, smem, s>>>(b);
   return 2;

@@ -728,11 +728,8 @@ int oz_gemm_pooled(std::vector<OzProb>& probs, void* pool, size_t bytes, int* st
 namespace {
 template <int CAP>
 int launch_all(const std::vector<OzProb>& probs, int* status, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_oz_gemm<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
-    attr = true;
-  }
+  static PerDevice smem;
+  smem([] { return allow_smem(k_oz_gemm<CAP>, OZ_SMEM); });
   int launches = 0;
   size_t i0 = 0;
   while (i0 < probs.size()) {

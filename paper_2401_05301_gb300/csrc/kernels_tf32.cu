@@ -504,11 +504,8 @@ size_t tc_workspace_bytes(int M, int N, int K, int batch) {
 namespace {
 template <int CAP>
 int launch_all(const std::vector<TcGemmProb>& probs, int* status, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_tf32x3<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    attr = true;
-  }
+  static PerDevice smem;
+  smem([] { return allow_smem(k_tf32x3<CAP>, SMEM_BYTES); });
   int launches = 0;
   for (size_t i = 0; i < probs.size();) {
     TfBatch<CAP> gb;

@@ -4,11 +4,36 @@
 #include <complex>
 #include <cstddef>
 #include <cstdint>
+#include <mutex>
 #include <vector>
 
 #include <cuda_runtime.h>
 
 namespace ptebd {
+
+// What a kernel needs once per device before its first launch: its dynamic shared memory beyond 48 KB, its
+// occupancy.  Handles are used from several threads, so a launch waits until the setup is done; make()
+// returns the value to keep, 0 (a refused call) is tried again at the next launch.
+class PerDevice {
+ public:
+  template <class F>
+  int operator()(F make) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return make();
+    std::lock_guard<std::mutex> lock(mutex_);
+    if (dev >= (int)value_.size()) value_.resize(dev + 1, 0);
+    if (value_[dev] == 0) value_[dev] = make();
+    return value_[dev];
+  }
+
+ private:
+  std::mutex mutex_;
+  std::vector<int> value_;
+};
+template <class K>
+int allow_smem(K* kernel, int bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess ? 1 : 0;
+}
 
 // ---- host gate builder (gates_host.cpp) --------------------------------------
 std::vector<std::complex<double>> three_site_term(int L, int n_max, double U, double J, double Jnnn,

@@ -1287,11 +1287,8 @@ int decompose(tebd_ctx* c, std::vector<Cut*>& cuts, std::vector<char*>& bases, s
     TruncCut* dtc = stage(c, tc, &err);
     if (err) return err;
     const size_t smem = (size_t)maxP * (sizeof(double) + sizeof(int));
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(k_trunc_u1, cudaFuncAttributeMaxDynamicSharedMemorySize, 16384 * 12);
-      attr = true;
-    }
+    static PerDevice allowed;
+    allowed([] { return allow_smem(k_trunc_u1, 16384 * 12); });
     int most = 1;
     for (const TruncCut& T : tc) most = std::max(most, T.ncand);
     k_cand_norms<<<dim3((most + 7) / 8, (unsigned)nc), 256, 0, c->stream>>>(dtc);
