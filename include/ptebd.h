@@ -347,7 +347,8 @@ int tebd_gate_host_supersite(int L, int n_max, double U, double J, double J_NNN,
  * projection engine: eight 7-bit digits per row-scaled real, exact integer
  * accumulation, one final rounding; error below 2^-53 max|A_i.| max|B_.j| K).
  * Precision 1 and 2 allocate and free their workspace (operand planes) stream-ordered
- * on cuda_stream.  Enqueued on cuda_stream (NULL = legacy default stream), not
+ * on cuda_stream; precision 1 works block by block where the planes of the whole
+ * product do not fit (one tile's take 4 KB per k).  Enqueued on cuda_stream (NULL = legacy default stream), not
  * synchronised.  Sizes >= 1, leading dimensions >= the row lengths; otherwise
  * TEBD_ERR_ARG. */
 int tebd_zgemm(int precision, int opB, int M, int N, int K, double alpha, const double* A, long long lda,

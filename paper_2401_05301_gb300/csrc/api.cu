@@ -1160,24 +1160,36 @@ int tebd_zgemm(int precision, int opB, int M, int N, int K, double alpha, const 
   }
   try {
     Gemm g(true, OP_N, opB ? OP_C : OP_N);
-    GemmProb& p = g.add(M, N, K, A, lda, B, ldb, C, ldc);
-    p.alpha_re = alpha;
     if (precision == 1) {
       cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+      // Planes of the whole product or, where the device has no room for them, of as large a block of it as fits
+      // (halved down to one tile): a tile's arithmetic does not depend on the block that it is in.
+      int mb = M, nb = N;
       void* ws = nullptr;
-      const size_t bytes = tc_workspace_bytes(M, N, K, 1);
-      if (bytes > 0 && ws_alloc(&ws, bytes, st) != cudaSuccess) {
+      for (size_t bytes; (bytes = tc_workspace_bytes(mb, nb, K, 1)) > 0 && ws_alloc(&ws, bytes, st) != cudaSuccess;) {
         cudaGetLastError();
-        return TEBD_ERR_OOM;
+        ws = nullptr;
+        if (mb <= TC_TILE_M && nb <= TC_TILE_N) return TEBD_ERR_OOM;
+        // a row of A takes 16 bytes of planes per k, a column of B 32
+        if (nb <= TC_TILE_N || (mb > TC_TILE_M && mb >= 2LL * nb)) mb = ((mb + 1) / 2 + TC_TILE_M - 1) / TC_TILE_M * TC_TILE_M;
+        else nb = ((nb + 1) / 2 + TC_TILE_N - 1) / TC_TILE_N * TC_TILE_N;
       }
       try {
-        g.launch_tf32(st, nullptr, &ws);
+        for (int m0 = 0; m0 < M; m0 += mb)
+          for (int n0 = 0; n0 < N; n0 += nb) {
+            const double* a = A + 2 * (long long)m0 * lda;
+            const double* b = B + 2 * (opB ? (long long)n0 * ldb : (long long)n0);
+            g.add(std::min(mb, M - m0), std::min(nb, N - n0), K, a, lda, b, ldb, C + 2 * ((long long)m0 * ldc + n0), ldc)
+                .alpha_re = alpha;
+            g.launch_tf32(st, nullptr, &ws);
+          }
       } catch (...) {
         if (ws) cudaFreeAsync(ws, st);
         return TEBD_ERR_OOM;
       }
       if (ws) cudaFreeAsync(ws, st);
     } else {
+      g.add(M, N, K, A, lda, B, ldb, C, ldc).alpha_re = alpha;
       g.launch(static_cast<cudaStream_t>(cuda_stream));
     }
   } catch (...) {

@@ -43,8 +43,8 @@ namespace ptebd {
 
 namespace {
 
-constexpr int TM = 128;               // rows of the real product per CTA (UMMA M)
-constexpr int TN = 128;               // columns of the real product per CTA (UMMA N) = 64 complex
+constexpr int TM = TC_TILE_M;         // rows of the real product per CTA (UMMA M)
+constexpr int TN = 2 * TC_TILE_N;     // columns of the real product per CTA (UMMA N) = 64 complex
 constexpr int TK = 32;                // reals of K per slab (one 128-byte swizzle row of fp32)
 constexpr int DW = 8;                 // drain warps: 4 lane groups x 2 column halves
 constexpr int NT = 32 * (DW + 2);     // + one copy warp + one MMA warp

@@ -97,6 +97,7 @@ struct TcGemmProb {
   void* ws;  // tc_workspace_bytes(M, N, K, batch) bytes, 256-byte aligned, owned by the caller
 };
 constexpr int TC_MAXP = 64;
+constexpr int TC_TILE_M = 128, TC_TILE_N = 64;  // complex outputs of a CTA
 size_t tc_workspace_bytes(int M, int N, int K, int batch);
 int tc_gemm_launch(const std::vector<TcGemmProb>& probs, int* status, cudaStream_t s);
 // The same with the workspaces taken from one pool (bytes >= the largest problem's need).
