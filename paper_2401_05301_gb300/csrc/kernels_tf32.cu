@@ -372,7 +372,8 @@ __global__ void __launch_bounds__(NT, 1) k_tf32x3(const __grid_constant__ TfBatc
           mma_tf32(d, smem_desc(a_hi + off), smem_desc(b_hi + off), idesc, 1u);
           mma_commit(&accfull[kk]);
         }
-        if (ok) mma_commit(&empty[st]);
+        // (no copy waits for the last stages: an arrival there could outlive the CTA)
+        if (ok && kt + STAGES < nk) mma_commit(&empty[st]);
       }
       if (!ok) {
         *fail_sh = 1;
