@@ -595,13 +595,66 @@ __global__ void k_z_to_u(const __grid_constant__ EigBatch b, int use_z2) {
 // Bound: the FP64 pipe, 8 instructions per 32 rows and reflector and 14 for the dot product's sum.
 // Measured: 61 vectors of 4 matrices of 244 1.9 ms (8 vectors per block with block-wide sums 2.7 ms), 8 vectors
 // of matrices of 4 to 24 35 us (167 us).
-constexpr int BTS_SMEM = 12288 * 16;  // one vector of the largest matrix (m <= 12288)
+constexpr int BTS_SMEM = 12288 * 16;  // one vector of the largest matrix (m <= 12288), four of BTS_WARP
+constexpr int BTS_WARP = 3072;        // largest matrix for a warp per vector
+// Larger matrices: two vectors fit a block, or one, and the FP64 pipe of an SM is four quarters that one warp cannot
+// fill, so four or eight warps share a vector (rows dealt in turn, partial dots added in a fixed order).
+// Measured, eigenvector stage of an FP64 layer, against a warp per vector: chi = 1024, d = 4 (m = 4096) 750 -> 462 ms,
+// chi = 1536 (m = 6144) 3290 -> 1450 ms.
+__host__ __device__ __forceinline__ int btw_vectors(int m) { return m <= 6144 ? 2 : 1; }  // per block of 8 warps
+template <int NW>
+__device__ __forceinline__ void btw_vector(const EigMat& M, const double* Z, double2* u, double2* out, double2* slots,
+                                           int vec, int part) {
+  constexpr int STEP = 32 * NW;  // rows keep their warp and lane
+  const int m = M.m, lane = threadIdx.x & 31, first = 32 * part + lane;
+  int phase = 0;
+  for (int r = first; r < m; r += STEP) u[r] = make_double2(Z[(size_t)r * M.K], 0.0);
+  for (int k = m - 2; k >= 0; --k) {
+    const double2 tau = M.tau[k];
+    if (tau.x == 0.0 && tau.y == 0.0) continue;
+    const double2* v = M.H + (size_t)k * m;
+    const int r0 = ((k + 1) & ~(STEP - 1)) + first;
+    double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int r = r0; r < m; r += STEP)
+      if (r > k) acc = cfma_conj(v[r], u[r], acc);
+    acc = warp_sum2(acc);
+    // two sets of sums in turn: one is written again only after the barrier that follows its reading
+    double2* sums = slots + 8 * phase;
+    phase ^= 1;
+    if (lane == 0) sums[part] = acc;
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + vec), "r"(STEP) : "memory");
+    acc = sums[0];
+#pragma unroll
+    for (int q = 1; q < NW; ++q) acc = cadd(acc, sums[q]);
+    double2 w = cmul(tau, acc);
+    w = make_double2(-w.x, -w.y);
+#pragma unroll 4
+    for (int r = r0; r < m; r += STEP)
+      if (r > k) u[r] = cfma(w, v[r], u[r]);
+  }
+  for (int r = first; r < m; r += STEP) out[r] = u[r];
+}
+
+// WIDE: 8 warps a block, for a batch that holds such matrices (the others take four of the warps).
+template <bool WIDE>
 __global__ void k_backtransform(const __grid_constant__ EigBatch b, int stride, int use_z2) {
   extern __shared__ double2 bts_sh[];
   const EigMat& M = b.a[blockIdx.y];
   const int m = M.m, K = M.K, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int j = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (j >= K) return;
+  if (WIDE && m > BTS_WARP) {
+    __shared__ double2 slots[16];  // two sets of a sum per warp
+    const int nv = btw_vectors(m), nw = 8 / nv, vec = warp / nw, part = warp - vec * nw, j = blockIdx.x * nv + vec;
+    if (j >= K) return;
+    const double* Z = (use_z2 ? M.Z2 : M.Z) + j;
+    double2* u = bts_sh + (size_t)vec * ((m + 31) & ~31);
+    double2* out = M.U + (size_t)j * m;
+    if (nw == 4) btw_vector<4>(M, Z, u, out, slots + 4 * vec, vec, part);
+    else btw_vector<8>(M, Z, u, out, slots, vec, part);
+    return;
+  }
+  const int j = blockIdx.x * 4 + warp;
+  if (j >= K || (WIDE && warp >= 4)) return;
   const double* Z = (use_z2 ? M.Z2 : M.Z) + j;
   double2* out = M.U + (size_t)j * m;
   constexpr int R = 8;
@@ -1570,11 +1623,23 @@ int eig_vectors(const EigBatch& b0, bool mixed, void* const* oz_ws, int* status,
   const int mm = max_m(b);
   const int nblk = bt_blocks(mm);
   static PerDevice smem;
-  smem([] { return allow_smem(k_backtransform, BTS_SMEM) & allow_smem(k_bt_T, BT * (BT + 1) * 16); });
-  if (!mixed) {  // as many warps per block as their vectors fit, at most 4: few vectors spread over the SMs
-    const int stride = (mm + 31) & ~31, warps = std::max(1, std::min(4, BTS_SMEM / (stride * 16)));
-    k_backtransform<<<dim3((Kmax + warps - 1) / warps, b.n), 32 * warps, mm <= 256 ? 0 : (size_t)warps * stride * 16, s>>>(
-        b, stride, in_z2 ? 1 : 0);
+  smem([] {
+    return allow_smem(k_backtransform<false>, BTS_SMEM) & allow_smem(k_backtransform<true>, BTS_SMEM) &
+           allow_smem(k_bt_T, BT * (BT + 1) * 16);
+  });
+  if (!mixed) {  // four vectors per block: few of them spread over the SMs
+    int m1 = 0, blocks = 1;  // the largest matrix of a warp per vector
+    size_t bytes = 0;
+    for (int i = 0; i < b.n; ++i) {
+      const int m = b.a[i].m, nv = m <= BTS_WARP ? 4 : btw_vectors(m);
+      blocks = std::max(blocks, (b.a[i].K + nv - 1) / nv);
+      if (m <= BTS_WARP) m1 = std::max(m1, m);
+      if (m > 256) bytes = std::max(bytes, (size_t)nv * ((m + 31) & ~31) * 16);
+    }
+    const dim3 grid(blocks, b.n);
+    const int stride = (m1 + 31) & ~31, z2 = in_z2 ? 1 : 0;
+    if (mm > BTS_WARP) k_backtransform<true><<<grid, 256, bytes, s>>>(b, stride, z2);
+    else k_backtransform<false><<<grid, 128, bytes, s>>>(b, stride, z2);
     return launches + 1;
   }
   k_z_to_u<<<dim3((mm + 31) / 32, (Kmax + 31) / 32, b.n), dim3(32, 8), 0, s>>>(b, in_z2 ? 1 : 0);
