@@ -11,6 +11,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 using namespace ptebd;
@@ -1079,27 +1080,29 @@ int graph_step(tebd_ctx* c, const std::vector<tebd_ctx*>& hs, const std::vector<
 }
 
 int ensure_measure_ws(tebd_ctx* c) {
-  if (!c->mN) {  // super sites: two physical densities per site, 2L - 1 physical bonds; then partial sums
-    const size_t n = c->ss ? 2 * (size_t)c->L : (size_t)c->L;
-    c->mC = dalloc<double2>(c, n + MEAS_CHUNK * TRACE_PARTS);
-    c->mN = dalloc<double>(c, n * (1 + DENSITY_PARTS));
-    if (!c->mC || !c->mN) return TEBD_ERR_OOM;
-  }
-  if (c->u1 && c->have_charges) return TEBD_OK;  // the blocked correlators use their own arena
-  if (!c->mX) {
+  // each buffer by itself: a call that finds no memory leaves the ones it got to the next call
+  bool ok = true;
+  auto need = [&](auto*& p, size_t n) {
+    if (!p) p = dalloc<std::remove_reference_t<decltype(*p)>>(c, n);
+    ok = ok && p;
+  };
+  // super sites: two physical densities per site, 2L - 1 physical bonds; then partial sums
+  const size_t n = c->ss ? 2 * (size_t)c->L : (size_t)c->L;
+  need(c->mC, n + MEAS_CHUNK * TRACE_PARTS);
+  need(c->mN, n * (1 + DENSITY_PARTS));
+  if (!(c->u1 && c->have_charges)) {  // (the blocked correlators use their own arena)
     const long long capmax = std::max<long long>(1, *std::max_element(c->cap.begin(), c->cap.end()));
     const long long big = capmax * c->d * capmax;
     if (c->ss) {  // super sites shift one position of a pair: the shifted factors are formed
-      c->mP = dalloc<double2>(c, MEAS_CHUNK * big);
-      c->mQ = dalloc<double2>(c, MEAS_CHUNK * big);
+      need(c->mP, MEAS_CHUNK * big);
+      need(c->mQ, MEAS_CHUNK * big);
     } else {      // weights of the products' reductions
-      c->mW = dalloc<double>(c, MEAS_CHUNK * (capmax + 1) * (c->d - 1));
+      need(c->mW, MEAS_CHUNK * (capmax + 1) * (c->d - 1));
     }
-    c->mY = dalloc<double2>(c, MEAS_CHUNK * capmax * capmax);
-    c->mX = dalloc<double2>(c, MEAS_CHUNK * capmax * capmax);
-    if ((c->ss ? !c->mP || !c->mQ : !c->mW) || !c->mX || !c->mY) return TEBD_ERR_OOM;
+    need(c->mY, MEAS_CHUNK * capmax * capmax);
+    need(c->mX, MEAS_CHUNK * capmax * capmax);
   }
-  return TEBD_OK;
+  return ok ? TEBD_OK : TEBD_ERR_OOM;
 }
 
 #define CHECK_HANDLE(h)                         \

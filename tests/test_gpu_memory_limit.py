@@ -1,8 +1,10 @@
-"""Products when the device is nearly full."""
+"""Calls when the device is nearly full."""
 import ctypes
 
+import numpy as np
 import pytest
 
+import workloads
 from device_memory import MB, only
 
 pytestmark = pytest.mark.gpu
@@ -28,3 +30,30 @@ def test_split_tf32_product_in_blocks(lib, opB, M, N, K):
         assert product(out) == 0
         torch.cuda.synchronize()
     assert torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("form", ["dense", "supersite"])
+def test_measurement_after_one_without_memory(lib, form):
+    """A measurement whose buffers do not fit reports it; the next one, with memory, is the ordinary one."""
+    from paper_2401_05301_gb300 import SuperSiteTEBD, TEBD
+    from paper_2401_05301_gb300.binding import TEBDError
+    args = (20, 3, 256, 4.0, 1.0, 0.1, 0.004, 10.5, 0.02) if form == "dense" else (20, 3, 128, 4.0, 1.0, 0.1, 0.004, 10.5, 0.02)
+
+    def simulation():
+        g = (TEBD if form == "dense" else SuperSiteTEBD)(*args)
+        L, d = (20, 4) if form == "dense" else (10, 16)
+        B, lam, _ = workloads.synthetic_state(L, d, args[2])
+        g.set_state(B, lam)
+        return g
+
+    ref = simulation()
+    n, cur = ref.measure()
+    ref.close()
+    g = simulation()
+    with only(12 * MB):
+        with pytest.raises(TEBDError) as e:
+            g.measure()
+        assert e.value.status == -2
+    for a, b in zip(g.measure(), (n, cur)):
+        assert np.array_equal(a, b)
+    g.close()
