@@ -207,7 +207,7 @@ int build_gates(tebd_ctx* c) {
   }
   c->G_bytes = taus.size() * L2 * DD * sizeof(double2);
   c->G = G;
-  return TEBD_OK;
+  return finish_uploads();
 }
 
 int alloc_workspace(tebd_ctx* c) {
@@ -1300,7 +1300,7 @@ int create_impl(int L, int L_phys, bool ss, int n_max, int chi_max, double U, do
     if (cudaMemcpy(c->dB, c->B.data(), L * sizeof(double2*), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(c->dlam, c->lam.data(), (L + 1) * sizeof(double*), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(c->d_status, 0, sizeof(int)) != cudaSuccess ||
-        cudaMemset(c->d_bar, 0, 4 * sizeof(unsigned int)) != cudaSuccess) {
+        cudaMemset(c->d_bar, 0, 4 * sizeof(unsigned int)) != cudaSuccess || finish_uploads() != TEBD_OK) {
       cudaGetLastError();
       tebd_destroy(c);
       return TEBD_ERR_CUDA;
@@ -1521,7 +1521,7 @@ int tebd_set_state(tebd_handle h, const int* chi, const double* const* B_ptrs, c
   h->w_total = 0.0;
   h->gate_updates = 0;
   h->have_state = true;
-  return TEBD_OK;
+  return finish_uploads() == TEBD_OK ? TEBD_OK : fail_cuda(h);
 }
 
 int tebd_step(tebd_handle h, int n_steps) {

@@ -190,6 +190,13 @@ int ensure_pinned(tebd_ctx* c, size_t n);
 // One batch of independent local updates with every product and decomposition
 // taken block by block over the conserved boson number.
 int update_chunk_u1(tebd_ctx* c, std::vector<Triple>& ts, int tidx);
+// A copy from pageable memory returns once its source is staged: a handle's stream that does not wait for
+// the legacy one (a non-blocking stream of the caller's) must not start before it has arrived.
+inline int finish_uploads() {
+  if (cudaStreamSynchronize(nullptr) == cudaSuccess) return TEBD_OK;
+  cudaGetLastError();
+  return TEBD_ERR_CUDA;
+}
 // Gates restricted to their total-occupation blocks, from the dense table (host,
 // Gall: ngates x D x D); allocates and fills c->Gblk.
 int u1_build_gate_blocks(tebd_ctx* c, const std::vector<std::complex<double>>& Gall, size_t ngates);

@@ -2020,6 +2020,7 @@ int rand_cut_body(tebd_ctx* c, std::vector<Triple>& ts, bool second) {
     fa[t] = FrobArgs{in[t].X, in[t].lam, in[t].m, in[t].n, in[t].d,
                      reinterpret_cast<double*>(sl[t]->a2.base + align256(16 * (size_t)in[t].n * ell[t]))};
   }
+  if (finish_uploads() != TEBD_OK) return fail_cuda(c);
   {
     int err = TEBD_OK;
     FrobArgs* dfa = stage(c, fa, &err);
