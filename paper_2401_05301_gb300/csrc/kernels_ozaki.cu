@@ -352,6 +352,19 @@ __device__ __forceinline__ void tile_of(const OzTile& P, int local, int& mt, int
   nt = rem;
 }
 
+// oz_value at the ends of the range (out of line: it would cost the ordinary path registers): a subnormal result is
+// rounded where its last bit is, the upper end overflows as the library does.  t: the leading 64 bits, m: their
+// first 53, rounded.
+__device__ __noinline__ double oz_edge(unsigned long long t, bool rest, unsigned long long m, int ex, bool neg) {
+  if (ex >= 2046) return ldexp(neg ? -(double)m : (double)m, ex - 1075);
+  const int drop = 12 - ex;  // low bits of t that go
+  if (drop > 64) return 0.0;
+  const unsigned long long low = drop < 64 ? t << (64 - drop) : t, tie = 1ull << 63;
+  unsigned long long r = drop < 64 ? t >> drop : 0ull;
+  if (low > tie || (low == tie && (rest || (r & 1ull)))) ++r;
+  return __longlong_as_double((long long)(r | (neg ? 1ull << 63 : 0ull)));
+}
+
 // (P_hi 2^28 + P_lo) 2^x rounded once to FP64, on the integer pipe.
 __device__ __forceinline__ double oz_value(long long Phi, long long Plo, int x) {
   unsigned long long lo = (unsigned long long)Phi << 28;
@@ -383,8 +396,7 @@ __device__ __forceinline__ double oz_value(long long Phi, long long Plo, int x) 
   const unsigned long long sticky = (t & 0x3FFull) | (rest ? 1ull : 0ull), half = t & 0x400ull;
   unsigned long long m = t >> 11;  // 53 bits with the leading one
   if (half && (sticky || (m & 1ull))) ++m;
-  if (ex <= 0 || ex >= 2046)  // near the ends of the range: let the library round or overflow
-    return ldexp(neg ? -(double)m : (double)m, n - 52 + x);
+  if (ex <= 0 || ex >= 2046) return oz_edge(t, rest != 0, m, ex, neg);
   const unsigned long long bits = (m + ((unsigned long long)(ex - 1) << 52)) | (neg ? 1ull << 63 : 0ull);
   return __longlong_as_double((long long)bits);
 }
