@@ -138,7 +138,7 @@ int tebd_create_supersite(int L, int n_max, int chi_max, double U, double J, dou
  *   "graph_test_fallback" n >= 0 (diagnostic): treat the next n accepted replays as
  *             failed checks (state restored from the backup, step run the ordinary way),
  *             to test that path; unlike every other option it keeps the cached graph.
- *   "panel_blocks" 0 (default: as many as fit, at most 3) or 1..3: blocks per SM of the
+ *   "panel_blocks" 0 (default: as many as fit, two) or 1..3: blocks per SM of the
  *             tridiagonal reduction's cooperative grid (a launch shape; the arithmetic and
  *             its order do not depend on it).  Chosen per (chi, d) bucket by the package's
  *             autotuner (paper_2401_05301_gb300/autotune.py).

@@ -20,7 +20,7 @@ import time
 import numpy as np
 
 SLOTS = (4, 8, 16, 24)
-PANEL_BLOCKS = (1, 2, 3)
+PANEL_BLOCKS = (1, 2)  # two is what fits an SM, and the default
 BUCKETS = (("dense", 64, 4), ("dense", 128, 4), ("dense", 256, 4), ("dense", 256, 5),
            ("u1", 256, 5), ("u1", 512, 5), ("u1", 1024, 5))
 
@@ -71,7 +71,7 @@ def tune(buckets=BUCKETS, L: int = 16, seed: int = 240105301):
             for pb in PANEL_BLOCKS:
                 trials.append((_time_layer(form, L, d, chi, state, slots, pb), slots, pb))
         t, slots, pb = min(trials)
-        default = next(x for x in trials if x[1] == 24 and x[2] == 3)[0]
+        default = next(x for x in trials if x[1] == 24 and x[2] == 2)[0]
         out["buckets"].append({"form": form, "chi": chi, "d": d, "max_slots": slots, "panel_blocks": pb,
                                "layer_ms": 1e3 * t, "default_layer_ms": 1e3 * default,
                                "trials_ms": {f"{s}x{p}": 1e3 * x for x, s, p in trials}})

@@ -177,8 +177,9 @@ __global__ void __launch_bounds__(256) k_sturm_prep(const __grid_constant__ EigB
 // minors p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (Sturm's theorem), with
 // a zero minor counted as a change.  Bound: the FP64 pipe, three dependent instructions of 64 clocks
 // a step for a warp alone on its scheduler, so only the recurrence runs there: signs and zeros are
-// read from the upper words, and the range is checked every fourth step only (a step changes the
-// magnitude by less than 2^3 up and 2^60 down: x and d_i are doubles below 4), by exact rescaling.
+// read from the upper words, and the range is checked every fourth step only, by exact rescaling: a step
+// raises the magnitude by less than 2^3 (x and d_i are below 4), and lowers it by more than the 2^60 of a rounded
+// difference only beside a minor that vanishes, whose size the count does not use.
 __device__ __forceinline__ int sturm_count(const double2* __restrict__ P, int m, double x) {
   double pm = 0.0, p = 1.0;
   int hp = 0x3FF00000, cnt = 0;  // upper word of p
@@ -807,7 +808,7 @@ constexpr int TD_NB = 32;      // columns per panel of the blocked reduction
 constexpr int REFL_FLUSH_EXP = 340;
 // The last TD_TAIL or fewer columns of every matrix are reduced by one block per
 // matrix with the trailing matrix in shared memory (k_tridiag_tail): there the
-// cooperative kernel would pay three grid barriers per column for very little work.
+// cooperative kernel would pay two grid barriers per column for very little work.
 // A matrix takes part in the panels k0 < tail_start(m) (a multiple of TD_NB), so the
 // split depends on its own size only and each result is independent of its batch.
 constexpr int TD_TAIL = 64;
@@ -1070,7 +1071,7 @@ __device__ __forceinline__ int td_find(const int* pre, int n, int it) {
   return lo;
 }
 
-// Item counts of every matrix as prefix sums (warp 0; a lane takes EIG_MAXP / 32 neighbours).
+// Item counts of every matrix as prefix sums (one warp; a lane takes EIG_MAXP / 32 neighbours).
 template <class F>
 __device__ __forceinline__ void td_prefix(int* pre, int n, F count) {
   constexpr int W = EIG_MAXP / 32;

@@ -233,7 +233,7 @@ __device__ __forceinline__ int row_exp(int hi) {
   return max(hi >> 20, 1) - 1022;
 }
 
-// Largest magnitude of each of the 32 rows of row block rb into mx[32] (256 threads).
+// Largest magnitude of each of the 32 rows of row block rb into part[0] (256 threads).
 __device__ __forceinline__ void row_magnitudes(const OzPackJob& J, int rb, int (&part)[8][33]) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (J.ks == 1) {  // rows contiguous along k: a warp per row

@@ -175,8 +175,9 @@ int oz_gemm_pooled(std::vector<OzProb>& probs, void* pool, size_t bytes, int* st
 
 // Workspace of a product without a handle (tebd_zgemm), stream-ordered, freed with cudaFreeAsync.  It comes
 // from a memory pool of the device that keeps at most 128 MB between calls (the default pool gives
-// everything back at each synchronisation: 200 us a call); ws_trim gives that back too, when an
-// allocation of a handle fails.
+// everything back at each synchronisation: 200 us a call).  An allocation that finds too little takes that back: the
+// driver does so for cudaMalloc (measured: a blocked step that needs 66 MB runs with 5 MB free beside it),
+// and dalloc asks for it with ws_trim.
 cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s);
 void ws_trim();
 
@@ -234,7 +235,7 @@ struct EigBatch {
   int n;
   unsigned int* bar;  // grid-barrier state {count, generation, error} for the persistent reduction
   long long wait_clocks;  // limit of each grid-barrier wait of the reduction (clock64 ticks)
-  int panel_blocks;       // blocks per SM of the reduction's cooperative grid (0: as many as fit, at most 3)
+  int panel_blocks;       // blocks per SM of the reduction's cooperative grid (0: as many as fit: two)
   int range;              // traces outside 2^+-range are scaled for the reduction (set by eig_tridiagonalize)
   int few;                // 1: dense form, a batch of at most 24 matrices (the bisection spreads wider)
 };

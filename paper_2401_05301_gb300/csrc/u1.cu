@@ -137,12 +137,6 @@ struct TruncCut {
   int* status;
 };
 
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return __shfl_sync(0xffffffffu, v, 0);
-}
-
 // Bitonic sort of (s, key) over P entries (P a power of two): descending s with
 // ascending key on ties (desc_s), or ascending key (otherwise).
 __device__ void bitonic(double* s, int* key, int P, bool desc_s) {
@@ -178,7 +172,7 @@ __global__ void __launch_bounds__(256) k_cand_norms(const TruncCut* __restrict__
     const double2 v = y[c];
     acc = fma(v.x, v.x, fma(v.y, v.y, acc));
   }
-  acc = warp_sum_d(acc);
+  acc = warp_sum(acc);
   if (lane == 0) A.s_out[g] = sqrt(acc);
 }
 
@@ -291,7 +285,7 @@ __global__ void k_right_scale(const RightRows* __restrict__ rr) {
     const double2 t = R.T[(size_t)r * R.K + k];
     acc = fma(t.x, t.x, fma(t.y, t.y, acc));
   }
-  acc = warp_sum_d(acc);
+  acc = warp_sum(acc);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -441,8 +435,8 @@ __global__ void k_trace_bonds(const TraceBond* __restrict__ bonds, const TraceBl
       im = fma(x.x, y.y, fma(x.y, y.x, im));
     }
   }
-  re = warp_sum_d(re);
-  im = warp_sum_d(im);
+  re = warp_sum(re);
+  im = warp_sum(im);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   if (l == 0) { re_sh[w] = re; im_sh[w] = im; }
   __syncthreads();
@@ -843,7 +837,6 @@ size_t eig_ws_bytes(int b, int kmax) {
   size_t z = 0;
   auto upd = [&](size_t x) { z = std::max(z, x); };
   upd(oz_workspace_bytes(b, b, 64, false));
-  upd(oz_workspace_bytes(64, 64, b, true));
   upd(oz_workspace_bytes(kmax, 64, b, false));
   upd(oz_workspace_bytes(kmax, 64, 64, false));
   upd(oz_workspace_bytes(kmax, b, 64, false));
@@ -1905,7 +1898,7 @@ __global__ void k_frob(const FrobArgs* __restrict__ fa) {
     const double2 v = F.X[e];
     acc = fma(l * l, fma(v.x, v.x, v.y * v.y), acc);
   }
-  acc = warp_sum_d(acc);
+  acc = warp_sum(acc);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
   __syncthreads();
   if (threadIdx.x == 0) {
